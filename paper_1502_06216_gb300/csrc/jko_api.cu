@@ -508,10 +508,19 @@ double pass_flops(const jko_handle* h, int which) {
   return 2.0 * (2.0 * r + 1.0) * (double)h->N;
 }
 
-// `pairs` pairs as one persistent launch: the tensor-core loop kernel, or the
-// heat kernel's persistent form.
+template <typename T>
+cudaError_t enqueue_strip(jko_handle* h, int pairs, cudaStream_t st) {
+  return jko::strip_launch<T>(h->strip, h->ek, h->grid.nx, h->grid.ny, h->rx, h->ry,
+                              (const T*)h->taps_x, (const T*)h->taps_y, (const T*)h->q, (T*)h->a,
+                              (T*)h->p, jko::prox_args<T>(h), h->ctrl, h->strip_words, pairs, st);
+}
+
+// `pairs` pairs as one persistent launch: the tensor-core loop kernel, the
+// heat kernel's persistent form or the CUDA-core filter's.
 cudaError_t enqueue_loop(jko_handle* h, int pairs, cudaStream_t st) {
   if (h->tc) return jko::tc_enqueue_loop(h->tc, pairs, st);
+  if (!h->heat_L)
+    return h->fp64 ? enqueue_strip<double>(h, pairs, st) : enqueue_strip<float>(h, pairs, st);
   const int nx = h->grid.nx, ny = h->grid.ny;
   const uint8_t* mask = (const uint8_t*)h->mask;
   if (h->fp64)
@@ -694,7 +703,8 @@ void free_handle(jko_handle* h) {
                   h->a2, h->b2, h->tgt, h->s1, h->s2, h->E2,
                   h->fft_khat_x, h->fft_tw_x, h->fft_khat_y, h->fft_tw_y,
                   h->tape, h->adj, h->adj2, h->adj_red, h->hb.d[0], h->hb.d[1], h->hb.d[2],
-                  h->hb.d[3], h->hb.coef, h->a3, h->b3, h->s3, h->t2, h->t3, h->mpair};
+                  h->hb.d[3], h->hb.coef, h->a3, h->b3, h->s3, h->t2, h->t3, h->mpair,
+                  h->strip_words};
   for (void* b : bufs) if (b) cudaFree(b);
   if (h->ctrl_init) cudaFreeHost(h->ctrl_init);
   if (h->poll) cudaFreeHost(h->poll);
@@ -956,6 +966,19 @@ jko_status setup_simt(jko_handle* h) {
     CK(h, upload<T>(&h->fft_khat_y, kh));
     CK(h, upload<T>(&h->fft_tw_y, tw));
   }
+  return JKO_OK;
+}
+
+// The persistent CUDA-core form, where its rule takes this grid.
+template <typename T>
+jko_status setup_strip(jko_handle* h) {
+  h->strip = jko::strip_plan<T>(h->grid.nx, h->grid.ny, h->rx, h->ry, h->ek, jko::prox_args<T>(h),
+                                0);
+  if (h->strip.G == 0) return JKO_OK;
+  const size_t bytes = sizeof(unsigned long long) * h->strip.words;
+  CK(h, cudaMalloc((void**)&h->strip_words, bytes));
+  CK(h, cudaMemset(h->strip_words, 0, bytes));
+  h->use_loop = 1;
   return JKO_OK;
 }
 
@@ -1271,7 +1294,8 @@ jko_status flow_impl(jko_handle* h, const T* p0, int n_steps, T* traj, T* p_fina
   // The loop graph and the per-step reports are set up at the first flow of
   // any length (a one-step flow does it for the longer flows after it).
   if (!(h->prm.finish && h->tc)) {
-    build_step_loop(h);
+    if (h->use_loop) h->step_loop_state = 1;
+    else build_step_loop(h);
     if (h->step_loop_state == 1 && h->flow_cap < n_steps) {
       const int cap = std::max(n_steps, 64);
       if (h->flow_ctrl) cudaFreeHost(h->flow_ctrl);
@@ -1315,7 +1339,8 @@ jko_status flow_impl(jko_handle* h, const T* p0, int n_steps, T* traj, T* p_fina
       CK(h, cudaEventRecord(h->flow_ev[2 * t], st));
       jko_status sb = enqueue_step_begin<T>(h, q, st);
       if (sb != JKO_OK) return sb;
-      CK(h, cudaGraphLaunch(h->step_loop, st));
+      // a persistent kernel ends the step by itself: no loop around it
+      CK(h, h->use_loop ? launch_chunk(h, st) : cudaGraphLaunch(h->step_loop, st));
       CK(h, jko::launch_finalize_reduce<T>((const T*)h->p, h->ns, P, h->ctrl, h->part,
                                            h->part_cap, st));
       CK(h, jko::launch_finalize_write<T>((const T*)h->p, out, h->ns, h->prm.renormalize,
@@ -1350,7 +1375,7 @@ jko_status flow_impl(jko_handle* h, const T* p0, int n_steps, T* traj, T* p_fina
         // the last one completed) and their loop conditions, the finalisation
         const long long chunks =
             h->use_loop ? 1 : (c.it + 1 + h->chunk_iters - 1) / h->chunk_iters;
-        info.kernels = (int)(1 + chunks * (per_chunk + 1) + 2);
+        info.kernels = (int)(1 + chunks * (per_chunk + (h->use_loop ? 0 : 1)) + 2);
         info.iters_finish = 0;
       }
       if (sk == JKO_ERR_NUMERIC) set_err(h, sk, "NaN or Inf in the scaling iterates");
@@ -1476,8 +1501,8 @@ jko_status jko_create(const jko_grid* grid, const jko_params* params, const jko_
     if (h->attract || h->species == 2)   // the tensor-core passes' b-update partials
       np = std::max(np, 3 * jko::tc_multi_tiles(grid->nx, grid->ny, 1));
     if (h->pair_alpha > 0) np = std::max(np, h->nparts_pw);
-    e = cudaMalloc((void**)&h->part, sizeof(double) * np);
     h->part_cap = np;
+    e = cudaMalloc((void**)&h->part, sizeof(double) * np);
     if (e != cudaSuccess) return fail(cuda_err(h, e, "cudaMalloc(partials)"));
     e = cudaMemset(h->part, 0, sizeof(double) * np);
     if (e != cudaSuccess) return fail(cuda_err(h, e, "cudaMemset(partials)"));
@@ -1514,6 +1539,11 @@ jko_status jko_create(const jko_grid* grid, const jko_params* params, const jko_
   if (h->prec == JKO_FP64 || h->prec == JKO_FP32) {
     // the heat kernel needs no Gaussian taps
     if (!h->heat_L) s = h->fp64 ? setup_simt<double>(h) : setup_simt<float>(h);
+    if (s == JKO_OK && !h->heat_L && !h->fft && !h->attract && h->species != 2 &&
+        params->loop != 2) {
+      // one persistent launch per step where that is the faster form (loop 2: never)
+      s = h->fp64 ? setup_strip<double>(h) : setup_strip<float>(h);
+    }
   } else {
     jko::TcConfig cfg{};
     cfg.nx = grid->nx; cfg.ny = grid->ny; cfg.lx = grid->lx; cfg.ly = grid->ly;
@@ -1699,7 +1729,8 @@ jko_status jko_profile_passes(jko_handle* h, int reps, float* ms, double* flops)
 jko_status jko_profile_loop(jko_handle* h, int pairs, int reps, float* ms, double* flops) {
   if (!h) return set_err(nullptr, JKO_ERR_INVALID_ARG, "NULL handle");
   if (pairs < 1 || reps < 1 || !ms) return set_err(h, JKO_ERR_INVALID_ARG, "pairs < 1, reps < 1 or NULL ms");
-  if (!h->use_loop) return set_err(h, JKO_ERR_UNSUPPORTED, "the handle does not use the loop kernel");
+  if (!h->use_loop || h->strip.G > 0)
+    return set_err(h, JKO_ERR_UNSUPPORTED, "the handle does not use the loop kernel");
   DeviceGuard dg(h->device);
   cudaStream_t st = h->stream;
   // a running control block that never stops (as in jko_profile_passes)
@@ -1815,6 +1846,7 @@ struct jko_batch {
   cudaEvent_t ev_poll[2] = {nullptr, nullptr};
   int last_iters = 0;
   bool per_pass = false;             // run every flow on per-pass kernels
+  bool all_loop = false;             // every flow's chunk is one persistent launch
   int tuned = -1;                    // candidate the batch autotuner chose
   std::vector<jko::TcGroup*> groups; // grouped launches (one per precision)
   std::vector<int> group_pairs;      // pairs one grouped launch may run
@@ -1877,8 +1909,8 @@ cudaError_t flow_prologue(jko_handle* h, cudaStream_t s) {
 cudaError_t flow_chunk(jko_handle* h, int C, bool per_pass, cudaStream_t s, int loop_pairs = 0) {
   // a flow on the loop kernel: one launch runs its whole pair budget and stops
   // itself; later chunks of the step find it stopped and return at once
-  if (h->use_loop && h->tc && !per_pass)
-    return jko::tc_enqueue_loop(h->tc, loop_pairs > 0 ? loop_pairs : h->chunk_iters, s);
+  if (h->use_loop && !per_pass)
+    return enqueue_loop(h, loop_pairs > 0 ? loop_pairs : h->chunk_iters, s);
   for (int i = 0; i < C; ++i) {
     cudaError_t e = enqueue_pair(h, s);
     if (e != cudaSuccess) return e;
@@ -2173,7 +2205,7 @@ jko_status jko_batch_create(int n_flows, const jko_grid* grids, const jko_params
     }
   }
   for (auto* h : b->h)
-    if (h->tc) h->chunk_iters = h->use_loop ? h->prm.max_iter + 1 : C;
+    h->chunk_iters = h->use_loop ? h->prm.max_iter + 1 : C;
   jko_status s = capture_batch(
       b, no_op, [](jko_handle* h, cudaStream_t st) { return flow_prologue(h, st); },
       [b](cudaStream_t root) { return begin_groups(b, root); }, &b->g_pro);
@@ -2198,6 +2230,7 @@ jko_status jko_batch_create(int n_flows, const jko_grid* grids, const jko_params
   bool all_loop = !b->per_pass;
   for (auto* h : b->h) all_loop = all_loop && h->use_loop;
   if (all_loop) b->C = b->max_iter + 1;
+  b->all_loop = all_loop;
   s = capture_batch(
       b, no_op, [](jko_handle* h, cudaStream_t st) { return flow_finalize(h, st); },
       [b](cudaStream_t root) { return jko::launch_gather_ctrl(b->ctrl_ptrs, b->ctrl_all, b->n, root); },
@@ -2260,7 +2293,8 @@ jko_status jko_batch_flow(jko_batch* b, const void* const* p0_dev, int n_steps,
     for (int i = 0; i < ahead; ++i) BCK(b, launch());
     bool stopped = false;
     while (!stopped) {
-      if (launched - polled < 2 && launched < max_chunks) BCK(b, launch());
+      // (a chunk of persistent launches covers the whole budget: none behind it)
+      if (launched - polled < (b->all_loop ? 1 : 2) && launched < max_chunks) BCK(b, launch());
       const int target = launched - 1 - ((launched - polled) >= 2 ? 1 : 0);
       const int slot = target & 1;
       BCK(b, cudaEventSynchronize(b->ev_poll[slot]));

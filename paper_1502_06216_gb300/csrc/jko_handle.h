@@ -68,6 +68,8 @@ struct jko_handle {
   int part_cap = 0;       // entries of part (residual and mass partials)
   int use_loop = 0;       // chunks run as one persistent kernel (tensor cores or heat kernel)
   int heat_G = 0;         // blocks of the heat kernel's persistent form
+  jko::StripPlan strip;   // the CUDA-core form's persistent kernel (G = 0: per-pass kernels)
+  unsigned long long* strip_words = nullptr;   // its exchange buffers
   int tc_multi = 0;       // several couplings on the tensor cores (tc_multi.cu)
   void* mpair = nullptr;  // bf16 forms of several couplings: pairs of the first pass's images
   Ctrl* ctrl_init = nullptr;   // pinned initial value

@@ -69,6 +69,28 @@ template <typename T>
 cudaError_t simt_pass(int epi, int ek, const PassArgs<T>& A, const ProxArgs<T>& P,
                       cudaStream_t st);
 
+// Persistent form of a step on one density (strip.cu): one cooperative launch of
+// G blocks, each owning nc columns and nr rows of the images in shared memory.
+// strip_plan: G = 0 where the kernels per pass are the faster form or the strips do
+// not fit; max_blocks > 0: at most that many blocks.
+struct StripPlan {
+  int G = 0;           // blocks (0: not available)
+  int nc = 0, nr = 0;  // columns and rows per block
+  int rb = 0;          // outputs per work item
+  int threads = 0;
+  size_t smem = 0;
+  size_t x1_words = 0, x2_words = 0, words = 0;   // exchange buffers, 8 bytes a word
+};
+template <typename T>
+StripPlan strip_plan(int nx, int ny, int rx, int ry, int ek, const ProxArgs<T>& P, int max_blocks);
+// words: sp.words 8-byte words, zeroed once before the first launch (the epochs
+// of the exchanges go on from launch to launch).
+template <typename T>
+cudaError_t strip_launch(const StripPlan& sp, int ek, int nx, int ny, int rx, int ry,
+                         const T* taps_x, const T* taps_y, const T* q, T* a, T* p,
+                         const ProxArgs<T>& P, Ctrl* ctrl, unsigned long long* words, int pairs,
+                         cudaStream_t st);
+
 // Step prologue / epilogue kernels (jko_step_kernels.cu).
 template <typename T>
 cudaError_t launch_fill(T* x, T v, long long n, cudaStream_t st);
