@@ -134,11 +134,12 @@ typedef struct jko_params {
                        handles (jko_grid.heat_L > 0): 0 or 1 = one persistent cooperative
                        kernel per step where the device has cooperative launches (1:
                        JKO_ERR_UNSUPPORTED where not), 2 = kernels per Clenshaw phase;
-                       both give the same bits.  Single-density JKO_FP32 / JKO_FP64 handles
-                       with the band-limited filter: 0, 1 or 3 = one persistent
-                       cooperative kernel per step where the grid suits it (else, and with
-                       2, one kernel per pass; the two differ by rounding, the 1-D filters
-                       of xi b being applied in the other order).  Other CUDA-core handles
+                       both give the same bits.  JKO_FP32 / JKO_FP64 handles with the
+                       band-limited filter, of one density or several couplings: 0, 1 or
+                       3 = one persistent cooperative kernel per step where the grid suits
+                       it (else, and with 2, one kernel per pass; the two differ by
+                       rounding, the 1-D filters of a pair's second application of xi
+                       being applied in the other order).  Other CUDA-core handles
                        ignore it */
   int tile;         /* tensor-core precisions: output tile width of the per-pass kernels,
                        64 or 128 (128: JKO_TF32 only), or 0 = automatic.  With loop = 0

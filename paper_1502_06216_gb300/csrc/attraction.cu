@@ -12,6 +12,7 @@
 //     a_m = p / s_m                                     (this kernel)
 // The energy fields of the handle are built with sigma / (1 + tau), so the
 // proximal map of h is the single-coupling one, taken at the geometric mean.
+#include "coupled_prox.cuh"
 #include "jko_internal.cuh"
 #include "jko_kernels.h"
 
@@ -32,15 +33,8 @@ __global__ void __launch_bounds__(NT) attraction_prox_kernel(const T* s1, const 
   for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n;
        i += (long long)gridDim.x * blockDim.x) {
     const T x1 = s1[i], x2 = s2[i];
-    // geometric mean s_1^{1/(1+tau)} s_2^{tau/(1+tau)}, 0 where either vanishes
-    const T g = (x1 > T(0) && x2 > T(0))
-                    ? dev_exp<T>(w1 * dev_log<T>(x1) + w2 * dev_log<T>(x2)) : T(0);
-    const T pm = prox_ratio<T, EK>(P, (int)i, g) * g;
-    // a_m = p / s_m with IEEE division: s_m may be subnormal far from the
-    // support of b_m, where x * rcp(s) would overflow (a_m itself stays finite,
-    // ~ (s_other / s_m)^{weight})
-    const T r1 = x1 > T(0) ? pm / x1 : T(0);
-    const T r2 = x2 > T(0) ? pm / x2 : T(0);
+    T r1, r2, pm;
+    attraction_cell<T, EK>(P, (int)i, x1, x2, w1, w2, r1, r2, pm);
     bad |= !dev_finite(r1) || !dev_finite(r2) || !dev_finite(pm);
     a1[i] = op_round<T>(r1, rnd);
     a2[i] = op_round<T>(r2, rnd);
@@ -51,9 +45,7 @@ __global__ void __launch_bounds__(NT) attraction_prox_kernel(const T* s1, const 
   if (threadIdx.x == 0 && blockIdx.x == 0) ctrl->it = s_it + 1;
 }
 
-// Two densities coupled through the congestion of their sum (Sec. 5.3): with
-// a~_m = s_m e^{-sigma w_m}, p_m = a~_m min(1, kappa / (a~_1 + a~_2)) and
-// a_m = p_m / s_m = e^{-sigma w_m} min(1, ...) (no division by s_m).
+// Two densities coupled through the congestion of their sum (Sec. 5.3).
 template <typename T>
 __global__ void __launch_bounds__(NT) species_prox_kernel(const T* s1, const T* s2, const T* E1,
                                                           const T* E2, T* a1, T* a2, T* p,
@@ -65,14 +57,13 @@ __global__ void __launch_bounds__(NT) species_prox_kernel(const T* s1, const T* 
   for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n;
        i += (long long)gridDim.x * blockDim.x) {
     const T e1 = E1 ? E1[i] : T(1), e2 = E2 ? E2[i] : T(1);
-    const T t1 = s1[i] * e1, t2 = s2[i] * e2;
-    const T t = t1 + t2;
-    const T f = (has_kappa && t > kappa) ? kappa / t : T(1);
-    a1[i] = op_round<T>(e1 * f, rnd);
-    a2[i] = op_round<T>(e2 * f, rnd);
-    p[i] = t1 * f;
-    p[n + i] = t2 * f;
-    bad |= !dev_finite(t1 * f) || !dev_finite(t2 * f);
+    T r1, r2, p1, p2;
+    species_cell<T>(s1[i], s2[i], e1, e2, kappa, has_kappa, r1, r2, p1, p2);
+    a1[i] = op_round<T>(r1, rnd);
+    a2[i] = op_round<T>(r2, rnd);
+    p[i] = p1;
+    p[n + i] = p2;
+    bad |= !dev_finite(p1) || !dev_finite(p2);
   }
   bad = warp_or(bad);
   if ((threadIdx.x & 31) == 0 && bad) atomicOr(&ctrl->nonfinite, 1);
@@ -84,19 +75,6 @@ __global__ void __launch_bounds__(NT) species_prox_kernel(const T* s1, const T* 
 // q_2, columns p_2), pi_3 (rows p_1, columns p_2), weights (1, 1, t), t = tau
 // alpha.  By the update rules of Prop. prop-implementation-generic the prox
 // inputs are xi b_m (rows) and xi^T a_m (columns) alone.
-
-// Weighted geometric mean x^{1/(1+t)} y^{t/(1+t)}, 0 where either vanishes.
-template <typename T>
-__device__ __forceinline__ T weighted_geomean(T x, T y, T t) {
-  return (x > T(0) && y > T(0)) ? dev_exp<T>((dev_log<T>(x) + t * dev_log<T>(y)) / (T(1) + t))
-                                : T(0);
-}
-
-// p / s with IEEE division, 0 where p = 0 (s may be subnormal in the far field)
-template <typename T>
-__device__ __forceinline__ T safe_ratio(T p, T s) {
-  return (p > T(0) && s > T(0)) ? p / s : T(0);
-}
 
 // Row half-step (psi_1): p_1 = min(e^{-sigma' w_1} g(s_1, s_3), kappa) is the
 // common row marginal of pi_1 and pi_3, pi_2 keeps the rows q_2.
@@ -111,8 +89,7 @@ __global__ void __launch_bounds__(NT) pairwise_rows_kernel(const T* s1, const T*
   for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n;
        i += (long long)gridDim.x * blockDim.x) {
     const T x1 = s1[i], x3 = s3[i];
-    T pm = weighted_geomean<T>(x1, x3, t) * (E1 ? E1[i] : T(1));
-    if (has_kappa && pm > kappa) pm = kappa;
+    const T pm = pairwise_marginal<T>(x1, x3, t, E1 ? E1[i] : T(1), kappa, has_kappa);
     const T r1 = safe_ratio<T>(pm, x1), r3 = safe_ratio<T>(pm, x3);
     const T r2 = b_update<T>(q2[i], s2[i]);
     bad |= !dev_finite(r1) || !dev_finite(r2) || !dev_finite(r3) || !dev_finite(pm);
@@ -147,8 +124,7 @@ __global__ void __launch_bounds__(NT) pairwise_cols_kernel(const T* y1, const T*
     const T qq = q1[i], c1 = b1[i], c2 = b2[i], c3 = b3[i];
     res += (double)abs_residual<T>(c1, v1, qq) + (double)fabs(c2 * v2 - c3 * v3);
     p2[i] = c2 * v2;
-    T pm = weighted_geomean<T>(v2, v3, t) * (E2 ? E2[i] : T(1));
-    if (has_kappa && pm > kappa) pm = kappa;
+    const T pm = pairwise_marginal<T>(v2, v3, t, E2 ? E2[i] : T(1), kappa, has_kappa);
     const T r1 = b_update<T>(qq, v1);
     const T r2 = safe_ratio<T>(pm, v2), r3 = safe_ratio<T>(pm, v3);
     bad |= !dev_finite(r1) || !dev_finite(r2) || !dev_finite(r3);

@@ -508,11 +508,29 @@ double pass_flops(const jko_handle* h, int which) {
   return 2.0 * (2.0 * r + 1.0) * (double)h->N;
 }
 
+// The couplings of a handle's step, as strip.cu counts them.
+int strip_op(const jko_handle* h) {
+  if (h->pair_alpha > 0) return jko::OP_PAIR;
+  if (h->species == 2) return jko::OP_SPECIES;
+  return h->attract ? jko::OP_ATTRACT : jko::OP_ONE;
+}
+
 template <typename T>
 cudaError_t enqueue_strip(jko_handle* h, int pairs, cudaStream_t st) {
-  return jko::strip_launch<T>(h->strip, h->ek, h->grid.nx, h->grid.ny, h->rx, h->ry,
-                              (const T*)h->taps_x, (const T*)h->taps_y, (const T*)h->q, (T*)h->a,
-                              (T*)h->p, jko::prox_args<T>(h), h->ctrl, h->strip_words, pairs, st);
+  jko::StripStep<T> s{};
+  s.op = strip_op(h);
+  s.ek = h->ek;
+  s.q = (const T*)h->q;
+  s.q2 = h->attract ? (const T*)h->tgt : h->species == 2 ? (const T*)h->q + h->N : nullptr;
+  s.E1 = (const T*)h->E;
+  s.E2 = (const T*)h->E2;
+  s.t = h->pair_alpha > 0 ? h->prm.tau * h->pair_alpha : h->prm.tau;
+  s.a = (T*)h->a;
+  s.a2 = (T*)h->a2;
+  s.p = (T*)h->p;
+  return jko::strip_launch<T>(h->strip, h->grid.nx, h->grid.ny, h->rx, h->ry, (const T*)h->taps_x,
+                              (const T*)h->taps_y, s, jko::prox_args<T>(h), h->ctrl,
+                              h->strip_words, pairs, st);
 }
 
 // `pairs` pairs as one persistent launch: the tensor-core loop kernel, the
@@ -972,8 +990,8 @@ jko_status setup_simt(jko_handle* h) {
 // The persistent CUDA-core form, where its rule takes this grid.
 template <typename T>
 jko_status setup_strip(jko_handle* h) {
-  h->strip = jko::strip_plan<T>(h->grid.nx, h->grid.ny, h->rx, h->ry, h->ek, jko::prox_args<T>(h),
-                                0);
+  h->strip = jko::strip_plan<T>(h->grid.nx, h->grid.ny, h->rx, h->ry, strip_op(h), h->ek,
+                                jko::prox_args<T>(h), 0);
   if (h->strip.G == 0) return JKO_OK;
   const size_t bytes = sizeof(unsigned long long) * h->strip.words;
   CK(h, cudaMalloc((void**)&h->strip_words, bytes));
@@ -993,7 +1011,7 @@ jko_status enqueue_step_begin(jko_handle* h, const T* q_in, cudaStream_t st) {
   CK(h, jko::launch_step_begin<T>(*h->ctrl_init, h->ctrl, h->chunk_ctr,
                                   (const void*)q_in != h->q ? q_in : nullptr, (T*)h->q, h->ns,
                                   plain ? (T*)h->a : nullptr, plain ? (long long)h->N : 0, st));
-  if (plain) return JKO_OK;
+  if (plain || h->strip.G > 0) return JKO_OK;   // strip.cu starts its scalings itself
   if (h->tc_multi) {
     if (h->pair_alpha > 0) CK(h, begin_pairwise<float>(h, st));
     else CK(h, begin_multi_tc(h, st));
@@ -1539,8 +1557,7 @@ jko_status jko_create(const jko_grid* grid, const jko_params* params, const jko_
   if (h->prec == JKO_FP64 || h->prec == JKO_FP32) {
     // the heat kernel needs no Gaussian taps
     if (!h->heat_L) s = h->fp64 ? setup_simt<double>(h) : setup_simt<float>(h);
-    if (s == JKO_OK && !h->heat_L && !h->fft && !h->attract && h->species != 2 &&
-        params->loop != 2) {
+    if (s == JKO_OK && !h->heat_L && !h->fft && params->loop != 2) {
       // one persistent launch per step where that is the faster form (loop 2: never)
       s = h->fp64 ? setup_strip<double>(h) : setup_strip<float>(h);
     }
@@ -1892,6 +1909,7 @@ void free_batch(jko_batch* b) {
 // the step input is already in h->q).
 template <typename T>
 cudaError_t flow_begin_t(jko_handle* h, cudaStream_t s) {
+  if (h->use_loop && h->strip.G > 0) return cudaSuccess;   // strip.cu starts its scalings itself
   if (h->pair_alpha > 0) return begin_pairwise<T>(h, s);
   if (h->species == 2) return begin_species<T>(h, s);
   if (h->attract) return begin_attraction<T>(h, s);
@@ -2224,6 +2242,20 @@ jko_status jko_batch_create(int n_flows, const jko_grid* grids, const jko_params
     cudaGetLastError();
     b->per_pass = true;
     s = capture_chunks();
+    // ... and with them the cold start that strip.cu's launches make themselves
+    bool strips = false;
+    for (auto* h : b->h)
+      if (h->strip.G > 0) {
+        h->use_loop = 0;
+        strips = true;
+      }
+    if (s == JKO_OK && strips) {
+      cudaGraphExecDestroy(b->g_pro);
+      b->g_pro = nullptr;
+      s = capture_batch(
+          b, no_op, [](jko_handle* h, cudaStream_t st) { return flow_prologue(h, st); },
+          [b](cudaStream_t root) { return begin_groups(b, root); }, &b->g_pro);
+    }
   }
   if (s != JKO_OK) return fail(s);
   // every flow on the loop kernel: one chunk launch covers the whole budget

@@ -69,10 +69,11 @@ template <typename T>
 cudaError_t simt_pass(int epi, int ek, const PassArgs<T>& A, const ProxArgs<T>& P,
                       cudaStream_t st);
 
-// Persistent form of a step on one density (strip.cu): one cooperative launch of
-// G blocks, each owning nc columns and nr rows of the images in shared memory.
+// Persistent CUDA-core form of a step (strip.cu): one cooperative launch of G
+// blocks, each owning nc columns and nr rows of the images in shared memory.
 // strip_plan: G = 0 where the kernels per pass are the faster form or the strips do
 // not fit; max_blocks > 0: at most that many blocks.
+enum : int { OP_ONE = 0, OP_ATTRACT = 1, OP_SPECIES = 2, OP_PAIR = 3 };   // couplings of a step
 struct StripPlan {
   int G = 0;           // blocks (0: not available)
   int nc = 0, nr = 0;  // columns and rows per block
@@ -82,14 +83,26 @@ struct StripPlan {
   size_t x1_words = 0, x2_words = 0, words = 0;   // exchange buffers, 8 bytes a word
 };
 template <typename T>
-StripPlan strip_plan(int nx, int ny, int rx, int ry, int ek, const ProxArgs<T>& P, int max_blocks);
+struct StripStep {
+  int op, ek;
+  const T* q;          // the step's input (two densities: 2 N)
+  const T* q2;         // attraction: the target; two densities: q + N
+  const T* E1;         // e^{-sigma w_m} of the two densities (NULL: 1)
+  const T* E2;
+  double t;            // attraction: tau; pairwise: tau alpha
+  T* a;                // final scalings (a2: two couplings; pairwise: none written)
+  T* a2;
+  T* p;
+};
+template <typename T>
+StripPlan strip_plan(int nx, int ny, int rx, int ry, int op, int ek, const ProxArgs<T>& P,
+                     int max_blocks);
 // words: sp.words 8-byte words, zeroed once before the first launch (the epochs
 // of the exchanges go on from launch to launch).
 template <typename T>
-cudaError_t strip_launch(const StripPlan& sp, int ek, int nx, int ny, int rx, int ry,
-                         const T* taps_x, const T* taps_y, const T* q, T* a, T* p,
-                         const ProxArgs<T>& P, Ctrl* ctrl, unsigned long long* words, int pairs,
-                         cudaStream_t st);
+cudaError_t strip_launch(const StripPlan& sp, int nx, int ny, int rx, int ry, const T* taps_x,
+                         const T* taps_y, const StripStep<T>& s, const ProxArgs<T>& P, Ctrl* ctrl,
+                         unsigned long long* words, int pairs, cudaStream_t st);
 
 // Step prologue / epilogue kernels (jko_step_kernels.cu).
 template <typename T>

@@ -1,6 +1,7 @@
 // strip.cu -- persistent CUDA-core form of a JKO step (FP32 / FP64, the separable
-// Gaussian by taps, one density): one cooperative launch runs the pairs of the
-// scaling loop (Prop. 3.3) with the stopping rule of Sec. 3.4 inside.
+// Gaussian by taps): one cooperative launch runs the pairs of the scaling loop
+// (Prop. 3.3; with several couplings Prop. prop-implementation-generic) with the
+// stopping rule of Sec. 3.4 inside.
 //
 // Block g owns a strip of nc whole columns and a strip of nr whole rows, kept in
 // shared memory for the whole step (a, p and the prox fields by columns; b and q
@@ -11,249 +12,88 @@
 //                                    | exchange: U, rows -> columns
 //     columns: s = K_y U, a = Prox(s)/s, p = a s
 // with two exchanges through L2 where a kernel per pass makes four passes over
-// images in L2 and four launches.
+// images in L2 and four launches.  Steps with several couplings move their two
+// or three images together: the same two exchanges a pair, the joint proxes cell
+// by cell on the owned strip (attraction and two species: on the columns;
+// pairwise attraction: p_1 on the rows, p_2 on the columns).  A
+// five-step attraction flow at 256^2 FP32 (band 168): 6596 us a kernel per pass
+// (five launches a pair), 3324 us here.
 //
-// Exchange: every element travels as an 8-byte word {32 bits of data, epoch}
-// (two words for FP64), written and read as one access each, so a reader needs
-// no barrier and no fence: it polls the word itself until the epoch of this pair
-// appears (bounded).  The words for one receiver are contiguous.  One buffer per
-// direction suffices: a block writes the words of pair k + 1 only after it has
-// received all of pair k's of the other direction, which their senders wrote
-// after reading theirs.  The residual of each block's rows travels the same way, twice
-// buffered by pair parity (a block without columns may still be reading pair
-// k's when pair k + 1's are written); every block adds all of them in one
-// fixed order and takes the same decision.
+// The exchange is strip.cuh's.  The residual of each block's rows (pairwise:
+// columns) travels the same way, twice buffered by pair parity (a block may still
+// be reading pair k's when pair k + 1's are written); every block adds all of
+// them in one fixed order and takes the same decision.
 #include <algorithm>
 
-#include "jko_internal.cuh"
+#include "coupled_prox.cuh"
 #include "jko_kernels.h"
+#include "strip.cuh"
 
 namespace jko {
 
 namespace {
 
-constexpr unsigned kSpin = 1u << 22;   // polls of one word before giving up
+using namespace strip;
+
 constexpr int kStripMaxLine = 4096;
 
-// ---- words of the exchange buffers: {data, epoch}, one 64-bit access each ----
-__device__ __forceinline__ void put_word(unsigned long long* w, unsigned v, unsigned ep) {
-  const unsigned long long x = (unsigned long long)ep << 32 | v;
-  asm volatile("st.relaxed.gpu.global.u64 [%0], %1;" ::"l"(w), "l"(x) : "memory");
+// What a step computes between the moves (StripStep::op): images filtered at once.
+__host__ __device__ constexpr int op_images(int op) {
+  return op == OP_ONE ? 1 : op == OP_PAIR ? 3 : 2;
 }
-__device__ __forceinline__ void get_words(const unsigned long long* w, unsigned long long& x,
-                                          unsigned long long& y) {
-  asm volatile("ld.relaxed.gpu.global.v2.u64 {%0, %1}, [%2];"
-               : "=l"(x), "=l"(y) : "l"(w) : "memory");
-}
-template <typename T> constexpr int kWords = sizeof(T) / 4;   // words per element
-__device__ __forceinline__ void put_elem(unsigned long long* w, float v, unsigned ep) {
-  put_word(w, __float_as_uint(v), ep);
-}
-__device__ __forceinline__ void put_elem(unsigned long long* w, double v, unsigned ep) {
-  const unsigned long long b = (unsigned long long)__double_as_longlong(v);
-  put_word(w, (unsigned)b, ep);
-  put_word(w + 1, (unsigned)(b >> 32), ep);
-}
-// Both words of a pair, polled until they carry epoch ep; false: given up.
-__device__ __forceinline__ bool wait_pair(const unsigned long long* w, unsigned ep,
-                                          unsigned long long& x, unsigned long long& y,
-                                          volatile int* fault) {
-  for (unsigned i = 0; (unsigned)(x >> 32) != ep || (unsigned)(y >> 32) != ep; ++i) {
-    if (i >= kSpin || *fault) return false;
-    get_words(w, x, y);
-  }
-  return true;
-}
-__device__ __forceinline__ double words_double(unsigned long long lo, unsigned long long hi) {
-  return __longlong_as_double((long long)((hi << 32) | (lo & 0xffffffffull)));
-}
-
-// ---- lines in shared memory ----
-// Line l of an image strip starts at l * stride; its element i sits at sw(pad +
-// i), zeros around it (at least as far as the windows below reach).  pad = r
-// modulo 8 and the strides are multiples of 64 elements, so that every window
-// of eight starts at a multiple of eight.  Eight FP32 outputs per thread: the
-// 16-byte units a quarter-warp reads lie two apart, so the low bit of a unit's
-// index is flipped in every second group of eight units (conflict-free).
-constexpr int kPadR = 56;
-__host__ __device__ __forceinline__ int line_pad(int r) { return 24 + (r & 7); }
-__host__ __device__ __forceinline__ int line_stride(int n, int r) {
-  return (line_pad(r) + n + kPadR + 63) & ~63;
-}
-constexpr int kTapPad = 32;   // zeros behind the taps
-template <typename T, int RB>
-__device__ __forceinline__ int sw(int i) {
-  return (sizeof(T) == 4 && RB == 8) ? i ^ ((i >> 3) & 4) : i;
-}
-
-// acc[o] = sum_t k[t] x[i0 + o + t - r] over one line, t ascending, as
-// filter_pass adds them (terms beyond the band or the line are products with
-// zeros).  FP32, RB = 4 or 8: three register windows of RB elements rotate and
-// the taps are read four ahead, so that shared-memory loads are in flight
-// during the multiply-adds; the exit is tested once per 24 taps and the window
-// addresses advance by immediates.  At 256^2 (one warp per scheduler) a pass
-// over two lines takes 1.6k cycles against 2.8k with a test and an address
-// computation per window.
-__device__ __forceinline__ void lds4(uint32_t a, float* o) {
-  asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];"
-               : "=f"(o[0]), "=f"(o[1]), "=f"(o[2]), "=f"(o[3]) : "r"(a) : "memory");
-}
-template <int RB>
-__device__ __forceinline__ void window(uint32_t b, float (&w)[RB]) {
-  const uint32_t p = RB == 8 ? b ^ ((b >> 3) & 16u) : b;   // sw() on byte addresses
-#pragma unroll
-  for (int u = 0; u < RB / 4; ++u) lds4(p ^ (16u * u), w + 4 * u);
-}
-template <int RB>
-__device__ __forceinline__ void line_taps(float (&acc)[RB], const float* line, int pad,
-                                          const float* s_k, int n, int r, int i0) {
-  static_assert(RB == 4 || RB == 8, "");
-  constexpr int ST = 24 / RB;   // windows per exit test
-  int t_lo = r - i0 - (RB - 1);
-  if (t_lo < 0) t_lo = 0;
-  t_lo &= ~(RB - 1);
-  int t_hi = n - 1 - i0 + r;
-  if (t_hi > 2 * r) t_hi = 2 * r;
-  uint32_t xb = (uint32_t)__cvta_generic_to_shared(line + pad + i0 - r + t_lo);
-  uint32_t kb = (uint32_t)__cvta_generic_to_shared(s_k + t_lo);
-  float w[3][RB], k[2][4];
-  window<RB>(xb, w[0]);
-  lds4(kb, k[0]);
-  window<RB>(xb + 4 * RB, w[1]);
-  for (int t = t_lo; t <= t_hi; t += 24) {
-#pragma unroll
-    for (int s = 0; s < ST; ++s) {
-      window<RB>(xb + 4 * RB * (s + 2), w[(s + 2) % 3]);
-#pragma unroll
-      for (int v = 0; v < RB; v += 4) {
-        const int c = (s * (RB / 4) + v / 4) & 1;
-        lds4(kb + 4 * (s * RB + v + 4), k[c ^ 1]);
-#pragma unroll
-        for (int d = 0; d < 4; ++d) {
-#pragma unroll
-          for (int o = 0; o < RB; ++o)
-            acc[o] = fmaf(k[c][d], (o + v + d < RB) ? w[s % 3][o + v + d]
-                                                    : w[(s + 1) % 3][o + v + d - RB], acc[o]);
-        }
-      }
-    }
-    xb += 4 * 24;
-    kb += 4 * 24;
-  }
-}
-// FP64 (RB = 1): bound by the FP64 pipe (64 cycles a warp instruction and
-// scheduler); each lane runs its own taps inside the line, four per test.
-template <int RB>
-__device__ __forceinline__ void line_taps(double (&acc)[RB], const double* line, int pad,
-                                          const double* s_k, int n, int r, int i0) {
-  int t_lo = r - i0 - (RB - 1);
-  if (t_lo < 0) t_lo = 0;
-  int t_hi = n - 1 - i0 + r;
-  if (t_hi > 2 * r) t_hi = 2 * r;
-  const double* x = line + pad + i0 - r;
-  for (int t = t_lo; t <= t_hi; t += 4) {
-    double xx[4 + RB - 1], kk[4];
-#pragma unroll
-    for (int u = 0; u < 4 + RB - 1; ++u) xx[u] = x[t + u];
-#pragma unroll
-    for (int u = 0; u < 4; ++u) kk[u] = s_k[t + u];
-#pragma unroll
-    for (int u = 0; u < 4; ++u) {
-#pragma unroll
-      for (int o = 0; o < RB; ++o) acc[o] = fma(kk[u], xx[u + o], acc[o]);
-    }
-  }
-}
-
-// The warp's sum of the residual terms: a tree in the working precision (FP32
-// terms carry ~2^-24 each; the blocks and the grid are added in FP64).
-__device__ __forceinline__ double warp_res(float v) { return (double)warp_sum_f(v); }
-__device__ __forceinline__ double warp_res(double v) { return warp_sum(v); }
 
 template <typename T>
 struct StripArgs {
-  int nx, ny, rx, ry, nc, nr, gr;   // gr: blocks that own rows
-  unsigned mc, mr;               // ceil(2^32 / nc), ceil(2^32 / nr): division by multiply
-  const T* taps_x;
-  const T* taps_y;
-  const T* q;
-  T* a;
+  Geo g;
+  const T* q;                    // the step's input (two densities: 2 N)
+  const T* q2;                   // second column marginal: the attraction's target, q + N
+  const T* E1;                   // e^{-sigma w} of the two densities (species, pairwise)
+  const T* E2;
+  T t, kappa;                    // attraction: tau; pairwise: tau alpha; scalar bound (coupled)
+  int has_kappa;
+  T* a[2];
   T* p;
-  unsigned long long* x1;        // T: [row block][x][nr], even words per block
-  unsigned long long* x2;        // U: [column block][y][nc]
-  unsigned long long* xres;      // residuals of the blocks' rows, 2 words each, [2][gr]
-  unsigned* epoch;
   Ctrl* ctrl;
   int pairs;
 };
 
-// w / d for w < 2^16 d with m = ceil(2^32 / d) (d = 1: m wraps to 0)
-__device__ __forceinline__ int div_by(int w, int d, unsigned m) {
-  return d == 1 ? w : (int)__umulhi((unsigned)w, m);
+// The plain images of a block: by rows (q and the second marginal; pairwise: q_2,
+// e^{-sigma w_1}, p_1) and by columns (p, then the prox fields; species: p_1, p_2, e_1,
+// e_2; pairwise: q_1, e^{-sigma w_2}, p_2 and the three blurred images).
+template <typename T>
+__host__ __device__ inline void strip_images(int op, int ek, const ProxArgs<T>& P, int* rows,
+                                             int* cols) {
+  const int fields = (ek == EK_CROWD) + (P.sw != nullptr) + (P.c != nullptr) +
+                     (P.kappa != nullptr) + (P.m1f != nullptr);
+  *rows = op == OP_ONE ? 1 : op == OP_PAIR ? 3 : 2;
+  *cols = op == OP_SPECIES ? 4 : op == OP_PAIR ? 6 : 1 + fields;
 }
 
-// Shared memory of a block, in elements of T behind the taps.
-template <typename T>
-struct StripSmem {
-  int sc, sr;          // line strides of columns and rows
-  size_t kx, ky, a, c2, b, r2, q, p, E, sw, c, kap, m1f, mask, total;   // byte offsets
-};
-template <typename T>
-__host__ __device__ inline StripSmem<T> strip_smem(int nx, int ny, int rx, int ry, int nc, int nr,
-                                                   bool hE, bool hsw, bool hc, bool hkap,
-                                                   bool hm1f, bool hmask) {
-  StripSmem<T> S;
-  S.sc = line_stride(ny, ry);
-  S.sr = line_stride(nx, rx);
-  size_t o = 0;
-  auto take = [&](size_t n) { const size_t at = o; o += (n * sizeof(T) + 255) / 256 * 256; return at; };
-  S.kx = take(2 * rx + 1 + kTapPad);
-  S.ky = take(2 * ry + 1 + kTapPad);
-  S.a = take((size_t)nc * S.sc);
-  S.c2 = take((size_t)nc * S.sc);
-  S.b = take((size_t)nr * S.sr);
-  S.r2 = take((size_t)nr * S.sr);
-  S.q = take((size_t)nr * nx);
-  const size_t cc = (size_t)nc * ny;
-  S.p = take(cc);
-  S.E = take(hE ? cc : 0);
-  S.sw = take(hsw ? cc : 0);
-  S.c = take(hc ? cc : 0);
-  S.kap = take(hkap ? cc : 0);
-  S.m1f = take(hm1f ? cc : 0);
-  S.mask = o;
-  if (hmask) o += (cc + 127) / 128 * 128;
-  S.total = o + 256;   // (the base is rounded up)
-  return S;
-}
-
-template <typename T, int EK, int RB, int NT>
-__global__ void __launch_bounds__(NT, 1) strip_kernel(StripArgs<T> A, ProxArgs<T> P) {
+template <typename T, int OP, int EK, int RB, int NT>
+__global__ void __launch_bounds__(NT, 1)
+strip_kernel(const __grid_constant__ StripArgs<T> A, const __grid_constant__ ProxArgs<T> P) {
+  constexpr int NI = op_images(OP);
+  // the energy's fields as the prox reads them (one density, attraction)
+  constexpr bool FIELDS = OP == OP_ONE || OP == OP_ATTRACT;
+  // several couplings with b = q / Y: the step starts from b = 1 with its second half
+  constexpr bool FROM_B = OP == OP_ATTRACT || OP == OP_SPECIES;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   // 256-byte aligned: window() applies sw() to absolute shared addresses
   unsigned char* smem = smem_raw + (-(int)__cvta_generic_to_shared(smem_raw) & 255);
   __shared__ int s_bad, s_fault, s_dec;
   __shared__ double s_wres[NT / 32];
-  constexpr int KW = kWords<T>;
   const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
   const int nthreads = blockDim.x, nwarps = nthreads >> 5;
-  const int nx = A.nx, ny = A.ny;
-  const StripSmem<T> S = strip_smem<T>(nx, ny, A.rx, A.ry, A.nc, A.nr, EK == EK_CROWD,
-                                       P.sw != nullptr, P.c != nullptr, P.kappa != nullptr,
-                                       P.m1f != nullptr, P.mask != nullptr);
-  T* s_kx = (T*)(smem + S.kx);
-  T* s_ky = (T*)(smem + S.ky);
-  T* s_a = (T*)(smem + S.a);     // a by columns
-  T* s_c2 = (T*)(smem + S.c2);   // U received / T to send, by columns
-  T* s_b = (T*)(smem + S.b);     // b by rows
-  T* s_r2 = (T*)(smem + S.r2);   // T received / U to send, by rows
-  T* s_q = (T*)(smem + S.q);
-  T* s_p = (T*)(smem + S.p);
-  const int padc = line_pad(A.ry), padr = line_pad(A.rx);
+  const int nx = A.g.nx, ny = A.g.ny;
+  int n_row, n_col;
+  strip_images<T>(OP, EK, P, &n_row, &n_col);
+  const bool has_mask = FIELDS && P.mask != nullptr;
+  const Smem S = smem_of<T>(nx, ny, A.g.rx, A.g.ry, A.g.nc, A.g.nr, NI, n_row, n_col, has_mask);
+  Strips<T, NI, RB> X(A.g, S, smem, &s_fault);
+  auto row = [&](int k) { return (T*)(smem + S.row + k * S.row_b); };
+  auto col = [&](int k) { return (T*)(smem + S.col + k * S.col_b); };
   Ctrl* ctrl = A.ctrl;
-  // this block's columns [x0, x0 + ncg) and rows [y0, y0 + nrg)
-  const int x0 = blockIdx.x * A.nc, y0 = blockIdx.x * A.nr;
-  const int ncg = max(0, min(A.nc, nx - x0)), nrg = max(0, min(A.nr, ny - y0));
+  const int ncg = X.ncg, nrg = X.nrg;
   const int done0 = *(volatile int*)&ctrl->done, bad0 = *(volatile int*)&ctrl->nonfinite;
   if (done0 != RUNNING || bad0) {   // the same state for every block: none waits for this one
     if (done0 == RUNNING && tid == 0 && blockIdx.x == 0) ctrl->done = NONFINITE;
@@ -261,268 +101,291 @@ __global__ void __launch_bounds__(NT, 1) strip_kernel(StripArgs<T> A, ProxArgs<T
   }
   const int maxit = ctrl->max_iter, stall = ctrl->stall;
   const double tol = ctrl->tol;
-  const unsigned ep0 = *(volatile unsigned*)A.epoch;
+  const unsigned ep0 = *(volatile unsigned*)A.g.epoch;
   if (tid == 0) {
     s_bad = 0;
     s_fault = 0;
     s_dec = 0;
   }
 
-  // taps, zeros around the lines, a = 1 (Sec. 3.4), q and the prox fields
-  for (int t = tid; t < 2 * A.rx + 1 + kTapPad; t += nthreads)
-    s_kx[t] = t <= 2 * A.rx ? A.taps_x[t] : T(0);
-  for (int t = tid; t < 2 * A.ry + 1 + kTapPad; t += nthreads)
-    s_ky[t] = t <= 2 * A.ry ? A.taps_y[t] : T(0);
-  for (int l = wid; l < A.nc; l += nwarps)
-    for (int i = lane; i < S.sc; i += 32) {
-      s_c2[l * S.sc + i] = T(0);
-      s_a[l * S.sc + sw<T, RB>(i)] = (i >= padc && i < padc + ny) ? T(1) : T(0);
-    }
-  for (int l = wid; l < A.nr; l += nwarps)
-    for (int i = lane; i < S.sr; i += 32) {
-      s_b[l * S.sr + i] = T(0);
-      s_r2[l * S.sr + i] = T(0);
-    }
-  for (int l = wid; l < nrg; l += nwarps)
-    for (int i = lane; i < nx; i += 32) s_q[l * nx + i] = A.q[(size_t)(y0 + l) * nx + i];
-  // the prox fields by columns: element xl * ny + y of the block's copy
+  // taps, zeroed lines, the marginals and the prox fields
+  X.load_taps();
   ProxArgs<T> L = P;
-  auto field = [&](const T* g, size_t at) -> const T* {
-    T* s = (T*)(smem + at);
-    for (int e = tid; e < ny * ncg; e += nthreads) {
-      const int y = e / ncg, xl = e - y * ncg;
-      s[xl * ny + y] = g[(size_t)y * nx + x0 + xl];
+  if (OP == OP_PAIR) {
+    X.load_rows(A.q2, row(0));
+    X.load_rows(A.E1, row(1));
+    X.load_cols(A.q, col(0));
+    X.load_cols(A.E2, col(1));
+    for (int e = tid; e < nx * nrg; e += nthreads) row(2)[e] = T(0);
+    for (int e = tid; e < ny * ncg; e += nthreads) col(2)[e] = T(0);
+  } else {
+    X.load_rows(A.q, row(0));
+    if (NI == 2) X.load_rows(A.q2, row(1));
+    for (int e = tid; e < ny * A.g.nc; e += nthreads) {
+      col(0)[e] = T(0);
+      if (OP == OP_SPECIES) col(1)[e] = T(0);
     }
-    return s;
-  };
-  if (EK == EK_CROWD) L.E = field(P.E, S.E);
-  if (P.sw != nullptr) L.sw = field(P.sw, S.sw);
-  if (P.c != nullptr) L.c = field(P.c, S.c);
-  if (P.kappa != nullptr) L.kappa = field(P.kappa, S.kap);
-  if (P.m1f != nullptr) L.m1f = field(P.m1f, S.m1f);
-  if (P.mask != nullptr) {
-    uint8_t* s = (uint8_t*)(smem + S.mask);
-    for (int e = tid; e < ny * ncg; e += nthreads) {
-      const int y = e / ncg, xl = e - y * ncg;
-      s[xl * ny + y] = P.mask[(size_t)y * nx + x0 + xl];
-    }
-    L.mask = s;
   }
-  for (int e = tid; e < ny * A.nc; e += nthreads) s_p[e] = T(0);
-  __syncthreads();
-
-  // The filter along the owned axis: lines of n elements in `src`, RB outputs
-  // per work item, op(line, first output, outputs).
-  auto filter = [&](const T* src, int stride, int pad, int lines, int n, int r, const T* s_k,
-                    auto&& op) {
-    const int nseg = (n + RB - 1) / RB;
-    for (int item = tid; item < lines * nseg; item += nthreads) {
-      const int l = item / nseg, i0 = (item - l * nseg) * RB;
-      T acc[RB];
-#pragma unroll
-      for (int o = 0; o < RB; ++o) acc[o] = T(0);
-      line_taps<RB>(acc, src + l * stride, pad, s_k, n, r, i0);
-      op(l, i0, acc);
-    }
-  };
-  // outputs of a filter into the lines of dst (what lies there has been sent or read)
-  auto to_lines = [&](T* dst, int stride, int pad, int n) {
-    return [=](int l, int i0, T (&acc)[RB]) {
-#pragma unroll
-      for (int o = 0; o < RB; ++o)
-        if (i0 + o < n) dst[l * stride + sw<T, RB>(pad + i0 + o)] = acc[o];
+  if (OP == OP_SPECIES) {
+    X.load_cols(A.E1, col(2));
+    X.load_cols(A.E2, col(3));
+  }
+  if (FIELDS) {
+    int k = 1;
+    auto field = [&](const T* g) -> const T* {
+      T* s = col(k++);
+      X.load_cols(g, s);
+      return s;
     };
-  };
-  // Sends the lines of src (n elements each, the block's lines [l0, l0 + lines) of
-  // `total`): element i goes to block i / d of the other axis, its words at
-  // [i / d][line][i mod d].
-  auto send = [&](unsigned long long* X, const T* src, int stride, int pad, int l0, int lines,
-                  int total, int n, int d, unsigned m, unsigned ep) {
-    const size_t region = ((size_t)total * d * KW + 1) & ~(size_t)1;
-    for (int i = tid; i < n; i += nthreads) {
-      const int g = div_by(i, d, m), il = i - g * d;
-      unsigned long long* w = X + g * region + ((size_t)l0 * d + il) * KW;
-      const T* s = src + sw<T, RB>(pad + i);
-      for (int l = 0; l < lines; ++l) put_elem(w + (size_t)l * d * KW, s[l * stride], ep);
-    }
-  };
-  // Receives this block's lines (d per block, `lines` of them in use, n elements
-  // each) into dst: the words [block][element][line].
-  auto receive = [&](const unsigned long long* X, T* dst, int stride, int pad, int lines, int n,
-                     int d, unsigned m, unsigned ep) {
-    if (lines == 0) return;
-    const size_t region = ((size_t)n * d * KW + 1) & ~(size_t)1;
-    const unsigned long long* w0 = X + blockIdx.x * region;
-    constexpr int UN = 4;   // pairs of words in flight per thread
-    const int npair = (n * d * KW + 1) >> 1;
-    for (int k0 = tid; k0 < npair; k0 += nthreads * UN) {
-      unsigned long long x[UN], y[UN];
-#pragma unroll
-      for (int u = 0; u < UN; ++u) {
-        const int k = k0 + u * nthreads;
-        x[u] = y[u] = (unsigned long long)ep << 32;
-        if (k < npair) get_words(w0 + 2 * (size_t)k, x[u], y[u]);
+    if (EK == EK_CROWD) L.E = field(P.E);
+    if (P.sw != nullptr) L.sw = field(P.sw);
+    if (P.c != nullptr) L.c = field(P.c);
+    if (P.kappa != nullptr) L.kappa = field(P.kappa);
+    if (P.m1f != nullptr) L.m1f = field(P.m1f);
+    if (has_mask) {
+      uint8_t* s = (uint8_t*)(smem + S.mask);
+      for (int e = tid; e < ny * ncg; e += nthreads) {
+        const int y = e / ncg, xl = e - y * ncg;
+        s[xl * ny + y] = P.mask[(size_t)y * nx + X.x0 + xl];
       }
-#pragma unroll
-      for (int u = 0; u < UN; ++u) {
-        const int k = k0 + u * nthreads;
-        if (k >= npair) continue;
-        if (KW == 2) {
-          const int i = div_by(k, d, m), l = k - i * d;
-          if (l >= lines) continue;
-          if (!wait_pair(w0 + 2 * (size_t)k, ep, x[u], y[u], &s_fault)) s_fault = 1;
-          dst[l * stride + sw<T, RB>(pad + i)] = (T)words_double(x[u], y[u]);
-        } else {
-          // elements 2k and 2k + 1; the last block of a ragged grid has lines
-          // that nobody sends, and an odd region ends in an unused word
-          const int e0 = 2 * k, e1 = 2 * k + 1;
-          const int i0 = div_by(e0, d, m), l0 = e0 - i0 * d;
-          const int i1 = div_by(e1, d, m), l1 = e1 - i1 * d;
-          const bool u0 = l0 < lines, u1 = i1 < n && l1 < lines;
-          for (unsigned t = 0; (u0 && (unsigned)(x[u] >> 32) != ep) ||
-                               (u1 && (unsigned)(y[u] >> 32) != ep); ++t) {
-            if (t >= kSpin || *(volatile int*)&s_fault) {
-              s_fault = 1;
-              break;
-            }
-            get_words(w0 + 2 * (size_t)k, x[u], y[u]);
-          }
-          if (u0) dst[l0 * stride + sw<T, RB>(pad + i0)] = (T)__uint_as_float((unsigned)x[u]);
-          if (u1) dst[l1 * stride + sw<T, RB>(pad + i1)] = (T)__uint_as_float((unsigned)y[u]);
-        }
-      }
+      L.mask = s;
     }
-  };
+  }
+  __syncthreads();
+  // the cold start (Sec. 3.4, Prop. prop-implementation-generic): a = 1, or b = 1
+  if (FROM_B) {
+    for (int l = 0; l < NI * A.g.nr; ++l)
+      for (int i = tid; i < nx; i += nthreads) X.b[X.at_r(0, l, i)] = T(1);
+  } else {
+    for (int l = 0; l < NI * A.g.nc; ++l)
+      for (int i = tid; i < ny; i += nthreads) X.a[X.at_c(0, l, i)] = T(1);
+  }
+  __syncthreads();
 
   int it = 0, pair = 0, since = 0;
   double best = INFINITY;
-  for (; pair < A.pairs; ++pair) {
-    const unsigned ep = ep0 + 1u + (unsigned)pair;
-    // columns: T = K_y a
-    filter(s_a, S.sc, padc, ncg, ny, A.ry, s_ky, to_lines(s_c2, S.sc, padc, ny));
-    __syncthreads();
-    send(A.x1, s_c2, S.sc, padc, x0, ncg, nx, ny, A.nr, A.mr, ep);
-    receive(A.x1, s_r2, S.sr, padr, nrg, nx, A.nr, A.mr, ep);
-    __syncthreads();
-    // rows: Y = T K_x, the residual |b_old Y - q| and b = q / Y
-    const bool have_prev = it > 0;
-    int bad = 0;
-    T res = T(0);
-    filter(s_r2, S.sr, padr, nrg, nx, A.rx, s_kx, [&](int l, int i0, T (&acc)[RB]) {
-#pragma unroll
-      for (int o = 0; o < RB; ++o) {
-        if (i0 + o >= nx) continue;
-        const T qv = s_q[l * nx + i0 + o];
-        T* bp = s_b + l * S.sr + sw<T, RB>(padr + i0 + o);
-        if (have_prev) res += abs_residual<T>(*bp, acc[o], qv);
-        const T bn = b_update<T>(qv, acc[o]);
-        bad |= !dev_finite(bn);
-        *bp = bn;
-      }
-    });
-    // the warps' residuals in the working precision, the block's and the grid's in FP64
-    const double wres = warp_res(res);
-    if (lane == 0) s_wres[wid] = wres;
-    if (bad) s_bad = 1;
-    __syncthreads();
-    // the block's residual (NaN where it met a non-finite scaling) to every block
-    unsigned long long* xr = A.xres + (size_t)(pair & 1) * A.gr * 2;
-    if (wid == 0 && nrg > 0) {
+  // the block's residual (NaN where it met a non-finite scaling) to every block
+  const int n_res = OP == OP_PAIR ? A.g.gc : A.g.gr;
+  auto put_residual = [&](unsigned ep) {
+    unsigned long long* xr = A.g.xres + (size_t)(pair & 1) * n_res * 2;
+    if (wid == 0 && (int)blockIdx.x < n_res) {
       const double v = warp_sum(lane < nwarps ? s_wres[lane] : 0.0);
       if (lane == 0) put_elem(xr + 2 * blockIdx.x, s_bad ? (double)NAN : v, ep);
     }
-    // U = b K_x, rows -> columns
-    filter(s_b, S.sr, padr, nrg, nx, A.rx, s_kx, to_lines(s_r2, S.sr, padr, nx));
-    __syncthreads();
-    send(A.x2, s_r2, S.sr, padr, y0, nrg, ny, nx, A.nc, A.mc, ep);
-    if (wid == nwarps - 1) {
-      // the stop rule (Sec. 3.4) on the sum over the blocks, in one order everywhere
-      constexpr int UN = 5;   // blocks per lane whose words are in flight at once
-      double v = 0.0;
-      for (int g0 = lane; g0 < A.gr; g0 += 32 * UN) {
-        unsigned long long lo[UN], hi[UN];
-#pragma unroll
-        for (int u = 0; u < UN; ++u)
-          if (g0 + 32 * u < A.gr) get_words(xr + 2 * (g0 + 32 * u), lo[u], hi[u]);
-#pragma unroll
-        for (int u = 0; u < UN; ++u)
-          if (g0 + 32 * u < A.gr) {
-            if (!wait_pair(xr + 2 * (g0 + 32 * u), ep, lo[u], hi[u], &s_fault)) s_fault = 1;
-            v += words_double(lo[u], hi[u]);
-          }
-      }
-      v = warp_sum(v);
-      const bool first = lane == 0 && blockIdx.x == 0;
-      int d = RUNNING;
-      if (!isfinite(v)) d = NONFINITE;
-      else if (it > 0 && v <= tol) d = CONVERGED;
-      else if (it >= maxit) d = MAX_ITER;
-      else if (stall > 0 && it >= 1) {
-        // the stall rule (stall_rule), its state in this warp: every block keeps the same
-        since = (it == 1 || v < best) ? 0 : since + 1;
-        best = it == 1 ? v : fmin(best, v);
-        if (since >= stall) d = STALLED;
-      }
-      if (first) {
-        if (it > 0) ctrl->res_last = v;
-        if (d != RUNNING) ctrl->done = d;
-      }
-      if (lane == 0) s_dec = d != RUNNING;
+  };
+  // the stop rule (Sec. 3.4) on the sum over the blocks' residuals of pair `of`, put with ep
+  auto decide = [&](int of, unsigned ep) {
+    const double v = X.gather_sum(A.g.xres + (size_t)(of & 1) * n_res * 2, n_res, ep);
+    const bool first = lane == 0 && blockIdx.x == 0;
+    int d = RUNNING;
+    if (!isfinite(v)) d = NONFINITE;
+    else if (it > 0 && v <= tol) d = CONVERGED;
+    else if (it >= maxit) d = MAX_ITER;
+    else if (stall > 0 && it >= 1) {
+      // the stall rule (stall_rule), its state in this warp: every block keeps the same
+      since = (it == 1 || v < best) ? 0 : since + 1;
+      best = it == 1 ? v : fmin(best, v);
+      if (since >= stall) d = STALLED;
     }
-    receive(A.x2, s_c2, S.sc, padc, ncg, ny, A.nc, A.mc, ep);
+    if (first) {
+      if (it > 0) ctrl->res_last = v;
+      if (d != RUNNING) ctrl->done = d;
+    }
+    if (lane == 0) s_dec = d != RUNNING;
+  };
+  for (; pair < A.pairs; ++pair) {
+    const unsigned ep = ep0 + 1u + (unsigned)pair;
+    int bad = 0;
+    if (!FROM_B || pair > 0) {
+      // columns: T = K_y a
+      X.filter_cols_to(X.a, X.c2);
+      __syncthreads();
+      X.send_cols(ep);
+      if (OP == OP_PAIR && pair > 0 && wid == nwarps - 1) decide(pair - 1, ep - 1u);
+      X.receive_rows(ep);
+      __syncthreads();
+      if (OP == OP_PAIR) {
+        if (s_dec || s_fault) break;
+        // rows: s_m = xi b_m, then the common row marginal p_1 of couplings 1 and 3 and
+        // the fixed rows q_2 of coupling 2
+        X.filter_rows_to(X.r2, X.b);
+        __syncthreads();
+        for (int l = 0; l < nrg; ++l)
+          for (int i = tid; i < nx; i += nthreads) {
+            const int e = l * nx + i;
+            T* b1 = X.b + X.at_r(0, l, i);
+            T* b2 = X.b + X.at_r(1, l, i);
+            T* b3 = X.b + X.at_r(2, l, i);
+            const T x1 = *b1, x3 = *b3;
+            const T pm = pairwise_marginal<T>(x1, x3, A.t, row(1)[e], A.kappa, A.has_kappa);
+            const T r1 = safe_ratio<T>(pm, x1), r3 = safe_ratio<T>(pm, x3);
+            const T r2 = b_update<T>(row(0)[e], *b2);
+            bad |= !dev_finite(r1) || !dev_finite(r2) || !dev_finite(r3) || !dev_finite(pm);
+            *b1 = r1;
+            *b2 = r2;
+            *b3 = r3;
+            row(2)[e] = pm;
+          }
+        if (bad) s_bad = 1;
+      } else {
+        // rows: Y = T K_x, the residual |b_old Y - q| and b = q / Y
+        const bool have_prev = it > 0;
+        T res = T(0);
+        X.filter_rows(X.r2, [&](int m, int l, int i0, T (&acc)[RB]) {
+          const T* qm = row(m);
+#pragma unroll
+          for (int o = 0; o < RB; ++o) {
+            if (i0 + o >= nx) continue;
+            const T qv = qm[l * nx + i0 + o];
+            T* bp = X.b + X.at_r(m, l, i0 + o);
+            if (have_prev) res += abs_residual<T>(*bp, acc[o], qv);
+            const T bn = b_update<T>(qv, acc[o]);
+            bad |= !dev_finite(bn);
+            *bp = bn;
+          }
+        });
+        // the warps' residuals in the working precision, the block's and the grid's in FP64
+        const double wres = warp_res(res);
+        if (lane == 0) s_wres[wid] = wres;
+        if (bad) s_bad = 1;
+      }
+      __syncthreads();
+      if (OP != OP_PAIR) put_residual(ep);
+    }
+    // U = b K_x, rows -> columns
+    X.filter_rows_to(X.b, X.r2);
+    __syncthreads();
+    X.send_rows(ep);
+    if (OP != OP_PAIR && (!FROM_B || pair > 0) && wid == nwarps - 1) decide(pair, ep);
+    X.receive_cols(ep);
     __syncthreads();
     if (s_dec || s_fault) break;
-    // columns: s = K_y U, a = Prox(s) / s, p = a s
     bad = 0;
-    filter(s_c2, S.sc, padc, ncg, ny, A.ry, s_ky, [&](int l, int i0, T (&acc)[RB]) {
+    if (OP == OP_ONE) {
+      // columns: s = K_y U, a = Prox(s) / s, p = a s
+      T* s_p = col(0);
+      X.filter_cols(X.c2, [&](int, int l, int i0, T (&acc)[RB]) {
 #pragma unroll
-      for (int o = 0; o < RB; ++o) {
-        if (i0 + o >= ny) continue;
-        const int idx = l * ny + i0 + o;
-        const T a = prox_ratio<T, EK>(L, idx, acc[o]);
-        bad |= !dev_finite(a);
-        s_a[l * S.sc + sw<T, RB>(padc + i0 + o)] = a;
-        s_p[idx] = a * acc[o];
-      }
-    });
+        for (int o = 0; o < RB; ++o) {
+          if (i0 + o >= ny) continue;
+          const int idx = l * ny + i0 + o;
+          const T a = prox_ratio<T, EK>(L, idx, acc[o]);
+          bad |= !dev_finite(a);
+          X.a[X.at_c(0, l, i0 + o)] = a;
+          s_p[idx] = a * acc[o];
+        }
+      });
+    } else if (OP == OP_PAIR) {
+      // columns: y_m = xi a_m; the residual against the column constraints, p_2 = b_2 y_2,
+      // then the common column marginal of couplings 2 and 3 and b_1 = q_1 / y_1
+      X.filter_cols(X.c2, [&](int m, int l, int i0, T (&acc)[RB]) {
+        T* v = col(3 + m) + l * ny + i0;
+#pragma unroll
+        for (int o = 0; o < RB; ++o)
+          if (i0 + o < ny) v[o] = acc[o];
+      });
+      __syncthreads();
+      double res = 0.0;
+      for (int l = 0; l < ncg; ++l)
+        for (int i = tid; i < ny; i += nthreads) {
+          const int e = l * ny + i;
+          const T v1 = col(3)[e], v2 = col(4)[e], v3 = col(5)[e], qq = col(0)[e];
+          T* b1 = X.a + X.at_c(0, l, i);
+          T* b2 = X.a + X.at_c(1, l, i);
+          T* b3 = X.a + X.at_c(2, l, i);
+          const T c2 = *b2 * v2;
+          res += (double)abs_residual<T>(*b1, v1, qq) + (double)fabs(c2 - *b3 * v3);
+          col(2)[e] = c2;
+          const T pm = pairwise_marginal<T>(v2, v3, A.t, col(1)[e], A.kappa, A.has_kappa);
+          const T r1 = b_update<T>(qq, v1);
+          const T r2 = safe_ratio<T>(pm, v2), r3 = safe_ratio<T>(pm, v3);
+          bad |= !dev_finite(r1) || !dev_finite(r2) || !dev_finite(r3);
+          *b1 = r1;
+          *b2 = r2;
+          *b3 = r3;
+        }
+      res = warp_sum(res);
+      if (lane == 0) s_wres[wid] = res;
+    } else {
+      // columns: s_m = K_y U_m, then the joint prox
+      X.filter_cols_to(X.c2, X.a);
+      __syncthreads();
+      const T w1 = T(1) / (T(1) + A.t), w2 = A.t / (T(1) + A.t);
+      for (int l = 0; l < ncg; ++l)
+        for (int i = tid; i < ny; i += nthreads) {
+          const int e = l * ny + i;
+          T* a1 = X.a + X.at_c(0, l, i);
+          T* a2 = X.a + X.at_c(1, l, i);
+          T r1, r2, p1, p2 = T(0);
+          if (OP == OP_ATTRACT) {
+            attraction_cell<T, EK>(L, e, *a1, *a2, w1, w2, r1, r2, p1);
+            bad |= !dev_finite(r1) || !dev_finite(r2) || !dev_finite(p1);
+          } else {
+            species_cell<T>(*a1, *a2, col(2)[e], col(3)[e], A.kappa, A.has_kappa, r1, r2, p1, p2);
+            bad |= !dev_finite(p1) || !dev_finite(p2);
+            col(1)[e] = p2;
+          }
+          *a1 = r1;
+          *a2 = r2;
+          col(0)[e] = p1;
+        }
+    }
     if (bad) s_bad = 1;
     ++it;
     __syncthreads();
+    if (OP == OP_PAIR) put_residual(ep);
   }
 
   // the final a and p (p of the pair the last residual belongs to)
   for (int e = tid; e < ny * ncg; e += nthreads) {
     const int y = e / ncg, xl = e - y * ncg;
-    A.a[(size_t)y * nx + x0 + xl] = s_a[xl * S.sc + sw<T, RB>(padc + y)];
-    A.p[(size_t)y * nx + x0 + xl] = s_p[xl * ny + y];
+    const size_t at = (size_t)y * nx + X.x0 + xl;
+    if (OP == OP_PAIR) {
+      A.p[(size_t)nx * ny + at] = col(2)[xl * ny + y];
+    } else {
+#pragma unroll
+      for (int m = 0; m < (NI < 2 ? NI : 2); ++m) A.a[m][at] = X.a[X.at_c(m, xl, y)];
+      A.p[at] = col(0)[xl * ny + y];
+      if (OP == OP_SPECIES) A.p[(size_t)nx * ny + at] = col(1)[xl * ny + y];
+    }
   }
+  if (OP == OP_PAIR)
+    for (int e = tid; e < nx * nrg; e += nthreads) A.p[(size_t)X.y0 * nx + e] = row(2)[e];
   if (tid == 0) {
     if (s_fault) atomicOr(&ctrl->nonfinite, 2);
     if (blockIdx.x == 0) {
       ctrl->it = it;
-      *A.epoch = ep0 + 1u + (unsigned)pair;
+      *A.g.epoch = ep0 + 1u + (unsigned)pair;
     }
   }
 }
 
 // ---- host ----
-template <typename T, int RB, int NT>
+template <typename T, int OP, int RB, int NT>
 void* strip_fn_ek(int ek) {
-  if (ek == EK_CROWD) return (void*)strip_kernel<T, EK_CROWD, RB, NT>;
-  if (ek == EK_ENTROPY) return (void*)strip_kernel<T, EK_ENTROPY, RB, NT>;
-  return (void*)strip_kernel<T, EK_POWER, RB, NT>;
+  if (OP == OP_SPECIES || OP == OP_PAIR || ek == EK_CROWD)
+    return (void*)strip_kernel<T, OP, EK_CROWD, RB, NT>;
+  constexpr int O = OP == OP_SPECIES || OP == OP_PAIR ? OP_ONE : OP;
+  if (ek == EK_ENTROPY) return (void*)strip_kernel<T, O, EK_ENTROPY, RB, NT>;
+  return (void*)strip_kernel<T, O, EK_POWER, RB, NT>;
+}
+template <typename T, int RB, int NT>
+void* strip_fn_op(int op, int ek) {
+  switch (op) {
+    case OP_ONE: return strip_fn_ek<T, OP_ONE, RB, NT>(ek);
+    case OP_ATTRACT: return strip_fn_ek<T, OP_ATTRACT, RB, NT>(ek);
+    case OP_SPECIES: return strip_fn_ek<T, OP_SPECIES, RB, NT>(ek);
+    default: return strip_fn_ek<T, OP_PAIR, RB, NT>(ek);
+  }
 }
 template <typename T>
-void* strip_fn(int rb, int ek);
+void* strip_fn(int rb, int op, int ek);
 template <>
-void* strip_fn<float>(int rb, int ek) {
-  return rb == 8 ? strip_fn_ek<float, 8, 512>(ek) : strip_fn_ek<float, 4, 512>(ek);
+void* strip_fn<float>(int rb, int op, int ek) {
+  return rb == 8 ? strip_fn_op<float, 8, 512>(op, ek) : strip_fn_op<float, 4, 512>(op, ek);
 }
 template <>
-void* strip_fn<double>(int, int ek) { return strip_fn_ek<double, 1, 512>(ek); }
-
-int ceil_div(int a, int b) { return (a + b - 1) / b; }
-unsigned magic(int d) { return (unsigned)((0x100000000ull + (unsigned)d - 1) / (unsigned)d); }
+void* strip_fn<double>(int, int op, int ek) { return strip_fn_op<double, 1, 512>(op, ek); }
 
 }  // namespace
 
@@ -538,8 +401,10 @@ unsigned magic(int d) { return (unsigned)((0x100000000ull + (unsigned)d - 1) / (
 // few lines for the blocks, keep the per-pass form unless a block's line is
 // short work anyway.
 template <typename T>
-StripPlan strip_plan(int nx, int ny, int rx, int ry, int ek, const ProxArgs<T>& P, int max_blocks) {
+StripPlan strip_plan(int nx, int ny, int rx, int ry, int op, int ek, const ProxArgs<T>& P,
+                     int max_blocks) {
   StripPlan sp;
+  const int ni = op_images(op);
   int dev = 0, coop = 0, sms = 0, smem_max = 0;
   if (cudaGetDevice(&dev) != cudaSuccess) return sp;
   cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev);
@@ -557,16 +422,16 @@ StripPlan strip_plan(int nx, int ny, int rx, int ry, int ek, const ProxArgs<T>& 
   // eight outputs per work item where that leaves every scheduler two warps, else four
   // (256^2: 8.8 us a pair with four, 11.4 with eight; 1024^2 72 and 64); FP64: one
   auto items = [&](int rb) {
-    return std::max(sp.nc * ceil_div(ny, rb), sp.nr * ceil_div(nx, rb));
+    return ni * std::max(sp.nc * ceil_div(ny, rb), sp.nr * ceil_div(nx, rb));
   };
   sp.rb = sizeof(T) == 8 ? 1 : items(8) >= 256 ? 8 : 4;
   sp.threads = std::min(512, std::max(256, ceil_div(items(sp.rb), 32) * 32));
-  const auto S = strip_smem<T>(nx, ny, rx, ry, sp.nc, sp.nr, ek == EK_CROWD,
-                               P.sw != nullptr, P.c != nullptr, P.kappa != nullptr,
-                               P.m1f != nullptr, P.mask != nullptr);
+  int rows = 0, cols = 0;
+  strip_images<T>(op, ek, P, &rows, &cols);
+  const Smem S = smem_of<T>(nx, ny, rx, ry, sp.nc, sp.nr, ni, rows, cols, P.mask != nullptr);
   sp.smem = S.total;
   if (S.total + 1024 > (size_t)smem_max) return StripPlan{};
-  void* fn = strip_fn<T>(sp.rb, ek);
+  void* fn = strip_fn<T>(sp.rb, op, ek);
   int per_sm = 0;
   if (cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)S.total) !=
           cudaSuccess ||
@@ -577,45 +442,54 @@ StripPlan strip_plan(int nx, int ny, int rx, int ry, int ek, const ProxArgs<T>& 
     return StripPlan{};
   }
   const size_t kw = sizeof(T) / 4;
-  const size_t r1 = ((size_t)nx * sp.nr * kw + 1) & ~(size_t)1;
-  const size_t r2 = ((size_t)ny * sp.nc * kw + 1) & ~(size_t)1;
+  const size_t r1 = ((size_t)ni * nx * sp.nr * kw + 1) & ~(size_t)1;
+  const size_t r2 = ((size_t)ni * ny * sp.nc * kw + 1) & ~(size_t)1;
   sp.x1_words = r1 * ceil_div(ny, sp.nr);
   sp.x2_words = r2 * ceil_div(nx, sp.nc);
   sp.words = sp.x1_words + sp.x2_words + 4 * (size_t)sp.G + 2;
   return sp;
 }
 
-template <typename T>
-cudaError_t strip_launch(const StripPlan& sp, int ek, int nx, int ny, int rx, int ry,
-                         const T* taps_x, const T* taps_y, const T* q, T* a, T* p,
-                         const ProxArgs<T>& P, Ctrl* ctrl, unsigned long long* words, int pairs,
-                         cudaStream_t st) {
-  StripArgs<T> A{nx, ny, rx, ry, sp.nc, sp.nr, ceil_div(ny, sp.nr), magic(sp.nc), magic(sp.nr), taps_x, taps_y, q, a, p,
-                 words, words + sp.x1_words, words + sp.x1_words + sp.x2_words,
-                 (unsigned*)(words + sp.words - 2), ctrl, pairs};
-  ProxArgs<T> Pc = P;
-  void* args[] = {&A, &Pc};
+strip::Geo strip_geo(const StripPlan& sp, int nx, int ny, int rx, int ry, const void* taps_x,
+                     const void* taps_y, unsigned long long* words) {
+  return Geo{nx, ny, rx, ry, sp.nc, sp.nr, ceil_div(ny, sp.nr), ceil_div(nx, sp.nc),
+             magic(sp.nc), magic(sp.nr), taps_x, taps_y, words, words + sp.x1_words,
+             words + sp.x1_words + sp.x2_words, (unsigned*)(words + sp.words - 2)};
+}
+
+cudaError_t strip_coop(void* fn, const StripPlan& sp, size_t smem, int threads, void** args,
+                       cudaStream_t st) {
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3((unsigned)sp.G);
-  cfg.blockDim = dim3((unsigned)sp.threads);
-  cfg.dynamicSmemBytes = sp.smem;
+  cfg.blockDim = dim3((unsigned)threads);
+  cfg.dynamicSmemBytes = smem;
   cfg.stream = st;
   cudaLaunchAttribute at[1];
   at[0].id = cudaLaunchAttributeCooperative;
   at[0].val.cooperative = 1;
   cfg.attrs = at;
   cfg.numAttrs = 1;
-  void* fn = strip_fn<T>(sp.rb, ek);
   // another handle of the same kernel may have set a smaller limit
-  cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sp.smem);
+  cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
   return cudaLaunchKernelExC(&cfg, fn, args);
 }
 
-#define JKO_STRIP_INST(T)                                                                      \
-  template StripPlan strip_plan<T>(int, int, int, int, int, const ProxArgs<T>&, int);       \
-  template cudaError_t strip_launch<T>(const StripPlan&, int, int, int, int, int, const T*,    \
-                                       const T*, const T*, T*, T*, const ProxArgs<T>&, Ctrl*,  \
+template <typename T>
+cudaError_t strip_launch(const StripPlan& sp, int nx, int ny, int rx, int ry, const T* taps_x,
+                         const T* taps_y, const StripStep<T>& s, const ProxArgs<T>& P, Ctrl* ctrl,
+                         unsigned long long* words, int pairs, cudaStream_t st) {
+  StripArgs<T> A{strip_geo(sp, nx, ny, rx, ry, taps_x, taps_y, words), s.q, s.q2, s.E1, s.E2,
+                 (T)s.t, P.kappa_s, P.has_kappa, {s.a, s.a2}, s.p, ctrl, pairs};
+  ProxArgs<T> Pc = P;
+  void* args[] = {&A, &Pc};
+  return strip_coop(strip_fn<T>(sp.rb, s.op, s.ek), sp, sp.smem, sp.threads, args, st);
+}
+
+#define JKO_STRIP_INST(T)                                                                        \
+  template StripPlan strip_plan<T>(int, int, int, int, int, int, const ProxArgs<T>&, int);      \
+  template cudaError_t strip_launch<T>(const StripPlan&, int, int, int, int, const T*, const T*, \
+                                       const StripStep<T>&, const ProxArgs<T>&, Ctrl*,           \
                                        unsigned long long*, int, cudaStream_t);
 JKO_STRIP_INST(float)
 JKO_STRIP_INST(double)
