@@ -268,6 +268,53 @@ jko_status backward_t(jko_handle* h, const T* grad_final, T* grad_p0, T* grad_w,
   return JKO_OK;
 }
 
+// The same walk with one cooperative launch per step (strip_adjoint.cu), whose
+// solves test their own convergence: the host waits once, for the statuses of all steps.
+template <typename T>
+jko_status backward_strip(jko_handle* h, size_t smem, const T* grad_final, T* grad_p0, T* grad_w,
+                          int* adj_iters) {
+  cudaStream_t st = h->stream;
+  const size_t N = (size_t)h->N;
+  const int n = h->tape_steps;
+  if (!h->adj) ACK(cudaMalloc(&h->adj, sizeof(T) * N));
+  if (h->adj_status_cap < n) {
+    if (h->adj_status) cudaFree(h->adj_status);
+    h->adj_status = nullptr;
+    h->adj_status_cap = 0;
+    ACK(cudaMalloc((void**)&h->adj_status, sizeof(jko::AdjStatus) * h->tape_cap));
+    h->adj_status_cap = h->tape_cap;
+  }
+  ACK(cudaMemsetAsync(h->adj_status, 0, sizeof(jko::AdjStatus) * n, st));
+  if (grad_w) ACK(cudaMemsetAsync(grad_w, 0, sizeof(T) * N, st));
+  jko::StripAdjoint<T> s{};
+  s.wbar = grad_w;
+  s.renorm = h->prm.renormalize;
+  s.tol = std::max(h->prm.tol, h->fp64 ? 1e-15 : 1e-7);
+  s.budget = std::max(16, 10 * h->prm.max_iter);
+  s.gin = grad_final;
+  for (int t = n - 1; t >= 0; --t) {
+    s.q = (const T*)h->tape + 2 * (size_t)t * N;
+    s.a = s.q + N;
+    s.gout = t == 0 && grad_p0 ? grad_p0 : (T*)h->adj;
+    s.mass = h->tape_mass[t];
+    s.out = h->adj_status + t;
+    ACK(jko::strip_adjoint_launch<T>(h->strip, smem, h->ek, h->grid.nx, h->grid.ny, h->rx, h->ry,
+                                     (const T*)h->taps_x, (const T*)h->taps_y, s,
+                                     jko::prox_args<T>(h), h->strip_words, st));
+    s.gin = s.gout;
+    s.after = s.out;
+  }
+  std::vector<jko::AdjStatus> res(n);
+  ACK(cudaMemcpyAsync(res.data(), h->adj_status, sizeof(jko::AdjStatus) * n,
+                      cudaMemcpyDeviceToHost, st));
+  ACK(cudaStreamSynchronize(st));
+  if (res[0].bad & 2)
+    return jko::handle_error(h, JKO_ERR_TIMEOUT, "a bounded device-side wait gave up");
+  if (res[0].bad) return jko::handle_error(h, JKO_ERR_NUMERIC, "adjoint iterates are not finite");
+  for (int t = 0; adj_iters && t < n; ++t) adj_iters[t] = res[t].iters;
+  return JKO_OK;
+}
+
 // ---- the Wasserstein attraction (Sec. 5.2), congestion/potential energy ----
 // The step's fixed point over both couplings: Y_m = xi a_m, b_m = t_m / Y_m
 // (t_1 = q, t_2 = r), s_m = xi b_m, p = min(E g, kappa) with the geometric mean
@@ -577,6 +624,8 @@ template <typename T>
 jko_status backward_dispatch(jko_handle* h, const void* gf, void* gp, void* gw, int* it) {
   if (h->attract) return backward_attraction<T>(h, (const T*)gf, (T*)gp, (T*)gw, it);
   if (h->species == 2) return backward_species<T>(h, (const T*)gf, (T*)gp, (T*)gw, it);
+  if (const size_t smem = jko::strip_adjoint_smem<T>(h->strip, h->grid.nx, h->grid.ny, h->rx, h->ry))
+    return backward_strip<T>(h, smem, (const T*)gf, (T*)gp, (T*)gw, it);
   switch (h->ek) {
     case jko::EK_CROWD:
       return backward_t<T, jko::EK_CROWD>(h, (const T*)gf, (T*)gp, (T*)gw, it);

@@ -722,7 +722,7 @@ void free_handle(jko_handle* h) {
                   h->fft_khat_x, h->fft_tw_x, h->fft_khat_y, h->fft_tw_y,
                   h->tape, h->adj, h->adj2, h->adj_red, h->hb.d[0], h->hb.d[1], h->hb.d[2],
                   h->hb.d[3], h->hb.coef, h->a3, h->b3, h->s3, h->t2, h->t3, h->mpair,
-                  h->strip_words};
+                  h->strip_words, h->adj_status};
   for (void* b : bufs) if (b) cudaFree(b);
   if (h->ctrl_init) cudaFreeHost(h->ctrl_init);
   if (h->poll) cudaFreeHost(h->poll);

@@ -70,6 +70,8 @@ struct jko_handle {
   int heat_G = 0;         // blocks of the heat kernel's persistent form
   jko::StripPlan strip;   // the CUDA-core form's persistent kernel (G = 0: per-pass kernels)
   unsigned long long* strip_words = nullptr;   // its exchange buffers
+  jko::AdjStatus* adj_status = nullptr;        // its reverse pass: one per step of the tape
+  int adj_status_cap = 0;
   int tc_multi = 0;       // several couplings on the tensor cores (tc_multi.cu)
   void* mpair = nullptr;  // bf16 forms of several couplings: pairs of the first pass's images
   Ctrl* ctrl_init = nullptr;   // pinned initial value

@@ -104,6 +104,33 @@ cudaError_t strip_launch(const StripPlan& sp, int nx, int ny, int rx, int ry, co
                          const T* taps_y, const StripStep<T>& s, const ProxArgs<T>& P, Ctrl* ctrl,
                          unsigned long long* words, int pairs, cudaStream_t st);
 
+// One step of the reverse pass on the same strips (strip_adjoint.cu).
+struct AdjStatus {
+  int iters;           // iterations of the adjoint solve
+  int bad;             // bit 0: its iterates are not finite; bit 1: a bounded wait gave up
+};
+template <typename T>
+struct StripAdjoint {
+  const T* q;          // the step's input and final a
+  const T* a;
+  const T* gin;        // gradient with respect to the step's output, and to its input
+  T* gout;
+  T* wbar;             // accumulates, or NULL
+  double mass;
+  int renorm;
+  double tol;
+  int budget;
+  AdjStatus* out;          // device, zeroed
+  const AdjStatus* after;  // status of the step walked before this one, or NULL
+};
+// shared memory of its launch; 0: the kernels per pass
+template <typename T>
+size_t strip_adjoint_smem(const StripPlan& sp, int nx, int ny, int rx, int ry);
+template <typename T>
+cudaError_t strip_adjoint_launch(const StripPlan& sp, size_t smem, int ek, int nx, int ny, int rx,
+                                 int ry, const T* taps_x, const T* taps_y, const StripAdjoint<T>& s,
+                                 const ProxArgs<T>& P, unsigned long long* words, cudaStream_t st);
+
 // Step prologue / epilogue kernels (jko_step_kernels.cu).
 template <typename T>
 cudaError_t launch_fill(T* x, T v, long long n, cudaStream_t st);

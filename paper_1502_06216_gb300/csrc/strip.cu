@@ -175,7 +175,7 @@ strip_kernel(const __grid_constant__ StripArgs<T> A, const __grid_constant__ Pro
   };
   // the stop rule (Sec. 3.4) on the sum over the blocks' residuals of pair `of`, put with ep
   auto decide = [&](int of, unsigned ep) {
-    const double v = X.gather_sum(A.g.xres + (size_t)(of & 1) * n_res * 2, n_res, ep);
+    const double v = gather_sum(A.g.xres + (size_t)(of & 1) * n_res * 2, n_res, ep, &s_fault);
     const bool first = lane == 0 && blockIdx.x == 0;
     int d = RUNNING;
     if (!isfinite(v)) d = NONFINITE;

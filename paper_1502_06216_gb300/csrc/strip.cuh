@@ -381,29 +381,29 @@ struct Strips {
     for (int e = threadIdx.x; e < G.nx * nrg; e += blockDim.x)
       dst[e] = g != nullptr ? g[(size_t)y0 * G.nx + e] : T(1);
   }
-
-  // The sum over `blocks` blocks of the doubles they put with epoch ep at xr, in
-  // one order everywhere (one warp; every lane gets it).
-  __device__ __forceinline__ double gather_sum(const unsigned long long* xr, int blocks,
-                                               unsigned ep) {
-    constexpr int UN = 5;   // blocks per lane whose words are in flight at once
-    const int lane = threadIdx.x & 31;
-    double v = 0.0;
-    for (int g0 = lane; g0 < blocks; g0 += 32 * UN) {
-      unsigned long long lo[UN], hi[UN];
-#pragma unroll
-      for (int u = 0; u < UN; ++u)
-        if (g0 + 32 * u < blocks) get_words(xr + 2 * (g0 + 32 * u), lo[u], hi[u]);
-#pragma unroll
-      for (int u = 0; u < UN; ++u)
-        if (g0 + 32 * u < blocks) {
-          if (!wait_pair(xr + 2 * (g0 + 32 * u), ep, lo[u], hi[u], fault)) *fault = 1;
-          v += words_double(lo[u], hi[u]);
-        }
-    }
-    return warp_sum(v);
-  }
 };
+
+// The sum over `blocks` blocks of the doubles they put with epoch ep at xr, in one
+// order everywhere (one warp; every lane gets it).
+__device__ __forceinline__ double gather_sum(const unsigned long long* xr, int blocks, unsigned ep,
+                                             int* fault) {
+  constexpr int UN = 5;   // blocks per lane whose words are in flight at once
+  const int lane = threadIdx.x & 31;
+  double v = 0.0;
+  for (int g0 = lane; g0 < blocks; g0 += 32 * UN) {
+    unsigned long long lo[UN], hi[UN];
+#pragma unroll
+    for (int u = 0; u < UN; ++u)
+      if (g0 + 32 * u < blocks) get_words(xr + 2 * (g0 + 32 * u), lo[u], hi[u]);
+#pragma unroll
+    for (int u = 0; u < UN; ++u)
+      if (g0 + 32 * u < blocks) {
+        if (!wait_pair(xr + 2 * (g0 + 32 * u), ep, lo[u], hi[u], fault)) *fault = 1;
+        v += words_double(lo[u], hi[u]);
+      }
+  }
+  return warp_sum(v);
+}
 
 }  // namespace strip
 

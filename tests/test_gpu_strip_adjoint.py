@@ -1,0 +1,60 @@
+"""The reverse pass on strips (strip_adjoint.cu) against the kernels per pass
+(loop = 2): every energy kind, one line a block, several, ragged last blocks, lines
+of one kind missing from some blocks.
+
+FP64: both solves stop where eight changes sum below 8e-12 of |abar|; the
+contraction of these flows leaves below 1e2 times that, so 1e-8 relative (2-norm)
+over two steps is generous.  FP32: each application of xi carries at most
+~(2r + 2) 2^-24 ~ 1e-5 relative in either order of its filters, again amplified by
+the solve's 1 / (1 - rho) ~ 10: 1e-4."""
+import numpy as np
+import pytest
+
+from paper_1502_06216_gb300 import inputs
+from tests.gpu_util import need_gpu
+
+pytestmark = pytest.mark.gpu
+
+
+def problem(kind, nx, ny):
+    if kind == "crowd":
+        return inputs.crowd_problem(nx, gamma=4e-3, ny=ny)
+    if kind == "porous":
+        pb = inputs.porous_problem(nx, seed=3, gamma=2e-3, ny=ny)
+        pb.w = 0.1 * np.linspace(0, 1, pb.N)
+        return pb
+    return inputs.varying_exponent_problem(nx, seed=3, ny=ny)
+
+
+@pytest.mark.parametrize("prec", ["FP32", "FP64"])
+@pytest.mark.parametrize("kind,nx,ny", [("crowd", 33, 70), ("crowd", 153, 152), ("crowd", 420, 150),
+                                        ("porous", 64, 48), ("porous", 160, 155),
+                                        ("exponents", 90, 61)])
+def test_reverse_pass_on_strips_equals_the_kernels_per_pass(kind, nx, ny, prec):
+    torch = need_gpu()
+    from paper_1502_06216_gb300 import jko
+    pb = problem(kind, nx, ny)
+    tol = 1e-12 if prec == "FP64" else 1e-7
+    grads = []
+    for loop in (2, 0):
+        h = jko.create_from_problem(pb, precision=jko.Precision[prec], loop=loop, tol=tol,
+                                    max_iter=2000)
+        assert jko.jko_handle_info(h)["loop"] == (loop == 0 and not (prec == "FP64" and nx > 304))
+        p0 = torch.tensor(pb.q0, dtype=h.dtype, device="cuda")
+        g = torch.tensor(np.random.default_rng(5).normal(size=pb.N), dtype=h.dtype, device="cuda")
+        want_w = kind != "exponents"
+        jko.jko_flow_record(h, p0, 2)
+        first = jko.jko_flow_backward(h, g, want_w=want_w)
+        again = jko.jko_flow_backward(h, g, want_w=want_w)
+        for a, b in zip(first[:2 if want_w else 1], again):
+            assert loop == 2 or torch.equal(a, b)
+        grads.append([x.double().cpu().numpy() for x in first[:2 if want_w else 1]])
+        jko.jko_destroy(h)
+    sup = pb.q0 > 0          # dL/dp_0 is compared where the flow started with mass
+    for name, a, b in zip(("p0", "w"), *grads):
+        if name == "p0":
+            a, b = a[sup], b[sup]
+        err = np.linalg.norm(b - a) / np.linalg.norm(a)
+        print(kind, nx, ny, prec, name, err)
+        assert np.isfinite(b).all()
+        assert err <= (1e-8 if prec == "FP64" else 1e-4)
