@@ -13,12 +13,22 @@
 // around only into the zero padding.  The circulant's first column c is
 // symmetric (c[d] = c[L - d] = k(d), d <= r), so its spectrum
 // K^[f] = sum_d c[d] e^{-2 pi i f d / L} is real; two real lines x, y packed as
-// x + i y give k * x + i (k * y) in one transform.  Per block: 8 columns of
-// the input as 4 complex lines in shared memory, a forward radix-2 transform
-// (decimation in time from a bit-reversed load), the product with K^ (which
-// carries 1/L), an inverse radix-2 transform (decimation in frequency with
-// conjugate twiddles, its output in bit-reversed order), then the epilogue as
-// in filter_pass.  Spectrum and twiddles are computed in FP64 on the host.
+// x + i y give k * x + i (k * y) in one transform.  Per block: FJ = 2 or 4
+// columns of the input as one or two complex lines in shared memory.  The
+// forward transform is decimation in frequency in place (natural order in,
+// bit-reversed out), two radix-2 levels at a time in registers; its innermost
+// levels, the product with K^ (which carries 1/L, read at the bit-reversed
+// index) and the first levels of the inverse, decimation in time from the
+// bit-reversed order, are one pass over the line, so no reordering is ever done.
+// The outermost levels read the image directly; where the line fills at most
+// half of L the zero half is left out.  Then the epilogue as in filter_pass.
+// Spectrum and twiddles are computed in FP64 on the host.
+//
+// FP64 is bound by its pipe (2 multiply-adds a cycle and SM): 28 instructions for
+// four points and two levels, so lines are spread over all SMs (512^2: 128 blocks of
+// two lines where 64 blocks of four left 88 SMs idle) and shared memory is
+// touched once per two levels.  512^2, L = 1024, FP64: a store pass 108 -> 42 us, with
+// the b-update 134 -> 56 us; its multiply-adds alone would take 32 us on all SMs.
 //
 // Rounding: the transforms are accurate normwise: each output carries an
 // error of about eps log2(L) times the largest entry of its input line,
@@ -33,9 +43,11 @@ namespace jko {
 
 namespace {
 
-constexpr int FNT = 256;   // threads per block
-constexpr int FJ = 8;      // input columns per block (4 complex lines)
-constexpr int FNL = FJ / 2;
+constexpr int FNT = 512;   // threads per block at most
+
+// Input columns per block: four (a 32-byte sector of FP64 per row), or two where four
+// would leave SMs without a block.
+__host__ __device__ constexpr int fft_cols(int n_j) { return n_j > 4 * 100 ? 4 : 2; }
 
 template <typename T> struct C2;
 template <> struct C2<float> { using t = float2; };
@@ -56,106 +68,189 @@ __device__ __forceinline__ V cmul_conj(V a, V b) {   // a * conj(b)
   return r;
 }
 
-template <typename T, int EPI, int EK>
+// Element i of a line sits at fpad(i): one element skipped per 128 bytes, so that the
+// strided accesses of the inner levels spread over the banks.
+template <typename T>
+__host__ __device__ __forceinline__ int fpad(int i) { return i + (i >> (sizeof(T) == 8 ? 3 : 4)); }
+
+// Two radix-2 levels on (x0, x1, x2, x3) = points k, k + h, k + 2h, k + 3h of a group
+// of m = 4h: forward (decimation in frequency) with w_j = e^{-2 pi i j k / m}, and its
+// mirror (decimation in time, conjugate twiddles, unnormalised).
+template <typename V>
+__device__ __forceinline__ void dif4(V& x0, V& x1, V& x2, V& x3, V w1, V w2, V w3) {
+  const V s0{x0.x + x2.x, x0.y + x2.y}, s1{x1.x + x3.x, x1.y + x3.y};
+  const V d0{x0.x - x2.x, x0.y - x2.y}, d1{x1.y - x3.y, x3.x - x1.x};   // d1 = -i (x1 - x3)
+  x0 = V{s0.x + s1.x, s0.y + s1.y};
+  x1 = cmul(V{s0.x - s1.x, s0.y - s1.y}, w2);
+  x2 = cmul(V{d0.x + d1.x, d0.y + d1.y}, w1);
+  x3 = cmul(V{d0.x - d1.x, d0.y - d1.y}, w3);
+}
+// ... where x2 = x3 = 0
+template <typename V>
+__device__ __forceinline__ void dif4_half(V& x0, V& x1, V& x2, V& x3, V w1, V w2, V w3) {
+  const V d1{x1.y, -x1.x};
+  x2 = cmul(V{x0.x + d1.x, x0.y + d1.y}, w1);
+  x3 = cmul(V{x0.x - d1.x, x0.y - d1.y}, w3);
+  const V s{x0.x - x1.x, x0.y - x1.y};
+  x0 = V{x0.x + x1.x, x0.y + x1.y};
+  x1 = cmul(s, w2);
+}
+template <typename V>
+__device__ __forceinline__ void dit4(V& y0, V& y1, V& y2, V& y3, V w1, V w2, V w3) {
+  const V b1 = cmul_conj(y1, w2), b2 = cmul_conj(y2, w1), b3 = cmul_conj(y3, w3);
+  const V s0{y0.x + b1.x, y0.y + b1.y}, s1{y0.x - b1.x, y0.y - b1.y};
+  const V d0{b2.x + b3.x, b2.y + b3.y}, d1{b3.y - b2.y, b2.x - b3.x};   // d1 = i (b2 - b3)
+  y0 = V{s0.x + d0.x, s0.y + d0.y};
+  y1 = V{s1.x + d1.x, s1.y + d1.y};
+  y2 = V{s0.x - d0.x, s0.y - d0.y};
+  y3 = V{s1.x - d1.x, s1.y - d1.y};
+}
+
+template <typename T, int EPI, int EK, int FJ>
 __global__ void __launch_bounds__(FNT)
 fft_pass_kernel(PassArgs<T> A, ProxArgs<T> P, FftArgs<T> F) {
   using V = typename C2<T>::t;
+  constexpr int FNL = FJ / 2;   // complex lines
   Ctrl* ctrl = A.ctrl;
   __shared__ int s_it;
   if (stop_gate(ctrl, A.part, A.nparts, A.decide != 0, &s_it)) return;
 
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  const int L = F.L, lg = F.log2L, half = L >> 1;
-  V* s_z = reinterpret_cast<V*>(smem_raw);          // FNL lines of L
-  V* s_w = s_z + (size_t)FNL * L;                     // twiddles e^{-2 pi i j / L}, j < L/2
+  const int L = F.L, lg = F.log2L, LP = fpad<T>(L) + 1;
+  V* s_z = reinterpret_cast<V*>(smem_raw);          // FNL padded lines of L
+  V* s_w = s_z + (size_t)FNL * LP;                    // twiddles e^{-2 pi i j / L}, j < 3 L / 4
   __shared__ double s_red[33];
-  const int tid = threadIdx.x;
-  for (int j = tid; j < half; j += FNT) s_w[j] = reinterpret_cast<const V*>(F.tw)[j];
-
-  // load columns j0 .. j0+7 (zero beyond n_j and beyond row n_i) into the 4
-  // lines at bit-reversed positions; columns 2m / 2m+1 are the real / imaginary
-  // parts of line m
+  const int tid = threadIdx.x, nt = blockDim.x;
+  for (int j = tid; j < (3 * L) / 4; j += nt) s_w[j] = reinterpret_cast<const V*>(F.tw)[j];
   const int j0 = blockIdx.x * FJ;
-  for (int e = tid; e < FJ * L; e += FNT) {
-    const int c = e % FJ, i = e / FJ;
-    const int jj = j0 + c;
-    const T v = (i < A.n_i && jj < A.n_j) ? __ldg(A.in + (size_t)i * A.n_j + jj) : T(0);
-    const int pos = (int)(__brev((unsigned)i) >> (32 - lg));
-    T* dst = reinterpret_cast<T*>(s_z + (size_t)(c >> 1) * L + pos) + (c & 1);
-    *dst = v;
+  auto at = [&](int line, int i) -> V& { return s_z[line * LP + fpad<T>(i)]; };
+  // row i of columns j0 + 2 line, + 1 (zero outside the image)
+  auto load = [&](int line, int i) -> V {
+    const int jj = j0 + 2 * line;
+    V v{T(0), T(0)};
+    if (i < A.n_i && jj < A.n_j) {
+      const T* g = A.in + (size_t)i * A.n_j + jj;
+      v.x = __ldg(g);
+      if (jj + 1 < A.n_j) v.y = __ldg(g + 1);
+    }
+    return v;
+  };
+  __syncthreads();   // the twiddles
+  const int quads = L >> 2;
+  const int mid = (lg & 1) ? 2 : 4;   // size of the innermost levels
+  // forward, outermost levels: straight from the image
+  if (L > mid) {
+    const int h = quads;
+    for (int b = tid; b < FNL * quads; b += nt) {
+      const int line = b % FNL, k = b / FNL;
+      V x0 = load(line, k), x1 = load(line, k + h), x2, x3;
+      if (2 * A.n_i <= L) {
+        dif4_half(x0, x1, x2, x3, s_w[k], s_w[2 * k], s_w[3 * k]);
+      } else {
+        x2 = load(line, k + 2 * h);
+        x3 = load(line, k + 3 * h);
+        dif4(x0, x1, x2, x3, s_w[k], s_w[2 * k], s_w[3 * k]);
+      }
+      at(line, k) = x0;
+      at(line, k + h) = x1;
+      at(line, k + 2 * h) = x2;
+      at(line, k + 3 * h) = x3;
+    }
+  } else {
+    for (int b = tid; b < FNL * L; b += nt) at(b % FNL, b / FNL) = load(b % FNL, b / FNL);
   }
   __syncthreads();
-
-  // forward transform: decimation in time, natural-order output
-  for (int s = 1; s <= lg; ++s) {
-    const int m = 1 << s, hm = m >> 1, tstep = L >> s;
-    for (int b = tid; b < FNL * half; b += FNT) {
-      const int line = b / half, bb = b - line * half;
-      const int grp = bb / hm, k = bb - grp * hm;
-      V* z = s_z + (size_t)line * L;
-      const int i1 = grp * m + k, i2 = i1 + hm;
-      const V t = cmul(s_w[k * tstep], z[i2]);
-      const V u = z[i1];
-      z[i1] = V{u.x + t.x, u.y + t.y};
-      z[i2] = V{u.x - t.x, u.y - t.y};
+  for (int lm = lg - 2; lm > 2; lm -= 2) {
+    const int h = 1 << (lm - 2), ts = lg - lm;
+    for (int b = tid; b < FNL * quads; b += nt) {
+      const int line = b / quads, bb = b - line * quads;
+      const int k = bb & (h - 1), i = ((bb >> (lm - 2)) << lm) + k, w = k << ts;
+      V &z0 = at(line, i), &z1 = at(line, i + h), &z2 = at(line, i + 2 * h),
+        &z3 = at(line, i + 3 * h);
+      V x0 = z0, x1 = z1, x2 = z2, x3 = z3;
+      dif4(x0, x1, x2, x3, s_w[w], s_w[2 * w], s_w[3 * w]);
+      z0 = x0;
+      z1 = x1;
+      z2 = x2;
+      z3 = x3;
     }
     __syncthreads();
   }
-  // times the real spectrum (with 1/L)
-  for (int e = tid; e < FNL * L; e += FNT) {
-    const T kh = F.khat[e % L];
-    V z = s_z[e];
-    z.x *= kh;
-    z.y *= kh;
-    s_z[e] = z;
+  // innermost levels (their twiddles are 1), the real spectrum (with 1/L), and back:
+  // position i holds frequency brev(i)
+  for (int b = tid; b < FNL * (L / mid); b += nt) {
+    const int line = b / (L / mid), i = (b - line * (L / mid)) * mid;
+    auto kh = [&](int e) { return __ldg(F.khat + (__brev((unsigned)(i + e)) >> (32 - lg))); };
+    V &z0 = at(line, i), &z1 = at(line, i + 1);
+    if (mid == 2) {
+      const T k0 = kh(0), k1 = kh(1);
+      const V u{(z0.x + z1.x) * k0, (z0.y + z1.y) * k0};
+      const V v{(z0.x - z1.x) * k1, (z0.y - z1.y) * k1};
+      z0 = V{u.x + v.x, u.y + v.y};
+      z1 = V{u.x - v.x, u.y - v.y};
+    } else {
+      V &z2 = at(line, i + 2), &z3 = at(line, i + 3);
+      const T k0 = kh(0), k1 = kh(1), k2 = kh(2), k3 = kh(3);
+      const V s0{z0.x + z2.x, z0.y + z2.y}, s1{z1.x + z3.x, z1.y + z3.y};
+      const V d0{z0.x - z2.x, z0.y - z2.y}, d1{z1.y - z3.y, z3.x - z1.x};
+      const V y0{(s0.x + s1.x) * k0, (s0.y + s1.y) * k0}, y1{(s0.x - s1.x) * k1, (s0.y - s1.y) * k1};
+      const V y2{(d0.x + d1.x) * k2, (d0.y + d1.y) * k2}, y3{(d0.x - d1.x) * k3, (d0.y - d1.y) * k3};
+      const V t0{y0.x + y1.x, y0.y + y1.y}, t1{y0.x - y1.x, y0.y - y1.y};
+      const V e0{y2.x + y3.x, y2.y + y3.y}, e1{y3.y - y2.y, y2.x - y3.x};
+      z0 = V{t0.x + e0.x, t0.y + e0.y};
+      z1 = V{t1.x + e1.x, t1.y + e1.y};
+      z2 = V{t0.x - e0.x, t0.y - e0.y};
+      z3 = V{t1.x - e1.x, t1.y - e1.y};
+    }
   }
   __syncthreads();
-  // inverse transform: decimation in frequency with conjugate twiddles,
-  // bit-reversed output
-  for (int s = lg; s >= 1; --s) {
-    const int m = 1 << s, hm = m >> 1, tstep = L >> s;
-    for (int b = tid; b < FNL * half; b += FNT) {
-      const int line = b / half, bb = b - line * half;
-      const int grp = bb / hm, k = bb - grp * hm;
-      V* z = s_z + (size_t)line * L;
-      const int i1 = grp * m + k, i2 = i1 + hm;
-      const V u = z[i1], v = z[i2];
-      z[i1] = V{u.x + v.x, u.y + v.y};
-      z[i2] = cmul_conj(V{u.x - v.x, u.y - v.y}, s_w[k * tstep]);
+  // inverse: the same levels outwards, natural-order output
+  for (int lm = 4 - (lg & 1); lm <= lg; lm += 2) {
+    const int h = 1 << (lm - 2), ts = lg - lm;
+    const bool half = lm == lg && 2 * A.n_i <= L;   // the upper half is not needed
+    for (int b = tid; b < FNL * quads; b += nt) {
+      const int line = b / quads, bb = b - line * quads;
+      const int k = bb & (h - 1), i = ((bb >> (lm - 2)) << lm) + k, w = k << ts;
+      V &z0 = at(line, i), &z1 = at(line, i + h);
+      V x0 = z0, x1 = z1, x2 = at(line, i + 2 * h), x3 = at(line, i + 3 * h);
+      dit4(x0, x1, x2, x3, s_w[w], s_w[2 * w], s_w[3 * w]);
+      z0 = x0;
+      z1 = x1;
+      if (!half) {
+        at(line, i + 2 * h) = x2;
+        at(line, i + 3 * h) = x3;
+      }
     }
     __syncthreads();
   }
 
-  // ---- epilogue: warp w owns output column j0 + w (out row), 32 outputs at a time ----
-  const int warp = tid >> 5, lane = tid & 31;
-  const int j = j0 + warp;
+  // ---- epilogue: FJ output rows (columns j0 + c), along each row ----
+  const int lane = tid & 31;
   T res_t = T(0);
   int bad = 0;
-  if (j < A.n_j) {
-    const size_t rowoff = (size_t)j * A.n_i;
-    const T* zl = reinterpret_cast<const T*>(s_z + (size_t)(warp >> 1) * L) + (warp & 1);
-    const bool have_prev = EPI == EPI_B && s_it > 0;
-    for (int i = lane; i < A.n_i; i += 32) {
-      const int pos = (int)(__brev((unsigned)i) >> (32 - lg));
-      const T acc = zl[2 * (size_t)pos];
-      const size_t idx = rowoff + i;
-      if (EPI == EPI_STORE) {
-        A.out[idx] = acc;
-      } else if (EPI == EPI_B) {
-        const T qv = A.q[idx];
-        if (have_prev) res_t += abs_residual<T>(A.out[idx], acc, qv);
-        const T bn = b_update<T>(qv, acc);
-        bad |= !dev_finite(bn);
-        A.out[idx] = bn;
-      } else {
-        // xi b >= 0 for b >= 0: an output below 0 is the transform's rounding
-        // (of the line's largest entry) and is taken as 0, so that p >= 0
-        const T sv = acc < T(0) ? T(0) : acc;
-        const T a = prox_ratio<T, EK>(P, (int)idx, sv);
-        bad |= !dev_finite(a);
-        A.out[idx] = a;
-        A.p[idx] = a * sv;
-      }
+  const bool have_prev = EPI == EPI_B && s_it > 0;
+  const int cols = min(FJ, A.n_j - j0);
+  for (int e = tid; e < cols * A.n_i; e += nt) {
+    const int c = e / A.n_i, i = e - c * A.n_i;
+    const V z = at(c >> 1, i);
+    const T acc = (c & 1) ? z.y : z.x;
+    const size_t idx = (size_t)(j0 + c) * A.n_i + i;
+    if (EPI == EPI_STORE) {
+      A.out[idx] = acc;
+    } else if (EPI == EPI_B) {
+      const T qv = A.q[idx];
+      if (have_prev) res_t += abs_residual<T>(A.out[idx], acc, qv);
+      const T bn = b_update<T>(qv, acc);
+      bad |= !dev_finite(bn);
+      A.out[idx] = bn;
+    } else {
+      // xi b >= 0 for b >= 0: an output below 0 is the transform's rounding
+      // (of the line's largest entry) and is taken as 0, so that p >= 0
+      const T sv = acc < T(0) ? T(0) : acc;
+      const T a = prox_ratio<T, EK>(P, (int)idx, sv);
+      bad |= !dev_finite(a);
+      A.out[idx] = a;
+      A.p[idx] = a * sv;
     }
   }
   if (EPI == EPI_STORE) return;
@@ -169,24 +264,33 @@ fft_pass_kernel(PassArgs<T> A, ProxArgs<T> P, FftArgs<T> F) {
 }
 
 template <typename T>
-size_t fft_smem(int L) {
-  return sizeof(typename C2<T>::t) * ((size_t)FNL * L + (size_t)(L / 2));
+size_t fft_smem(int L, int fj) {
+  return sizeof(typename C2<T>::t) * ((size_t)(fj / 2) * (fpad<T>(L) + 1) + (size_t)(3 * L) / 4);
 }
 
+template <typename T, int EPI, int EK, int FJ>
+cudaError_t launch_fft_fj(const PassArgs<T>& A, const ProxArgs<T>& P, const FftArgs<T>& F,
+                          cudaStream_t st) {
+  const size_t smem = fft_smem<T>(F.L, FJ);
+  auto kern = fft_pass_kernel<T, EPI, EK, FJ>;
+  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  if (e != cudaSuccess) return e;
+  // one thread per four points and line, 64 to 512
+  int threads = FJ / 2 * F.L / 4;
+  threads = threads < 64 ? 64 : threads > FNT ? FNT : threads;
+  kern<<<fft_pass_blocks(A.n_j), threads, smem, st>>>(A, P, F);
+  return cudaGetLastError();
+}
 template <typename T, int EPI, int EK>
 cudaError_t launch_fft(const PassArgs<T>& A, const ProxArgs<T>& P, const FftArgs<T>& F,
                        cudaStream_t st) {
-  const size_t smem = fft_smem<T>(F.L);
-  auto kern = fft_pass_kernel<T, EPI, EK>;
-  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  if (e != cudaSuccess) return e;
-  kern<<<fft_pass_blocks(A.n_j), FNT, smem, st>>>(A, P, F);
-  return cudaGetLastError();
+  return fft_cols(A.n_j) == 4 ? launch_fft_fj<T, EPI, EK, 4>(A, P, F, st)
+                              : launch_fft_fj<T, EPI, EK, 2>(A, P, F, st);
 }
 
 }  // namespace
 
-int fft_pass_blocks(int n_j) { return (n_j + FJ - 1) / FJ; }
+int fft_pass_blocks(int n_j) { return (n_j + fft_cols(n_j) - 1) / fft_cols(n_j); }
 
 // Transform length and tables of one axis of n cells with band radius r.
 bool fft_axis_tables(int n, int r, double length, double gamma, int max_len, int* L, int* log2L,
@@ -212,16 +316,13 @@ bool fft_axis_tables(int n, int r, double length, double gamma, int max_len, int
     }
     (*khat)[f] = s / Ln;
   }
-  tw->assign(Ln, 0.0);   // interleaved re, im of e^{-2 pi i j / L}, j < L/2
-  for (int j = 0; j < Ln / 2; ++j) {
+  tw->assign(2 * Ln, 0.0);   // interleaved re, im of e^{-2 pi i j / L}, j < L
+  for (int j = 0; j < Ln; ++j) {
     (*tw)[2 * j] = std::cos(2.0 * pi * j / Ln);
     (*tw)[2 * j + 1] = -std::sin(2.0 * pi * j / Ln);
   }
   return true;
 }
-
-template <typename T>
-size_t fft_pass_smem(int L) { return fft_smem<T>(L); }
 
 template <typename T>
 cudaError_t fft_pass(int epi, int ek, const PassArgs<T>& A, const ProxArgs<T>& P,
@@ -239,7 +340,5 @@ template cudaError_t fft_pass<float>(int, int, const PassArgs<float>&, const Pro
                                      const FftArgs<float>&, cudaStream_t);
 template cudaError_t fft_pass<double>(int, int, const PassArgs<double>&, const ProxArgs<double>&,
                                       const FftArgs<double>&, cudaStream_t);
-template size_t fft_pass_smem<float>(int);
-template size_t fft_pass_smem<double>(int);
 
 }  // namespace jko

@@ -2173,7 +2173,7 @@ jko_status jko_batch_create(int n_flows, const jko_grid* grids, const jko_params
     // and a heat-kernel flow runs its kernels per Clenshaw phase (its persistent
     // form is one cooperative launch over every SM)
     h->simt_latency = 0;
-    h->nparts_simt = jko::simt_pass_blocks(grids[f].nx, grids[f].ny, 0);
+    if (!h->fft) h->nparts_simt = jko::simt_pass_blocks(grids[f].nx, grids[f].ny, 0);
     if (h->heat_L) h->use_loop = 0;
     b->h.push_back(h);
     b->max_iter = std::max(b->max_iter, params[f].max_iter);

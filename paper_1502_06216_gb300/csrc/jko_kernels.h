@@ -41,14 +41,14 @@ struct PassArgs {
 // FFT form of the pass (fft_filter.cu): the same out[j][i'] and epilogues by
 // convolution through a transform of length L (a power of two >= n_i + r).
 // khat: the real spectrum of the circulant embedding of the taps, with 1/L
-// (L entries); tw: e^{-2 pi i j / L}, j < L/2, interleaved re, im.
+// (L entries); tw: e^{-2 pi i j / L}, j < L, interleaved re, im.
 template <typename T>
 struct FftArgs {
   int L = 0, log2L = 0;
   const T* khat = nullptr;
   const T* tw = nullptr;
 };
-// Longest transform per element type (the block's 4 lines and twiddles in
+// Longest transform per element type (a block's lines and twiddles in
 // shared memory).
 template <typename T> constexpr int fft_max_length() { return sizeof(T) == 4 ? 4096 : 2048; }
 template <typename T>
