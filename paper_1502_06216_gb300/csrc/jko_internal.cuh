@@ -236,6 +236,42 @@ template <> struct NewtonEps<double> { static constexpr double v = 1e-15; };
 //    is Eq. prox-entropy, y = l/(1 + c).  From y0 = l/(1 + c), where
 //    g(y0) = c ((e^{m1 y0} - 1)/m1 - y0) >= 0, Newton again decreases
 //    monotonically (g increasing and convex); expm1 keeps small m1 exact.
+//  * FP64: the same iteration in FP32 first (its pipe is 64 times as wide and an FP64
+//    e^y costs ~25 instructions: the FP64 loop from y0 = l ran 5 to 8 of them a cell), then
+//    Newton in FP64 from there, two steps as a rule.  One step from below the root lands above it (g convex), and the
+//    error after a step dy is at most m1/2 dy^2 (g'' <= m1 g'), so the loop ends
+//    where that is below the rounding of y: the root is the same to rounding.
+template <typename T, bool CELL>
+__device__ __forceinline__ T newton_start(T l, T, T, int) { return l; }
+template <>
+__device__ __forceinline__ double newton_start<double, false>(double l, double c, double m1, int n) {
+  const float lf = (float)l, cf = (float)c, mf = (float)m1;
+  float y = lf;
+  for (int it = 0; it < n; ++it) {
+    const float e = cf * expf(mf * y);
+    const float dy = (y + e - lf) / (1.0f + mf * e);
+    y -= dy;
+    if (!(dy > 1e-6f * (1.0f + fabsf(y)))) break;
+  }
+  return isfinite(y) ? (double)y : l;
+}
+template <>
+__device__ __forceinline__ double newton_start<double, true>(double l, double c, double m1, int n) {
+  const float lf = (float)l, cf = (float)c, mf = (float)m1;
+  float y = lf / (1.0f + cf);
+  for (int it = 0; it < n; ++it) {
+    const float dy = (y + cf * expm1f(mf * y) / mf - lf) / (1.0f + cf * expf(mf * y));
+    y -= dy;
+    if (!(dy > 1e-6f * (1.0f + fabsf(y)))) break;
+  }
+  return isfinite(y) ? (double)y : l / (1.0 + c);
+}
+__device__ __forceinline__ bool newton_done(float dy, float y, float) {
+  return !(dy > NewtonEps<float>::v * (1.0f + fabsf(y)));
+}
+__device__ __forceinline__ bool newton_done(double dy, double y, double m1) {
+  return !(m1 * dy * dy > 1e-16 * (1.0 + fabs(y)));
+}
 template <typename T>
 __device__ __forceinline__ T power_log_psi(const ProxArgs<T>& P, int idx, T l, T& k) {
   const T c = P.c[idx];
@@ -243,11 +279,12 @@ __device__ __forceinline__ T power_log_psi(const ProxArgs<T>& P, int idx, T l, T
     const T m1 = P.m1f[idx];
     T y = l / (T(1) + c);
     if (m1 > T(0)) {
+      if (sizeof(T) == 8) y = newton_start<T, true>(l, c, m1, P.newton);
       for (int it = 0; it < P.newton; ++it) {
         const T g = y + c * dev_expm1<T>(m1 * y) / m1 - l;
         const T dy = g / (T(1) + c * dev_exp<T>(m1 * y));
         y -= dy;
-        if (!(dy > NewtonEps<T>::v * (T(1) + fabs(y)))) break;
+        if (newton_done(dy, y, m1)) break;
       }
       k = c * dev_exp<T>(m1 * y);
     } else {
@@ -255,12 +292,12 @@ __device__ __forceinline__ T power_log_psi(const ProxArgs<T>& P, int idx, T l, T
     }
     return y;
   }
-  T y = l;
+  T y = newton_start<T, false>(l, c, P.m1, P.newton);
   for (int it = 0; it < P.newton; ++it) {
     const T e = c * dev_exp<T>(P.m1 * y);
     const T dy = (y + e - l) / (T(1) + P.m1 * e);
     y -= dy;
-    if (!(dy > NewtonEps<T>::v * (T(1) + fabs(y)))) break;
+    if (newton_done(dy, y, P.m1)) break;
   }
   k = P.m1 * c * dev_exp<T>(P.m1 * y);
   return y;
