@@ -20,7 +20,7 @@
 #include <cmath>
 #include <vector>
 
-#include "jko_internal.cuh"
+#include "heat_cell.cuh"
 #include "jko_kernels.h"
 
 namespace jko {
@@ -39,45 +39,6 @@ struct HeatGeom {
 
 __device__ __forceinline__ bool is_free(const HeatGeom& g, int i) {
   return g.mask == nullptr || g.mask[i] == 0;
-}
-
-// ---- the per-cell arithmetic of the recurrence ----
-// Written with explicit roundings, so that every kernel below (per phase or
-// persistent) performs the same operations whatever the compiler contracts.
-// The iterates W are FP64 for both precisions: a high-degree recurrence
-// cancels large intermediate terms in the far field, where the kernel's tail
-// is many orders below its peak, so single precision there costs digits (the
-// flows' error grew 16-fold with FP32 iterates).  Double-float iterates (two
-// floats, ~48 significant bits, on the FP32 pipe) were measured slower than
-// FP64 on GB300 (100^2: 4.8k against 5.3k pairs/s): the stencil is bound by
-// the latency of its dependent chains, which double-float arithmetic
-// lengthens, not by the FP64 pipe's throughput.
-template <typename T> struct HeatIter { using W = double; };
-
-// constants and inputs as iterates
-template <typename W> __device__ __forceinline__ W wc(double d) { return d; }
-__device__ __forceinline__ double wv(double v) { return v; }
-template <typename W> __device__ __forceinline__ W wzero() { return 0.0; }
-// c v (the first iterate b_D = c_D v)
-__device__ __forceinline__ double wscale(double c, double v) { return __dmul_rn(c, v); }
-
-// acc + c (vi - vj): one neighbour's term of A v
-__device__ __forceinline__ double nb_term(double acc, double c, double vi, double vj) {
-  return __fma_rn(c, __dsub_rn(vi, vj), acc);
-}
-// one Clenshaw step's value ck v + s (A b1 - theta b1) - b2
-__device__ __forceinline__ double cl_value(double ck, double v, double s, double Ab, double theta,
-                                          double b1, double b2) {
-  return __dsub_rn(__fma_rn(ck, v, __dmul_rn(s, __fma_rn(-theta, b1, Ab))), b2);
-}
-
-// The operator's output is clamped at 0: xi~ is positive, and the expansion's
-// error is normwise (~1e-15 of the largest entry), so where the true kernel
-// tail lies below it the sum can come out slightly negative; 0 there is the
-// same underflow the Gaussian kernel meets far from its support (the b-update
-// and the prox treat it so).  NaN passes through.
-template <typename T> __device__ __forceinline__ T close_out(double r) {
-  return (T)(r < 0.0 ? 0.0 : r);
 }
 
 // (A v)_i = v_i + sum over free neighbours j of c_dir (v_i - v_j)

@@ -1,0 +1,407 @@
+// heat_tile.cu -- the persistent form of a step with the heat kernel (heat.cu) on
+// resident tiles: one block per tile of the grid keeps v, the Clenshaw iterates
+// b_{k+1}, b_{k+2} and the step's images in shared memory for the whole step, with
+// a halo of H cells.  A phase runs up to H Clenshaw steps, each on the tile and a
+// halo one cell narrower than the one before (recomputed by the neighbours), then
+// the tiles exchange the H cells inside their edges: every value travels as 8-byte
+// words {32 bits, epoch} (strip.cuh), polled by their readers, so there is no grid
+// barrier, and the interior never leaves the SM.  The words are twice buffered by
+// epoch parity: a block writes exchange e + 2 only after it has every
+// neighbour's e + 1, which they wrote after reading e ("neighbour" is symmetric:
+// within H cells).  The arithmetic of a cell and the stop rule are those of heat.cu's
+// kernels, so the iterates have the same bits; the residual is added by tiles.
+//
+// Bound by the FP64 latency of its steps and the exchange between them: at 100^2 (150
+// tiles, degree 54) 0.9 us a step and 1.1 us an exchange; 33 pairs take 5.69 ms on
+// heat.cu's blocks with a grid barrier a phase, 4.36 here with H = 4 (7.0, 5.1, 4.5, 4.4
+// and 4.6 with H = 1, 2, 3, 5 and 6: halo work against exchanges).
+#include <algorithm>
+
+#include "heat_cell.cuh"
+#include "jko_kernels.h"
+#include "strip.cuh"
+
+namespace jko {
+
+namespace {
+
+using namespace strip;
+
+constexpr int HTT = 512;   // threads at most: work warps and one that takes the decision
+
+template <typename T>
+struct HeatTileArgs {
+  int nx, ny, tw, th, ntx, nb, H, D;
+  double cx, cy, two_over_delta, inv_delta, theta;
+  const double* coef;
+  const uint8_t* mask;
+  const T* q;
+  T* a;
+  T* p;
+  Ctrl* ctrl;
+  unsigned long long* xb;    // iterates: [2][cells][4]
+  unsigned long long* xv;    // v: [2][cells][2]
+  unsigned long long* xres;  // residuals: [2][nb][2]
+  unsigned* epoch;
+  int pairs;
+};
+
+__host__ __device__ inline size_t heat_tile_bytes(int tw, int th, int H, size_t es) {
+  const size_t box = (size_t)(tw + 2 * H) * (th + 2 * H);
+  return box * 25 + (size_t)tw * th * es * 4;
+}
+
+// quotient of small non-negative integers (exact below 2^20)
+__device__ __forceinline__ int quot(int i, float inv) { return (int)(((float)i + 0.5f) * inv); }
+
+template <typename T, int EK>
+__global__ void __launch_bounds__(HTT)
+heat_tile_kernel(const __grid_constant__ HeatTileArgs<T> A, const __grid_constant__ ProxArgs<T> P) {
+  extern __shared__ __align__(16) unsigned char smem[];
+  __shared__ int s_bad, s_fault, s_dec;
+  __shared__ double s_wres[HTT / 32];
+  const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+  const int nwork = blockDim.x - 32, nww = nwork >> 5;   // the last warp decides
+  const bool work = tid < nwork;
+  Ctrl* ctrl = A.ctrl;
+  const int done0 = *(volatile int*)&ctrl->done, bad0 = *(volatile int*)&ctrl->nonfinite;
+  if (done0 != RUNNING || bad0) {   // the same state for every block: none waits for this one
+    if (done0 == RUNNING && tid == 0 && blockIdx.x == 0) ctrl->done = NONFINITE;
+    return;
+  }
+  const int maxit = ctrl->max_iter, stall = ctrl->stall;
+  const double tol = ctrl->tol;
+  unsigned ep = *(volatile unsigned*)A.epoch;
+  const int nx = A.nx, ny = A.ny, H = A.H;
+  const size_t N = (size_t)nx * ny;
+  const int by = blockIdx.x / A.ntx, bx = blockIdx.x - by * A.ntx;
+  const int x0 = bx * A.tw, y0 = by * A.th;
+  const int w = min(A.tw, nx - x0), h = min(A.th, ny - y0);
+  const int SX = A.tw + 2 * H, box = SX * (A.th + 2 * H);
+  double* sv = (double*)smem;
+  double* cur1 = sv + box;
+  double* cur2 = cur1 + box;
+  T* s_b = (T*)(cur2 + box);
+  T* s_q = s_b + A.tw * A.th;
+  T* s_p = s_q + A.tw * A.th;
+  T* s_a = s_p + A.tw * A.th;
+  uint8_t* s_nb = (uint8_t*)(s_a + A.tw * A.th);
+  if (tid == 0) {
+    s_bad = 0;
+    s_fault = 0;
+    s_dec = 0;
+  }
+  // free flags of a cell and its four neighbours; v = a = 1 (Sec. 3.4)
+  auto is_free = [&](int x, int y) {
+    return x >= 0 && x < nx && y >= 0 && y < ny &&
+           (A.mask == nullptr || A.mask[(size_t)y * nx + x] == 0);
+  };
+  for (int c = tid; c < box; c += blockDim.x) {
+    const int ey = c / SX, ex = c - ey * SX, x = x0 + ex - H, y = y0 + ey - H;
+    const bool f = is_free(x, y);
+    s_nb[c] = !f ? 0 : 1 | is_free(x - 1, y) << 1 | is_free(x + 1, y) << 2 | is_free(x, y - 1) << 3 |
+                           is_free(x, y + 1) << 4;
+    sv[c] = f ? 1.0 : 0.0;
+    cur1[c] = cur2[c] = 0.0;
+  }
+  for (int c = tid; c < w * h; c += blockDim.x) {
+    const int y = c / w, x = c - y * w;
+    s_q[c] = A.q[(size_t)(y0 + y) * nx + x0 + x];
+    s_a[c] = T(1);
+    s_b[c] = s_p[c] = T(0);
+  }
+  __syncthreads();
+  const int BX = w + 2 * H, ring_tb = 2 * H * BX, ring = ring_tb + 2 * H * h;
+  const float inv_bx = 1.0f / (float)BX, inv_2h = 1.0f / (float)(2 * H);
+  // cell i of the halo ring: its place in the box and in the grid, -1 where nothing is free
+  auto ring_cell = [&](int i, int& c) -> int {
+    int ex, ey;
+    if (i < ring_tb) {
+      const int r = quot(i, inv_bx);
+      ex = i - r * BX;
+      ey = r < H ? r : h + r;
+    } else {
+      i -= ring_tb;
+      const int r = quot(i, inv_2h), col = i - r * 2 * H;
+      ex = col < H ? col : w + col;
+      ey = H + r;
+    }
+    c = ey * SX + ex;
+    return (s_nb[c] & 1) ? (y0 + ey - H) * nx + x0 + ex - H : -1;
+  };
+  auto edge = [&](int x, int y) { return x < H || x >= w - H || y < H || y >= h - H; };
+
+  int it = 0, pair = 0, since = 0;
+  double best = INFINITY;
+  bool run = true;
+  for (; pair < A.pairs && run; ++pair) {
+    for (int app = 0; app < 2; ++app) {
+      // v on the halo; meanwhile the last warp takes the stop decision (Sec. 3.4) on the
+      // b-update's residuals
+      ++ep;
+      if (work) {
+        unsigned long long* xv = A.xv + (size_t)(ep & 1) * N * 2;
+        const float inv_w = 1.0f / (float)w;
+        for (int i = tid; i < w * h; i += nwork) {
+          const int y = quot(i, inv_w), x = i - y * w, c = (y + H) * SX + x + H;
+          if (edge(x, y) && (s_nb[c] & 1))
+            put_elem(xv + 2 * ((size_t)(y0 + y) * nx + x0 + x), sv[c], ep);
+        }
+        for (int i = tid; i < ring; i += nwork) {
+          int c;
+          const int g = ring_cell(i, c);
+          if (g < 0) continue;
+          unsigned long long lo, hi;
+          get_words(xv + 2 * (size_t)g, lo, hi);
+          if (!wait_pair(xv + 2 * (size_t)g, ep, lo, hi, &s_fault)) s_fault = 1;
+          sv[c] = words_double(lo, hi);
+        }
+      } else if (app == 1) {
+        unsigned long long* xr = A.xres + (size_t)(pair & 1) * A.nb * 2;
+        const double mine = warp_sum(lane < nww ? s_wres[lane] : 0.0);
+        if (lane == 0) put_elem(xr + 2 * blockIdx.x, s_bad ? (double)NAN : mine, ep);
+        const double v = gather_sum(xr, A.nb, ep, &s_fault);
+        const bool first = lane == 0 && blockIdx.x == 0;
+        int d = RUNNING;
+        if (!isfinite(v)) d = NONFINITE;
+        else if (it > 0 && v <= tol) d = CONVERGED;
+        else if (it >= maxit) d = MAX_ITER;
+        else if (stall > 0 && it >= 1) {
+          // the stall rule (stall_rule), its state in this warp: every block keeps the same
+          since = (it == 1 || v < best) ? 0 : since + 1;
+          best = it == 1 ? v : fmin(best, v);
+          if (since >= stall) d = STALLED;
+        }
+        if (first) {
+          if (it > 0) ctrl->res_last = v;
+          if (d != RUNNING) ctrl->done = d;
+        }
+        if (lane == 0) s_dec = d != RUNNING;
+      }
+      __syncthreads();
+      if (s_dec || s_fault) {
+        run = false;
+        break;
+      }
+      // the first iterates b_D = c_D v, b_{D+1} = 0
+      const double cD = __ldg(A.coef + A.D);
+      for (int c = tid; c < box; c += blockDim.x) {
+        cur1[c] = wscale(cD, sv[c]);
+        cur2[c] = 0.0;
+      }
+      __syncthreads();
+      T res = T(0);
+      int bad = 0;
+      const bool have_prev = app == 0 && it > 0;
+      int ns = A.D % H == 0 ? H : A.D % H;
+      for (int k = A.D - 1; k >= 0;) {
+        for (int st = 0; st < ns; ++st) {
+          const int kk = k - st, hh = ns - 1 - st;
+          const double ck = __ldg(A.coef + kk);
+          const double sc = kk == 0 ? A.inv_delta : A.two_over_delta;
+          const int rx = w + 2 * hh, cells = rx * (h + 2 * hh);
+          const float inv = 1.0f / (float)rx;
+          const bool last = hh == 0;
+          unsigned long long* xb = A.xb + (size_t)((ep + 1) & 1) * N * 4;
+          for (int i = work ? tid : cells; i < cells; i += nwork) {
+            const int yy = quot(i, inv), xx = i - yy * rx;
+            const int c = (H - hh + yy) * SX + H - hh + xx;
+            const int f = s_nb[c];
+            const double bc = cur1[c];
+            double Ab = bc;
+            Ab = nb_term(Ab, f & 2 ? A.cx : 0.0, bc, cur1[c - 1]);
+            Ab = nb_term(Ab, f & 4 ? A.cx : 0.0, bc, cur1[c + 1]);
+            Ab = nb_term(Ab, f & 8 ? A.cy : 0.0, bc, cur1[c - SX]);
+            Ab = nb_term(Ab, f & 16 ? A.cy : 0.0, bc, cur1[c + SX]);
+            const double r = f ? cl_value(ck, sv[c], sc, Ab, A.theta, bc, cur2[c]) : 0.0;
+            if (!last || kk > 0) {
+              cur2[c] = r;
+              if (last && f && edge(xx, yy)) {
+                unsigned long long* x4 = xb + 4 * ((size_t)(y0 + yy) * nx + x0 + xx);
+                put_elem(x4, r, ep + 1);
+                put_elem(x4 + 2, bc, ep + 1);
+              }
+              continue;
+            }
+            // the closing step's output into the b-update or the prox
+            const T y = close_out<T>(r);
+            if (app == 0) {
+              const T qi = s_q[i];
+              if (have_prev) res += abs_residual<T>(s_b[i], y, qi);
+              const T bn = b_update<T>(qi, y);
+              bad |= !dev_finite(bn);
+              s_b[i] = bn;
+              sv[c] = f ? (double)bn : 0.0;
+            } else {
+              const T ai = prox_ratio<T, EK>(P, (y0 + yy) * nx + x0 + xx, y);
+              bad |= !dev_finite(ai);
+              sv[c] = f ? (double)ai : 0.0;
+              s_a[i] = ai;
+              s_p[i] = ai * y;
+            }
+          }
+          double* t = cur2;
+          cur2 = cur1;
+          cur1 = t;
+          if (!last) __syncthreads();
+        }
+        k -= ns;
+        ns = H;
+        if (k < 0) break;
+        // the neighbours' newest iterate and the one before, on the halo (the loads in
+        // flight while the block finishes its step)
+        ++ep;
+        unsigned long long* xb = A.xb + (size_t)(ep & 1) * N * 4;
+        constexpr int UN = 2;
+        unsigned long long q0[UN], q1[UN], q2[UN], q3[UN];
+        int cc[UN], gg[UN];
+#pragma unroll
+        for (int u = 0; u < UN; ++u) {
+          const int i = tid + u * nwork;
+          gg[u] = work && i < ring ? ring_cell(i, cc[u]) : -1;
+          if (gg[u] >= 0) {
+            get_words(xb + 4 * (size_t)gg[u], q0[u], q1[u]);
+            get_words(xb + 4 * (size_t)gg[u] + 2, q2[u], q3[u]);
+          }
+        }
+        __syncthreads();
+        auto take = [&](int g, int c, unsigned long long a, unsigned long long b,
+                        unsigned long long d, unsigned long long e) {
+          if (!wait_pair(xb + 4 * (size_t)g, ep, a, b, &s_fault) ||
+              !wait_pair(xb + 4 * (size_t)g + 2, ep, d, e, &s_fault))
+            s_fault = 1;
+          cur1[c] = words_double(a, b);
+          cur2[c] = words_double(d, e);
+        };
+#pragma unroll
+        for (int u = 0; u < UN; ++u)
+          if (gg[u] >= 0) take(gg[u], cc[u], q0[u], q1[u], q2[u], q3[u]);
+        for (int i = tid + UN * nwork; work && i < ring; i += nwork) {
+          int c;
+          const int g = ring_cell(i, c);
+          if (g < 0) continue;
+          unsigned long long a, b, d, e;
+          get_words(xb + 4 * (size_t)g, a, b);
+          get_words(xb + 4 * (size_t)g + 2, d, e);
+          take(g, c, a, b, d, e);
+        }
+        __syncthreads();
+        if (s_fault) break;
+      }
+      if (app == 0) {
+        const double wres = warp_res(res);
+        if (lane == 0) s_wres[wid] = wres;
+      } else {
+        ++it;
+      }
+      if (bad) s_bad = 1;
+      __syncthreads();
+    }
+  }
+
+  // the final a and p (p of the pair the last residual belongs to)
+  for (int i = tid; i < w * h; i += blockDim.x) {
+    const int y = i / w, x = i - y * w;
+    const size_t at = (size_t)(y0 + y) * nx + x0 + x;
+    A.a[at] = s_a[i];
+    A.p[at] = s_p[i];
+  }
+  if (tid == 0) {
+    if (s_fault) atomicOr(&ctrl->nonfinite, 2);
+    if (blockIdx.x == 0) {
+      ctrl->it = it;
+      *A.epoch = ep;
+    }
+  }
+}
+
+template <typename T>
+void* heat_tile_fn(int ek) {
+  if (ek == EK_CROWD) return (void*)heat_tile_kernel<T, EK_CROWD>;
+  if (ek == EK_ENTROPY) return (void*)heat_tile_kernel<T, EK_ENTROPY>;
+  return (void*)heat_tile_kernel<T, EK_POWER>;
+}
+
+// Work of a phase of H steps on a w x h tile, in warps.
+long long phase_warps(int w, int h, int H) {
+  long long s = 0;
+  for (int e = 0; e < H; ++e) s += ((long long)(w + 2 * e) * (h + 2 * e) + 31) / 32;
+  return s;
+}
+
+}  // namespace
+
+// One tile per block and at most one block per SM: the tile shape with the least work per
+// phase.  Where a tile with its halo does not fit the shared memory (about 900 cells a
+// side) heat.cu's form stays, whose blocks walk over several tiles.
+template <typename T>
+HeatTilePlan heat_tile_plan(int nx, int ny, int ek) {
+  HeatTilePlan tp;
+  int dev = 0, coop = 0, sms = 0, smem_max = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess) return tp;
+  cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev);
+  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  cudaDeviceGetAttribute(&smem_max, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+  if (!coop || sms < 1) return tp;
+  const int H = 4;
+  long long best = -1;
+  for (int gx = 1; gx <= std::min(nx, sms); ++gx) {
+    const int gy = std::min(ny, sms / gx);
+    const int w = ceil_div(nx, gx), h = ceil_div(ny, gy);
+    const long long c = phase_warps(w, h, H);
+    if (best < 0 || c < best) {
+      best = c;
+      tp.tw = w;
+      tp.th = h;
+    }
+  }
+  tp.H = H;
+  tp.ntx = ceil_div(nx, tp.tw);
+  const int nb = tp.ntx * ceil_div(ny, tp.th);
+  tp.smem = heat_tile_bytes(tp.tw, tp.th, H, sizeof(T));
+  const int area = (tp.tw + 2 * H - 2) * (tp.th + 2 * H - 2);
+  tp.threads = 32 + std::min(HTT - 32, (area + 31) / 32 * 32);
+  if (tp.smem + 1024 > (size_t)smem_max) return tp;
+  void* fn = heat_tile_fn<T>(ek);
+  int per_sm = 0;
+  if (cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)tp.smem) !=
+          cudaSuccess ||
+      cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, tp.threads, tp.smem) !=
+          cudaSuccess ||
+      per_sm * sms < nb) {
+    cudaGetLastError();
+    return tp;
+  }
+  tp.G = nb;
+  tp.words = (size_t)nx * ny * 12 + 4 * (size_t)nb + 2;
+  return tp;
+}
+
+template <typename T>
+cudaError_t heat_tile_launch(const HeatTilePlan& tp, const HeatPlan& hp, const HeatBuffers& B,
+                             int ek, const T* q, T* a, T* p, int nx, int ny, const uint8_t* mask,
+                             const ProxArgs<T>& P, Ctrl* ctrl, unsigned long long* words,
+                             int pairs, cudaStream_t st) {
+  const size_t N = (size_t)nx * ny;
+  const double inv_delta = hp.delta > 0 ? 1.0 / hp.delta : 0.0;
+  HeatTileArgs<T> A{nx, ny, tp.tw, tp.th, tp.ntx, tp.G, tp.H, hp.D, hp.cx, hp.cy, 2.0 * inv_delta,
+                    inv_delta, hp.theta, (const double*)B.coef, mask, q, a, p, ctrl, words,
+                    words + 8 * N, words + 12 * N, (unsigned*)(words + tp.words - 2), pairs};
+  ProxArgs<T> Pc = P;
+  void* args[] = {&A, &Pc};
+  StripPlan sp;
+  sp.G = tp.G;
+  return strip_coop(heat_tile_fn<T>(ek), sp, tp.smem, tp.threads, args, st);
+}
+
+#define JKO_HEAT_TILE_INST(T)                                                                    \
+  template HeatTilePlan heat_tile_plan<T>(int, int, int);                                        \
+  template cudaError_t heat_tile_launch<T>(const HeatTilePlan&, const HeatPlan&,                 \
+                                           const HeatBuffers&, int, const T*, T*, T*, int, int,  \
+                                           const uint8_t*, const ProxArgs<T>&, Ctrl*,            \
+                                           unsigned long long*, int, cudaStream_t);
+JKO_HEAT_TILE_INST(float)
+JKO_HEAT_TILE_INST(double)
+#undef JKO_HEAT_TILE_INST
+
+}  // namespace jko

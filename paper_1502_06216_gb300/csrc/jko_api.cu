@@ -533,12 +533,21 @@ cudaError_t enqueue_strip(jko_handle* h, int pairs, cudaStream_t st) {
                               h->strip_words, pairs, st);
 }
 
+template <typename T>
+cudaError_t enqueue_heat_tiles(jko_handle* h, int pairs, cudaStream_t st) {
+  return jko::heat_tile_launch<T>(h->htile, h->heat, h->hb, h->ek, (const T*)h->q, (T*)h->a,
+                                  (T*)h->p, h->grid.nx, h->grid.ny, (const uint8_t*)h->mask,
+                                  jko::prox_args<T>(h), h->ctrl, h->htile_words, pairs, st);
+}
+
 // `pairs` pairs as one persistent launch: the tensor-core loop kernel, the
 // heat kernel's persistent form or the CUDA-core filter's.
 cudaError_t enqueue_loop(jko_handle* h, int pairs, cudaStream_t st) {
   if (h->tc) return jko::tc_enqueue_loop(h->tc, pairs, st);
   if (!h->heat_L)
     return h->fp64 ? enqueue_strip<double>(h, pairs, st) : enqueue_strip<float>(h, pairs, st);
+  if (h->htile.G > 0)
+    return h->fp64 ? enqueue_heat_tiles<double>(h, pairs, st) : enqueue_heat_tiles<float>(h, pairs, st);
   const int nx = h->grid.nx, ny = h->grid.ny;
   const uint8_t* mask = (const uint8_t*)h->mask;
   if (h->fp64)
@@ -722,7 +731,7 @@ void free_handle(jko_handle* h) {
                   h->fft_khat_x, h->fft_tw_x, h->fft_khat_y, h->fft_tw_y,
                   h->tape, h->adj, h->adj2, h->adj_red, h->hb.d[0], h->hb.d[1], h->hb.d[2],
                   h->hb.d[3], h->hb.coef, h->a3, h->b3, h->s3, h->t2, h->t3, h->mpair,
-                  h->strip_words, h->adj_status};
+                  h->strip_words, h->adj_status, h->htile_words};
   for (void* b : bufs) if (b) cudaFree(b);
   if (h->ctrl_init) cudaFreeHost(h->ctrl_init);
   if (h->poll) cudaFreeHost(h->poll);
@@ -1552,6 +1561,16 @@ jko_status jko_create(const jko_grid* grid, const jko_params* params, const jko_
       s = set_err(h, JKO_ERR_UNSUPPORTED,
                   "the persistent heat-kernel loop cannot run here (no cooperative launch)");
     h->use_loop = h->heat_G > 0;
+    if (s == JKO_OK && h->use_loop) {
+      h->htile = h->fp64 ? jko::heat_tile_plan<double>(grid->nx, grid->ny, h->ek)
+                         : jko::heat_tile_plan<float>(grid->nx, grid->ny, h->ek);
+      if (h->htile.G > 0) {
+        const size_t wb = sizeof(unsigned long long) * h->htile.words;
+        e = cudaMalloc((void**)&h->htile_words, wb);
+        if (e == cudaSuccess) e = cudaMemset(h->htile_words, 0, wb);
+        if (e != cudaSuccess) s = cuda_err(h, e, "cudaMalloc(heat tiles)");
+      }
+    }
   }
   if (s != JKO_OK) return fail(s);
   if (h->prec == JKO_FP64 || h->prec == JKO_FP32) {

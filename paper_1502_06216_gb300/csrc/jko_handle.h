@@ -56,6 +56,8 @@ struct jko_handle {
   int nparts_pw = 0;            // residual partials of the pairwise column half-step
   jko::HeatPlan heat;
   jko::HeatBuffers hb;
+  jko::HeatTilePlan htile;       // the resident-tile form of a step (G = 0: not available)
+  unsigned long long* htile_words = nullptr;
   void *a2 = nullptr, *b2 = nullptr, *tgt = nullptr, *s1 = nullptr, *s2 = nullptr;
   uint8_t* mask = nullptr;
   double kappa_s = INFINITY;

@@ -242,6 +242,20 @@ cudaError_t heat_loop_launch(const HeatPlan& hp, const HeatBuffers& B, int ek, c
                              T* b, T* p, int nx, int ny, const uint8_t* mask, const ProxArgs<T>& P,
                              Ctrl* ctrl, double* part, int G, int pairs, cudaStream_t st);
 
+// The same on resident tiles (heat_tile.cu): G blocks, each a tile of tw x th cells and a
+// halo of H; G = 0 where the tiles do not fit.  words: zeroed once before the first launch.
+struct HeatTilePlan {
+  int G = 0, tw = 0, th = 0, ntx = 0, H = 0, threads = 0;
+  size_t smem = 0, words = 0;
+};
+template <typename T>
+HeatTilePlan heat_tile_plan(int nx, int ny, int ek);
+template <typename T>
+cudaError_t heat_tile_launch(const HeatTilePlan& tp, const HeatPlan& hp, const HeatBuffers& B,
+                             int ek, const T* q, T* a, T* p, int nx, int ny, const uint8_t* mask,
+                             const ProxArgs<T>& P, Ctrl* ctrl, unsigned long long* words,
+                             int pairs, cudaStream_t st);
+
 // Batched flows: copy the stop state of n control blocks into a contiguous
 // array (done flags only, or whole blocks).
 // A stopped step runs on: done = RUNNING, the stall counters restart (the

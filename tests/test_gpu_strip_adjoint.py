@@ -39,7 +39,8 @@ def test_reverse_pass_on_strips_equals_the_kernels_per_pass(kind, nx, ny, prec):
     for loop in (2, 0):
         h = jko.create_from_problem(pb, precision=jko.Precision[prec], loop=loop, tol=tol,
                                     max_iter=2000)
-        assert jko.jko_handle_info(h)["loop"] == (loop == 0 and not (prec == "FP64" and nx > 304))
+        strips = jko.jko_handle_info(h)["loop"]      # FP64: up to two lines a block
+        assert strips == (loop == 0 and not (prec == "FP64" and nx > 304))
         p0 = torch.tensor(pb.q0, dtype=h.dtype, device="cuda")
         g = torch.tensor(np.random.default_rng(5).normal(size=pb.N), dtype=h.dtype, device="cuda")
         want_w = kind != "exponents"
@@ -47,7 +48,7 @@ def test_reverse_pass_on_strips_equals_the_kernels_per_pass(kind, nx, ny, prec):
         first = jko.jko_flow_backward(h, g, want_w=want_w)
         again = jko.jko_flow_backward(h, g, want_w=want_w)
         for a, b in zip(first[:2 if want_w else 1], again):
-            assert loop == 2 or torch.equal(a, b)
+            assert not strips or torch.equal(a, b)
         grads.append([x.double().cpu().numpy() for x in first[:2 if want_w else 1]])
         jko.jko_destroy(h)
     sup = pb.q0 > 0          # dL/dp_0 is compared where the flow started with mass
