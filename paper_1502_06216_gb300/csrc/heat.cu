@@ -31,9 +31,8 @@ constexpr int HBX = 16, HBY = 8;   // small tiles: the work is FP64-bound per SM
 
 struct HeatGeom {
   int nx, ny;
-  double cx, cy;          // c / hx^2, c / hy^2
+  double ax, ay;          // 2 c / (delta hx^2), 2 c / (delta hy^2) (cl_value)
   const uint8_t* mask;    // 1 = obstacle, or NULL
-  double two_over_delta;  // 2 / delta (Clenshaw recurrence)
   bool linear;            // output not clamped at 0 (signed inputs: the adjoint)
 };
 
@@ -41,17 +40,16 @@ __device__ __forceinline__ bool is_free(const HeatGeom& g, int i) {
   return g.mask == nullptr || g.mask[i] == 0;
 }
 
-// (A v)_i = v_i + sum over free neighbours j of c_dir (v_i - v_j)
-template <typename W>
-__device__ __forceinline__ W apply_A(const HeatGeom& g, const W* v, int x, int y, W cx, W cy) {
+// One Clenshaw step at the free cell (x, y): b1 read at the stencil.
+__device__ __forceinline__ double cl_cell(const HeatGeom& g, double ck, double v, double b2,
+                                          double ax, double ay, const double* b1, int x, int y) {
   const int i = y * g.nx + x;
-  const W vi = v[i];
-  W acc = vi;
-  if (x > 0 && is_free(g, i - 1)) acc = nb_term(acc, cx, vi, v[i - 1]);
-  if (x + 1 < g.nx && is_free(g, i + 1)) acc = nb_term(acc, cx, vi, v[i + 1]);
-  if (y > 0 && is_free(g, i - g.nx)) acc = nb_term(acc, cy, vi, v[i - g.nx]);
-  if (y + 1 < g.ny && is_free(g, i + g.nx)) acc = nb_term(acc, cy, vi, v[i + g.nx]);
-  return acc;
+  const double c = b1[i];
+  const double l = x > 0 && is_free(g, i - 1) ? b1[i - 1] : c;
+  const double r = x + 1 < g.nx && is_free(g, i + 1) ? b1[i + 1] : c;
+  const double u = y > 0 && is_free(g, i - g.nx) ? b1[i - g.nx] : c;
+  const double d = y + 1 < g.ny && is_free(g, i + g.nx) ? b1[i + g.nx] : c;
+  return cl_value(ck, v, b2, ax, ay, l, r, u, d);
 }
 
 // First Clenshaw step: b_D = c_D v, b_{D+1} = 0 (v is 0 on the mask).
@@ -72,16 +70,14 @@ __global__ void __launch_bounds__(HBX * HBY) heat_cl_init(const T* v, void* b1_,
   b2[i] = wzero<W>();
 }
 
-// One Clenshaw step c_k v + s (B b1) - b2 with B = (A - theta Id) / delta:
-// s = 2 inside the recurrence (iterate out), s = 1 for the closing step
-// (CLOSE: T out, the operator's output).  out may alias b2 (each thread reads
+// One Clenshaw step c_k v + 2 B b1 - b2 with B = (A - theta Id) / delta (iterate
+// out); the closing step takes B b1 (CLOSE: T out, the operator's output).  out may alias b2 (each thread reads
 // its own b2 entry before writing it); b1 is read at the 5-point stencil and
 // is not written.
 template <typename T, bool CLOSE>
 __global__ void __launch_bounds__(HBX * HBY) heat_cl_step(const T* v, const void* b1_,
                                                           const void* b2_, void* out_, HeatGeom g,
-                                                          double ck_, double s_over_delta,
-                                                          double theta_, Ctrl* ctrl) {
+                                                          double ck, Ctrl* ctrl) {
   using W = typename HeatIter<T>::W;
   const W* b1 = (const W*)b1_;
   const W* b2 = (const W*)b2_;
@@ -95,9 +91,8 @@ __global__ void __launch_bounds__(HBX * HBY) heat_cl_step(const T* v, const void
     else ((W*)out_)[i] = wzero<W>();
     return;
   }
-  const W cx = wc<W>(g.cx), cy = wc<W>(g.cy);
-  const W Ab = apply_A<W>(g, b1, xx, yy, cx, cy);
-  const W r = cl_value(wc<W>(ck_), wv(v[i]), wc<W>(s_over_delta), Ab, wc<W>(theta_), b1[i], b2[i]);
+  const double s = CLOSE ? 0.5 : 1.0;
+  const W r = cl_cell(g, ck, wv(v[i]), b2[i], s * g.ax, s * g.ay, b1, xx, yy);
   if (CLOSE) ((T*)out_)[i] = g.linear ? (T)r : close_out<T>(r);
   else ((W*)out_)[i] = r;
 }
@@ -105,13 +100,13 @@ __global__ void __launch_bounds__(HBX * HBY) heat_cl_step(const T* v, const void
 // Two Clenshaw steps in one launch: b_k on the block's tile plus a one-cell
 // halo (shared memory), then b_{k-1} on the tile from it.  Reads b_{k+1} (at a
 // two-cell halo) and b_{k+2}; writes b_k (o1) and b_{k-1} (o2), buffers that no
-// block of this launch reads.  The second step is the closing one (s2 = 1 /
-// delta, CLOSE: o2 = the operator's output, of type T) when k - 1 = 0.
+// block of this launch reads.  The second step is the closing one (CLOSE: o2
+// = the operator's output, of type T) when k - 1 = 0.
 template <typename T, bool CLOSE>
 __global__ void __launch_bounds__(HBX * HBY) heat_cl_step2(const T* v, const void* b1_,
                                                            const void* b2_, void* o1_, void* o2_,
-                                                           HeatGeom g, double ck_, double ck1_,
-                                                           double s2_, double theta_, Ctrl* ctrl) {
+                                                           HeatGeom g, double ck, double ck1,
+                                                           Ctrl* ctrl) {
   using W = typename HeatIter<T>::W;
   const W* b1 = (const W*)b1_;
   const W* b2 = (const W*)b2_;
@@ -120,8 +115,6 @@ __global__ void __launch_bounds__(HBX * HBY) heat_cl_step2(const T* v, const voi
   __shared__ W sb[RY][RX];
   __shared__ int s_it;
   if (stop_gate(ctrl, nullptr, 0, false, &s_it)) return;
-  const W cx = wc<W>(g.cx), cy = wc<W>(g.cy), theta = wc<W>(theta_);
-  const W two = wc<W>(g.two_over_delta), ck = wc<W>(ck_);
   const int x0 = blockIdx.x * HBX, y0 = blockIdx.y * HBY;
   const int tid = threadIdx.y * HBX + threadIdx.x;
   for (int idx = tid; idx < RX * RY; idx += HBX * HBY) {
@@ -130,10 +123,7 @@ __global__ void __launch_bounds__(HBX * HBY) heat_cl_step2(const T* v, const voi
     W val = wzero<W>();
     if (x >= 0 && x < g.nx && y >= 0 && y < g.ny) {
       const int i = y * g.nx + x;
-      if (is_free(g, i)) {
-        const W Ab = apply_A<W>(g, b1, x, y, cx, cy);
-        val = cl_value(ck, wv(v[i]), two, Ab, theta, b1[i], b2[i]);
-      }
+      if (is_free(g, i)) val = cl_cell(g, ck, wv(v[i]), b2[i], g.ax, g.ay, b1, x, y);
     }
     sb[ry][rx] = val;
   }
@@ -149,13 +139,13 @@ __global__ void __launch_bounds__(HBX * HBY) heat_cl_step2(const T* v, const voi
     else ((W*)o2_)[i] = wzero<W>();
     return;
   }
-  // A b_k at (x, y) from the tile: the neighbour tests of apply_A
-  W acc = c;
-  if (x > 0 && is_free(g, i - 1)) acc = nb_term(acc, cx, c, sb[ty][tx - 1]);
-  if (x + 1 < g.nx && is_free(g, i + 1)) acc = nb_term(acc, cx, c, sb[ty][tx + 1]);
-  if (y > 0 && is_free(g, i - g.nx)) acc = nb_term(acc, cy, c, sb[ty - 1][tx]);
-  if (y + 1 < g.ny && is_free(g, i + g.nx)) acc = nb_term(acc, cy, c, sb[ty + 1][tx]);
-  const W r = cl_value(wc<W>(ck1_), wv(v[i]), wc<W>(s2_), acc, theta, c, b1[i]);
+  // b_k around (x, y) from the tile: the neighbour tests of cl_cell
+  const W l = x > 0 && is_free(g, i - 1) ? sb[ty][tx - 1] : c;
+  const W rr = x + 1 < g.nx && is_free(g, i + 1) ? sb[ty][tx + 1] : c;
+  const W u = y > 0 && is_free(g, i - g.nx) ? sb[ty - 1][tx] : c;
+  const W d = y + 1 < g.ny && is_free(g, i + g.nx) ? sb[ty + 1][tx] : c;
+  const double s = CLOSE ? 0.5 : 1.0;
+  const W r = cl_value(ck1, wv(v[i]), b1[i], s * g.ax, s * g.ay, l, rr, u, d);
   if (CLOSE) ((T*)o2_)[i] = g.linear ? (T)r : close_out<T>(r);
   else ((W*)o2_)[i] = r;
 }
@@ -235,7 +225,6 @@ struct HeatLoopArgs {
   HeatGeom g;
   const double* coef;      // c_0 .. c_D
   int D;
-  double theta, inv_delta;
   void* d[4];              // Clenshaw iterates (HeatIter<T>::W, 8 bytes per cell)
   const T* q;
   T* a;
@@ -252,8 +241,6 @@ struct HeatLoopArgs {
 template <typename T>
 __device__ __forceinline__ T ld_plain(const T* p) { return *p; }
 
-// A v at (x, y) where v is stored as c * v[j] (the first iterate b_D = c_D v):
-// the neighbour terms of apply_A on those values.
 // The closing step's output r at cell i of the grid, into the b-update (app 0)
 // or the prox (app 1).
 template <typename T, int EK>
@@ -298,7 +285,7 @@ template <typename T, int EK, typename W>
 __device__ __forceinline__ void heat_tile_steps(const HeatLoopArgs<T>& A, int app, int t, const T* v,
                                                 const W* b1, const W* b2, W* o_new, W* o_prev,
                                                 bool virt, W c1v, int k, int ns, bool have_prev,
-                                                HeatStageH<W>& S, W cx, W cy, W theta, double* s_red,
+                                                HeatStageH<W>& S, double* s_red,
                                                 int& bad) {
   constexpr int H = HMAX;
   const HeatGeom& g = A.g;
@@ -333,7 +320,7 @@ __device__ __forceinline__ void heat_tile_steps(const HeatLoopArgs<T>& A, int ap
   for (int st = 0; st < ns; ++st) {
     const int kk = k - st;
     const W ck = wc<W>(__ldg(A.coef + kk));
-    const W sc = wc<W>(kk == 0 ? A.inv_delta : g.two_over_delta);
+    const W ax = kk == 0 ? 0.5 * g.ax : g.ax, ay = kk == 0 ? 0.5 * g.ay : g.ay;
     if (st < ns - 1) {
       // b_kk on the tile and an (ns - 1 - st)-cell halo, into cur2's array
       const int h = ns - 1 - st;
@@ -344,12 +331,11 @@ __device__ __forceinline__ void heat_tile_steps(const HeatLoopArgs<T>& A, int ap
         W val = wzero<W>();
         if (S.fr[ey][ex]) {
           const W bc = cur1[ey][ex];
-          W Ab = bc;
-          if (S.fr[ey][ex - 1]) Ab = nb_term(Ab, cx, bc, cur1[ey][ex - 1]);
-          if (S.fr[ey][ex + 1]) Ab = nb_term(Ab, cx, bc, cur1[ey][ex + 1]);
-          if (S.fr[ey - 1][ex]) Ab = nb_term(Ab, cy, bc, cur1[ey - 1][ex]);
-          if (S.fr[ey + 1][ex]) Ab = nb_term(Ab, cy, bc, cur1[ey + 1][ex]);
-          val = cl_value(ck, S.v[ey][ex], sc, Ab, theta, bc, cur2[ey][ex]);
+          const W bl = S.fr[ey][ex - 1] ? cur1[ey][ex - 1] : bc;
+          const W br = S.fr[ey][ex + 1] ? cur1[ey][ex + 1] : bc;
+          const W bu = S.fr[ey - 1][ex] ? cur1[ey - 1][ex] : bc;
+          const W bd = S.fr[ey + 1][ex] ? cur1[ey + 1][ex] : bc;
+          val = cl_value(ck, S.v[ey][ex], cur2[ey][ex], ax, ay, bl, br, bu, bd);
         }
         cur2[ey][ex] = val;
       }
@@ -366,12 +352,11 @@ __device__ __forceinline__ void heat_tile_steps(const HeatLoopArgs<T>& A, int ap
         W r = wzero<W>();
         if (S.fr[ey][ex]) {
           const W bc = cur1[ey][ex];
-          W Ab = bc;
-          if (S.fr[ey][ex - 1]) Ab = nb_term(Ab, cx, bc, cur1[ey][ex - 1]);
-          if (S.fr[ey][ex + 1]) Ab = nb_term(Ab, cx, bc, cur1[ey][ex + 1]);
-          if (S.fr[ey - 1][ex]) Ab = nb_term(Ab, cy, bc, cur1[ey - 1][ex]);
-          if (S.fr[ey + 1][ex]) Ab = nb_term(Ab, cy, bc, cur1[ey + 1][ex]);
-          r = cl_value(ck, S.v[ey][ex], sc, Ab, theta, bc, cur2[ey][ex]);
+          const W bl = S.fr[ey][ex - 1] ? cur1[ey][ex - 1] : bc;
+          const W br = S.fr[ey][ex + 1] ? cur1[ey][ex + 1] : bc;
+          const W bu = S.fr[ey - 1][ex] ? cur1[ey - 1][ex] : bc;
+          const W bd = S.fr[ey + 1][ex] ? cur1[ey + 1][ex] : bc;
+          r = cl_value(ck, S.v[ey][ex], cur2[ey][ex], ax, ay, bl, br, bu, bd);
         }
         if (kk == 0) {
           heat_close_cell<T, EK>(A, app, i, close_out<T>(r), have_prev, res, bad);
@@ -471,7 +456,6 @@ __global__ void __launch_bounds__(HLT) heat_loop_kernel(HeatLoopArgs<T> A) {
       const T* v = app == 0 ? A.a : A.b;
       const bool have_prev = app == 0 && it > 0;
       const W cD = wc<W>(__ldg(A.coef + D));
-      const W cx = wc<W>(A.g.cx), cy = wc<W>(A.g.cy), theta = wc<W>(A.theta);
       W* dd[4] = {(W*)A.d[0], (W*)A.d[1], (W*)A.d[2], (W*)A.d[3]};
       // phases of up to HMAX steps from the first iterates (b_D = c_D v,
       // b_{D+1} = 0), the first one taking D mod HMAX steps; buffers: read
@@ -484,8 +468,8 @@ __global__ void __launch_bounds__(HLT) heat_loop_kernel(HeatLoopArgs<T> A) {
       while (k >= 0) {
         for (int t = blockIdx.x; t < A.ntiles; t += G)
           heat_tile_steps<T, EK, W>(A, app, t, v, virt ? nullptr : dd[r1], virt ? nullptr : dd[r2],
-                                    dd[f1], dd[f2], virt, cD, k, ns, have_prev, stg, cx, cy, theta,
-                                    s_red, bad);
+                                    dd[f1], dd[f2], virt, cD, k, ns, have_prev, stg, s_red,
+                                    bad);
         if (!barrier()) { run = false; break; }
         k -= ns;
         ns = hm;
@@ -594,7 +578,7 @@ cudaError_t heat_apply(const HeatPlan& hp, const HeatBuffers& B, const T* in, T*
                        int nx, int ny, const uint8_t* mask, Ctrl* ctrl, const double* part,
                        int nparts, int decide, cudaStream_t st, bool linear) {
   const double inv_delta = hp.delta > 0 ? 1.0 / hp.delta : 0.0;   // delta = 0: p(A) = c_0 Id
-  HeatGeom g{nx, ny, hp.cx, hp.cy, mask, 2.0 * inv_delta, linear};
+  HeatGeom g{nx, ny, 2.0 * inv_delta * hp.cx, 2.0 * inv_delta * hp.cy, mask, linear};
   const dim3 grid = heat_grid(nx, ny), block(HBX, HBY);
   void* d[4] = {B.d[0], B.d[1], B.d[2], B.d[3]};   // iterates (8 bytes per cell)
   const int D = hp.D;
@@ -606,23 +590,22 @@ cudaError_t heat_apply(const HeatPlan& hp, const HeatBuffers& B, const T* in, T*
   if (D % 2 == 1) {   // one single step so that the rest pairs up
     if (k == 0) {
       heat_cl_step<T, true><<<grid, block, 0, st>>>(in, d[r1], d[r2], out_x, g, hp.coef[0],
-                                                    inv_delta, hp.theta, ctrl);
+                                                    ctrl);
       return cudaGetLastError();
     }
     heat_cl_step<T, false><<<grid, block, 0, st>>>(in, d[r1], d[r2], d[r2], g, hp.coef[k],
-                                                   2.0 * inv_delta, hp.theta, ctrl);
+                                                   ctrl);
     std::swap(r1, r2);
     --k;
   }
   for (; k >= 1; k -= 2) {
     if (k == 1) {   // steps 1 and the closing 0
       heat_cl_step2<T, true><<<grid, block, 0, st>>>(in, d[r1], d[r2], d[f1], out_x, g, hp.coef[1],
-                                                     hp.coef[0], inv_delta, hp.theta, ctrl);
+                                                     hp.coef[0], ctrl);
       break;
     }
     heat_cl_step2<T, false><<<grid, block, 0, st>>>(in, d[r1], d[r2], d[f1], d[f2], g,
-                                                    hp.coef[k], hp.coef[k - 1],
-                                                    2.0 * inv_delta, hp.theta, ctrl);
+                                                    hp.coef[k], hp.coef[k - 1], ctrl);
     // b_{k-1} (f2) and b_k (f1) are the next step's b_{k'+1}, b_{k'+2}
     const int o1 = r1, o2 = r2;
     r1 = f2;
@@ -669,11 +652,9 @@ cudaError_t heat_loop_launch(const HeatPlan& hp, const HeatBuffers& B, int ek, c
                              Ctrl* ctrl, double* part, int G, int pairs, cudaStream_t st) {
   HeatLoopArgs<T> A{};
   const double inv_delta = hp.delta > 0 ? 1.0 / hp.delta : 0.0;
-  A.g = HeatGeom{nx, ny, hp.cx, hp.cy, mask, 2.0 * inv_delta};
+  A.g = HeatGeom{nx, ny, 2.0 * inv_delta * hp.cx, 2.0 * inv_delta * hp.cy, mask, false};
   A.coef = (const double*)B.coef;
   A.D = hp.D;
-  A.theta = hp.theta;
-  A.inv_delta = inv_delta;
   for (int i = 0; i < 4; ++i) A.d[i] = B.d[i];
   A.q = q;
   A.a = a;
@@ -708,7 +689,7 @@ cudaError_t heat_loop_launch(const HeatPlan& hp, const HeatBuffers& B, int ek, c
 template <typename T>
 cudaError_t heat_bupdate_launch(const T* Y, T* b, const T* q, int nx, int ny, Ctrl* ctrl,
                                 double* part, cudaStream_t st) {
-  HeatGeom g{nx, ny, 0.0, 0.0, nullptr};
+  HeatGeom g{nx, ny, 0.0, 0.0, nullptr, false};
   heat_bupdate<T><<<heat_grid(nx, ny), dim3(HBX, HBY), 0, st>>>(Y, b, q, g, ctrl, part);
   return cudaGetLastError();
 }
@@ -716,7 +697,7 @@ cudaError_t heat_bupdate_launch(const T* Y, T* b, const T* q, int nx, int ny, Ct
 template <typename T>
 cudaError_t heat_prox_launch(int ek, const T* s, T* a, T* p, int nx, int ny, const ProxArgs<T>& P,
                              Ctrl* ctrl, cudaStream_t st) {
-  HeatGeom g{nx, ny, 0.0, 0.0, nullptr};
+  HeatGeom g{nx, ny, 0.0, 0.0, nullptr, false};
   const dim3 grid = heat_grid(nx, ny), block(HBX, HBY);
   if (ek == EK_CROWD) heat_prox<T, EK_CROWD><<<grid, block, 0, st>>>(s, a, p, g, P, ctrl);
   else if (ek == EK_ENTROPY) heat_prox<T, EK_ENTROPY><<<grid, block, 0, st>>>(s, a, p, g, P, ctrl);

@@ -26,14 +26,15 @@ template <typename W> __device__ __forceinline__ W wzero() { return 0.0; }
 // c v (the first iterate b_D = c_D v)
 __device__ __forceinline__ double wscale(double c, double v) { return __dmul_rn(c, v); }
 
-// acc + c (vi - vj): one neighbour's term of A v
-__device__ __forceinline__ double nb_term(double acc, double c, double vi, double vj) {
-  return __fma_rn(c, __dsub_rn(vi, vj), acc);
-}
-// one Clenshaw step's value ck v + s (A b1 - theta b1) - b2
-__device__ __forceinline__ double cl_value(double ck, double v, double s, double Ab, double theta,
-                                          double b1, double b2) {
-  return __dsub_rn(__fma_rn(ck, v, __dmul_rn(s, __fma_rn(-theta, b1, Ab))), b2);
+// One Clenshaw step's value ck v + 2 B b1 - b2, B = (A - theta Id) / delta.  With theta = 1 +
+// delta and delta = 2 cx + 2 cy (the interval is [1, 1 + 4 cx + 4 cy]) the diagonal of B
+// vanishes on an interior cell, and where a neighbour is missing (Neumann) the cell's own
+// value takes its place: 2 B b1 = -ax (l + r) - ay (u + d), ax = 2 cx / delta, ay = 2 cy /
+// delta (the closing step's B b1: half of both).  Five FP64 operations four deep, where the
+// sum over differences c (b1_i - b1_j), less theta b1, scaled, took twelve nine deep.
+__device__ __forceinline__ double cl_value(double ck, double v, double b2, double ax, double ay,
+                                           double l, double r, double u, double d) {
+  return __fma_rn(-ay, __dadd_rn(u, d), __fma_rn(-ax, __dadd_rn(l, r), __fma_rn(ck, v, -b2)));
 }
 
 // The operator's output is clamped at 0: xi~ is positive, and the expansion's

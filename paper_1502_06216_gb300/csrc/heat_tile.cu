@@ -11,10 +11,12 @@
 // within H cells).  The arithmetic of a cell and the stop rule are those of heat.cu's
 // kernels, so the iterates have the same bits; the residual is added by tiles.
 //
-// Bound by the FP64 latency of its steps and the exchange between them: at 100^2 (150
-// tiles, degree 54) 0.9 us a step and 1.1 us an exchange; 33 pairs take 5.69 ms on
-// heat.cu's blocks with a grid barrier a phase, 4.36 here with H = 4 (7.0, 5.1, 4.5, 4.4
-// and 4.6 with H = 1, 2, 3, 5 and 6: halo work against exchanges).
+// Bound by the exchange and by the FP64 latency of its steps (five operations a cell, four
+// deep, on a pipe of half a lane a cycle and scheduler): 100^2, 150 tiles, degree 54, a
+// 33-pair step: 5.69 ms on heat.cu's blocks with a grid barrier a phase, 4.36 on tiles,
+// 3.01 with the five-operation step and each thread's cells kept in registers.  H = 4: with
+// the longer step 7.0, 5.1, 4.5, 4.4, 4.4 and 4.6 ms for H = 1 to 6 (exchanges against
+// halo work).
 #include <algorithm>
 
 #include "heat_cell.cuh"
@@ -28,11 +30,12 @@ namespace {
 using namespace strip;
 
 constexpr int HTT = 512;   // threads at most: work warps and one that takes the decision
+constexpr int H = 4;       // Clenshaw steps per exchange at most, and cells of the halo
 
 template <typename T>
 struct HeatTileArgs {
-  int nx, ny, tw, th, ntx, nb, H, D;
-  double cx, cy, two_over_delta, inv_delta, theta;
+  int nx, ny, tw, th, ntx, nb, D;
+  double ax, ay;
   const double* coef;
   const uint8_t* mask;
   const T* q;
@@ -46,7 +49,7 @@ struct HeatTileArgs {
   int pairs;
 };
 
-__host__ __device__ inline size_t heat_tile_bytes(int tw, int th, int H, size_t es) {
+__host__ __device__ inline size_t heat_tile_bytes(int tw, int th, size_t es) {
   const size_t box = (size_t)(tw + 2 * H) * (th + 2 * H);
   return box * 25 + (size_t)tw * th * es * 4;
 }
@@ -72,7 +75,7 @@ heat_tile_kernel(const __grid_constant__ HeatTileArgs<T> A, const __grid_constan
   const int maxit = ctrl->max_iter, stall = ctrl->stall;
   const double tol = ctrl->tol;
   unsigned ep = *(volatile unsigned*)A.epoch;
-  const int nx = A.nx, ny = A.ny, H = A.H;
+  const int nx = A.nx, ny = A.ny;
   const size_t N = (size_t)nx * ny;
   const int by = blockIdx.x / A.ntx, bx = blockIdx.x - by * A.ntx;
   const int x0 = bx * A.tw, y0 = by * A.th;
@@ -130,6 +133,16 @@ heat_tile_kernel(const __grid_constant__ HeatTileArgs<T> A, const __grid_constan
     return (s_nb[c] & 1) ? (y0 + ey - H) * nx + x0 + ex - H : -1;
   };
   auto edge = [&](int x, int y) { return x < H || x >= w - H || y < H || y >= h - H; };
+
+  // the cell a work thread takes in a step on the tile and an e-cell halo, where every
+  // step has a thread per cell (else the steps loop over cells)
+  const bool one = (w + 2 * (H - 1)) * (h + 2 * (H - 1)) <= nwork;
+  int c_of[H];
+#pragma unroll
+  for (int e = 0; e < H; ++e) {
+    const int rx = w + 2 * e, yy = quot(tid, 1.0f / (float)rx), xx = tid - yy * rx;
+    c_of[e] = work && one && yy < h + 2 * e ? (H - e + yy) * SX + H - e + xx : -1;
+  }
 
   int it = 0, pair = 0, since = 0;
   double best = INFINITY;
@@ -194,56 +207,93 @@ heat_tile_kernel(const __grid_constant__ HeatTileArgs<T> A, const __grid_constan
       int bad = 0;
       const bool have_prev = app == 0 && it > 0;
       int ns = A.D % H == 0 ? H : A.D % H;
-      for (int k = A.D - 1; k >= 0;) {
-        for (int st = 0; st < ns; ++st) {
-          const int kk = k - st, hh = ns - 1 - st;
-          const double ck = __ldg(A.coef + kk);
-          const double sc = kk == 0 ? A.inv_delta : A.two_over_delta;
-          const int rx = w + 2 * hh, cells = rx * (h + 2 * hh);
-          const float inv = 1.0f / (float)rx;
-          const bool last = hh == 0;
-          unsigned long long* xb = A.xb + (size_t)((ep + 1) & 1) * N * 4;
-          for (int i = work ? tid : cells; i < cells; i += nwork) {
-            const int yy = quot(i, inv), xx = i - yy * rx;
-            const int c = (H - hh + yy) * SX + H - hh + xx;
-            const int f = s_nb[c];
-            const double bc = cur1[c];
-            double Ab = bc;
-            Ab = nb_term(Ab, f & 2 ? A.cx : 0.0, bc, cur1[c - 1]);
-            Ab = nb_term(Ab, f & 4 ? A.cx : 0.0, bc, cur1[c + 1]);
-            Ab = nb_term(Ab, f & 8 ? A.cy : 0.0, bc, cur1[c - SX]);
-            Ab = nb_term(Ab, f & 16 ? A.cy : 0.0, bc, cur1[c + SX]);
-            const double r = f ? cl_value(ck, sv[c], sc, Ab, A.theta, bc, cur2[c]) : 0.0;
-            if (!last || kk > 0) {
-              cur2[c] = r;
-              if (last && f && edge(xx, yy)) {
-                unsigned long long* x4 = xb + 4 * ((size_t)(y0 + yy) * nx + x0 + xx);
-                put_elem(x4, r, ep + 1);
-                put_elem(x4 + 2, bc, ep + 1);
-              }
-              continue;
-            }
-            // the closing step's output into the b-update or the prox
-            const T y = close_out<T>(r);
-            if (app == 0) {
-              const T qi = s_q[i];
-              if (have_prev) res += abs_residual<T>(s_b[i], y, qi);
-              const T bn = b_update<T>(qi, y);
-              bad |= !dev_finite(bn);
-              s_b[i] = bn;
-              sv[c] = f ? (double)bn : 0.0;
-            } else {
-              const T ai = prox_ratio<T, EK>(P, (y0 + yy) * nx + x0 + xx, y);
-              bad |= !dev_finite(ai);
-              sv[c] = f ? (double)ai : 0.0;
-              s_a[i] = ai;
-              s_p[i] = ai * y;
-            }
+      double v_of[H];
+#pragma unroll
+      for (int e = 0; e < H; ++e) v_of[e] = c_of[e] >= 0 ? sv[c_of[e]] : 0.0;
+      // step kk at cell c
+      auto value = [&](int c, int kk, double ck, double v) -> double {
+        const double s = kk == 0 ? 0.5 : 1.0;
+        const int f = s_nb[c];
+        const double bc = cur1[c], b2 = cur2[c];
+        const double bl = cur1[c - 1], br = cur1[c + 1], bu = cur1[c - SX], bd = cur1[c + SX];
+        const double r = cl_value(ck, v, b2, s * A.ax, s * A.ay, f & 2 ? bl : bc, f & 4 ? br : bc,
+                                  f & 8 ? bu : bc, f & 16 ? bd : bc);
+        return f ? r : 0.0;
+      };
+      // the last step of a phase at cell i = (x, y) of the tile: to the neighbours, or closed
+      // into the b-update or the prox
+      auto finish = [&](int i, int x, int y, int c, int kk, double r) {
+        const bool f = s_nb[c] & 1;
+        if (kk > 0) {
+          const double bc = cur1[c];
+          cur2[c] = r;
+          if (f && edge(x, y)) {
+            unsigned long long* x4 = A.xb + (size_t)((ep + 1) & 1) * N * 4 +
+                                     4 * ((size_t)(y0 + y) * nx + x0 + x);
+            put_elem(x4, r, ep + 1);
+            put_elem(x4 + 2, bc, ep + 1);
           }
-          double* t = cur2;
-          cur2 = cur1;
-          cur1 = t;
-          if (!last) __syncthreads();
+          return;
+        }
+        const T yv = close_out<T>(r);
+        if (app == 0) {
+          const T qi = s_q[i];
+          if (have_prev) res += abs_residual<T>(s_b[i], yv, qi);
+          const T bn = b_update<T>(qi, yv);
+          bad |= !dev_finite(bn);
+          s_b[i] = bn;
+          sv[c] = f ? (double)bn : 0.0;
+        } else {
+          const T ai = prox_ratio<T, EK>(P, (y0 + y) * nx + x0 + x, yv);
+          bad |= !dev_finite(ai);
+          sv[c] = f ? (double)ai : 0.0;
+          s_a[i] = ai;
+          s_p[i] = ai * yv;
+        }
+      };
+      auto swap = [&]() {
+        double* t = cur2;
+        cur2 = cur1;
+        cur1 = t;
+      };
+      const float inv_w = 1.0f / (float)w;
+      for (int k = A.D - 1; k >= 0;) {
+        if (one) {
+          double ck[H];
+#pragma unroll
+          for (int e = 0; e < H; ++e) ck[e] = e < ns ? __ldg(A.coef + (k - (ns - 1 - e))) : 0.0;
+#pragma unroll
+          for (int e = H - 1; e >= 0; --e) {
+            if (e >= ns) continue;
+            const int kk = k - (ns - 1 - e), c = c_of[e];
+            if (c >= 0) {
+              const double r = value(c, kk, ck[e], v_of[e]);
+              if (e > 0) {
+                cur2[c] = r;
+              } else {
+                const int y = quot(tid, inv_w);
+                finish(tid, tid - y * w, y, c, kk, r);
+              }
+            }
+            swap();
+            if (e > 0) __syncthreads();
+          }
+        } else {
+          for (int e = ns - 1; e >= 0; --e) {
+            const int kk = k - (ns - 1 - e);
+            const double ck = __ldg(A.coef + kk);
+            const int rx = w + 2 * e, cells = rx * (h + 2 * e);
+            const float inv = 1.0f / (float)rx;
+            for (int i = work ? tid : cells; i < cells; i += nwork) {
+              const int yy = quot(i, inv), xx = i - yy * rx;
+              const int c = (H - e + yy) * SX + H - e + xx;
+              const double r = value(c, kk, ck, sv[c]);
+              if (e > 0) cur2[c] = r;
+              else finish(i, xx, yy, c, kk, r);
+            }
+            swap();
+            if (e > 0) __syncthreads();
+          }
         }
         k -= ns;
         ns = H;
@@ -323,7 +373,7 @@ void* heat_tile_fn(int ek) {
 }
 
 // Work of a phase of H steps on a w x h tile, in warps.
-long long phase_warps(int w, int h, int H) {
+long long phase_warps(int w, int h) {
   long long s = 0;
   for (int e = 0; e < H; ++e) s += ((long long)(w + 2 * e) * (h + 2 * e) + 31) / 32;
   return s;
@@ -343,22 +393,20 @@ HeatTilePlan heat_tile_plan(int nx, int ny, int ek) {
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   cudaDeviceGetAttribute(&smem_max, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
   if (!coop || sms < 1) return tp;
-  const int H = 4;
   long long best = -1;
   for (int gx = 1; gx <= std::min(nx, sms); ++gx) {
     const int gy = std::min(ny, sms / gx);
     const int w = ceil_div(nx, gx), h = ceil_div(ny, gy);
-    const long long c = phase_warps(w, h, H);
+    const long long c = phase_warps(w, h);
     if (best < 0 || c < best) {
       best = c;
       tp.tw = w;
       tp.th = h;
     }
   }
-  tp.H = H;
   tp.ntx = ceil_div(nx, tp.tw);
   const int nb = tp.ntx * ceil_div(ny, tp.th);
-  tp.smem = heat_tile_bytes(tp.tw, tp.th, H, sizeof(T));
+  tp.smem = heat_tile_bytes(tp.tw, tp.th, sizeof(T));
   const int area = (tp.tw + 2 * H - 2) * (tp.th + 2 * H - 2);
   tp.threads = 32 + std::min(HTT - 32, (area + 31) / 32 * 32);
   if (tp.smem + 1024 > (size_t)smem_max) return tp;
@@ -384,8 +432,8 @@ cudaError_t heat_tile_launch(const HeatTilePlan& tp, const HeatPlan& hp, const H
                              int pairs, cudaStream_t st) {
   const size_t N = (size_t)nx * ny;
   const double inv_delta = hp.delta > 0 ? 1.0 / hp.delta : 0.0;
-  HeatTileArgs<T> A{nx, ny, tp.tw, tp.th, tp.ntx, tp.G, tp.H, hp.D, hp.cx, hp.cy, 2.0 * inv_delta,
-                    inv_delta, hp.theta, (const double*)B.coef, mask, q, a, p, ctrl, words,
+  HeatTileArgs<T> A{nx, ny, tp.tw, tp.th, tp.ntx, tp.G, hp.D, 2.0 * inv_delta * hp.cx,
+                    2.0 * inv_delta * hp.cy, (const double*)B.coef, mask, q, a, p, ctrl, words,
                     words + 8 * N, words + 12 * N, (unsigned*)(words + tp.words - 2), pairs};
   ProxArgs<T> Pc = P;
   void* args[] = {&A, &Pc};

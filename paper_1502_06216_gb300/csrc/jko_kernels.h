@@ -242,10 +242,10 @@ cudaError_t heat_loop_launch(const HeatPlan& hp, const HeatBuffers& B, int ek, c
                              T* b, T* p, int nx, int ny, const uint8_t* mask, const ProxArgs<T>& P,
                              Ctrl* ctrl, double* part, int G, int pairs, cudaStream_t st);
 
-// The same on resident tiles (heat_tile.cu): G blocks, each a tile of tw x th cells and a
-// halo of H; G = 0 where the tiles do not fit.  words: zeroed once before the first launch.
+// The same on resident tiles (heat_tile.cu): G blocks, each a tile of tw x th cells and its
+// halo; G = 0 where the tiles do not fit.  words: zeroed once before the first launch.
 struct HeatTilePlan {
-  int G = 0, tw = 0, th = 0, ntx = 0, H = 0, threads = 0;
+  int G = 0, tw = 0, th = 0, ntx = 0, threads = 0;
   size_t smem = 0, words = 0;
 };
 template <typename T>
