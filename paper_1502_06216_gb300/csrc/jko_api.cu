@@ -515,22 +515,29 @@ int strip_op(const jko_handle* h) {
   return h->attract ? jko::OP_ATTRACT : jko::OP_ONE;
 }
 
+// A whole step from q_in to out in one launch (StripStep); fresh: it resets the control
+// block itself.
 template <typename T>
-cudaError_t enqueue_strip(jko_handle* h, int pairs, cudaStream_t st) {
+cudaError_t enqueue_strip(jko_handle* h, const T* q_in, T* out, int check, int fresh, Ctrl* record,
+                          cudaStream_t st) {
   jko::StripStep<T> s{};
+  s.out = out;
+  s.init = fresh ? h->ctrl_init : nullptr;
+  s.record = record;
+  s.check = check;
+  s.renorm = h->prm.renormalize;
   s.op = strip_op(h);
   s.ek = h->ek;
-  s.q = (const T*)h->q;
-  s.q2 = h->attract ? (const T*)h->tgt : h->species == 2 ? (const T*)h->q + h->N : nullptr;
+  s.q = q_in;
+  s.q2 = h->attract ? (const T*)h->tgt : h->species == 2 ? q_in + h->N : nullptr;
   s.E1 = (const T*)h->E;
   s.E2 = (const T*)h->E2;
   s.t = h->pair_alpha > 0 ? h->prm.tau * h->pair_alpha : h->prm.tau;
   s.a = (T*)h->a;
   s.a2 = (T*)h->a2;
-  s.p = (T*)h->p;
   return jko::strip_launch<T>(h->strip, h->grid.nx, h->grid.ny, h->rx, h->ry, (const T*)h->taps_x,
                               (const T*)h->taps_y, s, jko::prox_args<T>(h), h->ctrl,
-                              h->strip_words, pairs, st);
+                              h->strip_words, h->prm.max_iter + 1, st);
 }
 
 template <typename T>
@@ -541,11 +548,9 @@ cudaError_t enqueue_heat_tiles(jko_handle* h, int pairs, cudaStream_t st) {
 }
 
 // `pairs` pairs as one persistent launch: the tensor-core loop kernel, the
-// heat kernel's persistent form or the CUDA-core filter's.
+// heat kernel's persistent form.
 cudaError_t enqueue_loop(jko_handle* h, int pairs, cudaStream_t st) {
   if (h->tc) return jko::tc_enqueue_loop(h->tc, pairs, st);
-  if (!h->heat_L)
-    return h->fp64 ? enqueue_strip<double>(h, pairs, st) : enqueue_strip<float>(h, pairs, st);
   if (h->htile.G > 0)
     return h->fp64 ? enqueue_heat_tiles<double>(h, pairs, st) : enqueue_heat_tiles<float>(h, pairs, st);
   const int nx = h->grid.nx, ny = h->grid.ny;
@@ -562,6 +567,7 @@ cudaError_t enqueue_loop(jko_handle* h, int pairs, cudaStream_t st) {
 }
 
 jko_status capture_chunk(jko_handle* h) {
+  if (h->strip.G > 0) return JKO_OK;   // whole steps in one launch
   cudaGraph_t g = nullptr;
   CK(h, cudaStreamBeginCapture(h->cap, cudaStreamCaptureModeThreadLocal));
   cudaError_t e = cudaSuccess;
@@ -1020,7 +1026,7 @@ jko_status enqueue_step_begin(jko_handle* h, const T* q_in, cudaStream_t st) {
   CK(h, jko::launch_step_begin<T>(*h->ctrl_init, h->ctrl, h->chunk_ctr,
                                   (const void*)q_in != h->q ? q_in : nullptr, (T*)h->q, h->ns,
                                   plain ? (T*)h->a : nullptr, plain ? (long long)h->N : 0, st));
-  if (plain || h->strip.G > 0) return JKO_OK;   // strip.cu starts its scalings itself
+  if (plain) return JKO_OK;
   if (h->tc_multi) {
     if (h->pair_alpha > 0) CK(h, begin_pairwise<float>(h, st));
     else CK(h, begin_multi_tc(h, st));
@@ -1127,11 +1133,14 @@ jko_status step_impl(jko_handle* h, const T* q_in, T* p_out, jko_step_info* info
     return qs != JKO_OK ? qs : s;
   };
   CK(h, cudaEventRecord(h->ev0, st));
-  {
+  // strip.cu: the checks, the pairs and the finalisation in one launch (every caller has an
+  // output for it)
+  const bool whole = h->strip.G > 0;
+  if (!whole) {
     const jko_status sb = enqueue_step_begin<T>(h, q_in, st);   // resets the control block
     if (sb != JKO_OK) return sb;
   }
-  if (validate) {
+  if (validate && !whole) {
     CK(h, jko::launch_validate<T>(q_in, N, P, h->ctrl, st));
     if (h->species == 2) CK(h, jko::launch_validate<T>(q_in + N, N, P, h->ctrl, st));
   }
@@ -1212,8 +1221,18 @@ jko_status step_impl(jko_handle* h, const T* q_in, T* p_out, jko_step_info* info
     return JKO_OK;
   };
   int done = jko::RUNNING, it_tc = 0, it_end = 0, final_slot = -1, fin_slot = -1;
-  jko_status sr = run_chunks(false, h->last_iters, &done, &it_tc, &final_slot);
-  if (sr != JKO_OK) return q_check_after_error(sr);
+  jko_status sr = JKO_OK;
+  if (whole) {
+    h->kernels = 1;
+    CK(h, enqueue_strip<T>(h, q_in, p_out, validate ? 1 : 0, 1, nullptr, st));
+    CK(h, cudaEventRecord(h->ev1, st));
+    CK(h, cudaMemcpyAsync(h->poll, h->ctrl, sizeof(Ctrl), cudaMemcpyDeviceToHost, st));
+    CK(h, cudaStreamSynchronize(st));
+    final_slot = 0;
+  } else {
+    sr = run_chunks(false, h->last_iters, &done, &it_tc, &final_slot);
+    if (sr != JKO_OK) return q_check_after_error(sr);
+  }
   bool finished = false;
   if (done == jko::STALLED && h->prm.finish && h->tc) {
     // the tensor-core operands have reached their rounding floor: continue the
@@ -1364,6 +1383,12 @@ jko_status flow_impl(jko_handle* h, const T* p0, int n_steps, T* traj, T* p_fina
       // kernels only: the step's start, its chunk loop, the finalisation
       // (which also records the control block), no copy between them
       CK(h, cudaEventRecord(h->flow_ev[2 * t], st));
+      if (h->strip.G > 0) {   // the whole step in one launch
+        CK(h, enqueue_strip<T>(h, q, out, 0, 1, h->flow_ctrl_dev + t, st));
+        CK(h, cudaEventRecord(h->flow_ev[2 * t + 1], st));
+        q = out;
+        continue;
+      }
       jko_status sb = enqueue_step_begin<T>(h, q, st);
       if (sb != JKO_OK) return sb;
       // a persistent kernel ends the step by itself: no loop around it
@@ -1402,7 +1427,8 @@ jko_status flow_impl(jko_handle* h, const T* p0, int n_steps, T* traj, T* p_fina
         // the last one completed) and their loop conditions, the finalisation
         const long long chunks =
             h->use_loop ? 1 : (c.it + 1 + h->chunk_iters - 1) / h->chunk_iters;
-        info.kernels = (int)(1 + chunks * (per_chunk + (h->use_loop ? 0 : 1)) + 2);
+        info.kernels = h->strip.G > 0
+                           ? 1 : (int)(1 + chunks * (per_chunk + (h->use_loop ? 0 : 1)) + 2);
         info.iters_finish = 0;
       }
       if (sk == JKO_ERR_NUMERIC) set_err(h, sk, "NaN or Inf in the scaling iterates");
@@ -1872,6 +1898,11 @@ struct jko_batch {
   std::vector<cudaStream_t> cap;     // cap[0] is the capture root
   std::vector<cudaEvent_t> ev;       // fork / join events
   cudaGraphExec_t g_pro = nullptr, g_chunk = nullptr, g_fin = nullptr;
+  cudaGraphExec_t g_first = nullptr, g_step = nullptr;   // every flow on strips: a whole step
+  jko::CopyItem* copy_host = nullptr;  // pinned / device: the images copied in and out
+  jko::CopyItem* copy_dev = nullptr;
+  Ctrl* host_steps = nullptr;          // pinned: the control blocks of every step
+  int host_steps_cap = 0;
   int C = 16;
   int max_iter = 1;
   Ctrl** ctrl_ptrs = nullptr;        // device: control block of each flow
@@ -1912,6 +1943,11 @@ void free_batch(jko_batch* b) {
   if (b->g_pro) cudaGraphExecDestroy(b->g_pro);
   if (b->g_chunk) cudaGraphExecDestroy(b->g_chunk);
   if (b->g_fin) cudaGraphExecDestroy(b->g_fin);
+  if (b->g_first) cudaGraphExecDestroy(b->g_first);
+  if (b->g_step) cudaGraphExecDestroy(b->g_step);
+  if (b->copy_host) cudaFreeHost(b->copy_host);
+  if (b->copy_dev) cudaFree(b->copy_dev);
+  if (b->host_steps) cudaFreeHost(b->host_steps);
   for (auto s : b->cap) if (s) cudaStreamDestroy(s);
   for (auto e : b->ev) if (e) cudaEventDestroy(e);
   for (auto e : b->ev_poll) if (e) cudaEventDestroy(e);
@@ -1923,12 +1959,21 @@ void free_batch(jko_batch* b) {
   delete b;
 }
 
+// A flow whose step is one launch of strip.cu.
+bool on_strips(const jko_handle* h) { return h->use_loop && h->strip.G > 0; }
+
+// That launch inside the batch graphs: from h->q into h->q.
+cudaError_t flow_strip(jko_handle* h, int check, int fresh, cudaStream_t s) {
+  return h->fp64 ? enqueue_strip<double>(h, (const double*)h->q, (double*)h->q, check, fresh, nullptr, s)
+                 : enqueue_strip<float>(h, (const float*)h->q, (float*)h->q, check, fresh, nullptr, s);
+}
+
 // The start of a flow's step inside the batch graphs: the control block reset
 // and the cold start of its form (as enqueue_step_begin for a handle alone;
 // the step input is already in h->q).
 template <typename T>
 cudaError_t flow_begin_t(jko_handle* h, cudaStream_t s) {
-  if (h->use_loop && h->strip.G > 0) return cudaSuccess;   // strip.cu starts its scalings itself
+  if (on_strips(h)) return cudaSuccess;   // strip.cu starts its scalings itself
   if (h->pair_alpha > 0) return begin_pairwise<T>(h, s);
   if (h->species == 2) return begin_species<T>(h, s);
   if (h->attract) return begin_attraction<T>(h, s);
@@ -1946,6 +1991,7 @@ cudaError_t flow_prologue(jko_handle* h, cudaStream_t s) {
 cudaError_t flow_chunk(jko_handle* h, int C, bool per_pass, cudaStream_t s, int loop_pairs = 0) {
   // a flow on the loop kernel: one launch runs its whole pair budget and stops
   // itself; later chunks of the step find it stopped and return at once
+  if (on_strips(h) && !per_pass) return flow_strip(h, 0, 0, s);
   if (h->use_loop && !per_pass)
     return enqueue_loop(h, loop_pairs > 0 ? loop_pairs : h->chunk_iters, s);
   for (int i = 0; i < C; ++i) {
@@ -1957,6 +2003,7 @@ cudaError_t flow_chunk(jko_handle* h, int C, bool per_pass, cudaStream_t s, int 
 
 template <typename T>
 cudaError_t flow_finalize_t(jko_handle* h, cudaStream_t s) {
+  if (on_strips(h)) return cudaSuccess;   // strip.cu's launch has done it
   ProxArgs<T> P = jko::prox_args<T>(h);
   // h->ns: both densities of a two-species flow
   cudaError_t e = jko::launch_finalize_reduce<T>((const T*)h->p, h->ns, P, h->ctrl, h->part,
@@ -2135,23 +2182,103 @@ jko_status capture_batch(jko_batch* b, H head, F per_flow, G tail, cudaGraphExec
   return JKO_OK;
 }
 
+// The checks of a flow's p0, counted into its control block.
 template <typename T>
-jko_status check_input(jko_handle* h, const T* q, int flow, jko_batch* b) {
-  cudaStream_t st = h->stream;
+cudaError_t launch_input_check(jko_handle* h, const T* q, cudaStream_t st) {
   ProxArgs<T> P = jko::prox_args<T>(h);
-  BCK(b, cudaMemcpyAsync(h->ctrl, h->ctrl_init, sizeof(Ctrl), cudaMemcpyHostToDevice, st));
-  BCK(b, jko::launch_validate<T>(q, h->N, P, h->ctrl, st));
-  if (h->species == 2) BCK(b, jko::launch_validate<T>(q + h->N, h->N, P, h->ctrl, st));
-  BCK(b, cudaMemcpyAsync(h->poll, h->ctrl, sizeof(Ctrl), cudaMemcpyDeviceToHost, st));
-  BCK(b, cudaStreamSynchronize(st));
-  const Ctrl& c = h->poll[0];
-  if (c.q_bad || c.q_neg || std::fabs(c.q_sum - 1.0) > 1e-3 || c.q_masked || c.q_over) {
-    char buf[200];
-    snprintf(buf, sizeof buf, "flow %d: p0 must be finite, >= 0, sum to 1, vanish on the mask "
-                              "and stay below kappa", flow);
-    return batch_err(b, JKO_ERR_INVALID_ARG, buf);
+  cudaError_t e = cudaMemcpyAsync(h->ctrl, h->ctrl_init, sizeof(Ctrl), cudaMemcpyHostToDevice, st);
+  if (e == cudaSuccess) e = jko::launch_validate<T>(q, h->N, P, h->ctrl, st);
+  if (e == cudaSuccess && h->species == 2)
+    e = jko::launch_validate<T>(q + h->N, h->N, P, h->ctrl, st);
+  return e;
+}
+
+// ... and their outcome for all flows, the first invalid one reported.
+jko_status check_inputs(jko_batch* b, const Ctrl* cs) {
+  for (int f = 0; f < b->n; ++f) {
+    const Ctrl& c = cs[f];
+    if (c.q_bad || c.q_neg || std::fabs(c.q_sum - 1.0) > 1e-3 || c.q_masked || c.q_over) {
+      char buf[200];
+      snprintf(buf, sizeof buf, "flow %d: p0 must be finite, >= 0, sum to 1, vanish on the mask "
+                                "and stay below kappa", f);
+      return batch_err(b, JKO_ERR_INVALID_ARG, buf);
+    }
   }
   return JKO_OK;
+}
+
+// The reports of step t from the flows' control blocks; the worst status, most pairs.
+int batch_report(jko_batch* b, const Ctrl* cs, int t, jko_step_info* infos) {
+  int worst = JKO_OK, max_it = 0;
+  for (int f = 0; f < b->n; ++f) {
+    const Ctrl& c = cs[f];
+    const jko_status sf = step_status(c);
+    worst = worse(worst, sf);
+    max_it = std::max(max_it, c.it);
+    if (infos) {
+      jko_step_info& in = infos[(size_t)t * b->n + f];
+      in.iters = c.it;
+      in.status = sf;
+      in.residual_l1 = c.res_last;
+      in.mass = c.mass;
+      double mx;
+      std::memcpy(&mx, &c.maxpk_bits, sizeof mx);
+      in.max_p_over_kappa = b->h[f]->has_kappa ? mx : 0.0;
+      in.ms = 0.f;
+      in.kernels = 0;
+    }
+  }
+  b->last_iters = max_it;
+  return worst;
+}
+
+// n image copies in one launch.
+cudaError_t batch_copy(jko_batch* b, int first, int n, cudaStream_t st) {
+  if (n == 0) return cudaSuccess;
+  cudaError_t e = cudaMemcpyAsync(b->copy_dev + first, b->copy_host + first, sizeof(jko::CopyItem) * n,
+                                  cudaMemcpyHostToDevice, st);
+  return e == cudaSuccess ? jko::launch_copies(b->copy_dev + first, n, st) : e;
+}
+
+// A flow of a batch whose every step is one launch per flow (g_first, g_step): the steps
+// follow each other on the device, the host reads all control blocks once.
+jko_status batch_flow_strips(jko_batch* b, const void* const* p0_dev, int n_steps,
+                             void* const* p_final_dev, jko_step_info* infos) {
+  cudaStream_t st = b->stream;
+  const int n = b->n;
+  if (b->host_steps_cap < n_steps) {
+    if (b->host_steps) cudaFreeHost(b->host_steps);
+    b->host_steps = nullptr;
+    b->host_steps_cap = 0;
+    const int cap = std::max(n_steps, 16);
+    BCK(b, cudaMallocHost((void**)&b->host_steps, sizeof(Ctrl) * (size_t)n * cap));
+    b->host_steps_cap = cap;
+  }
+  for (int f = 0; f < n; ++f)
+    b->copy_host[f] = {p0_dev[f], b->h[f]->q, (long long)(b->h[f]->es * b->h[f]->ns)};
+  BCK(b, batch_copy(b, 0, n, st));
+  for (int t = 0; t < n_steps; ++t) {
+    BCK(b, cudaGraphLaunch(t == 0 ? b->g_first : b->g_step, st));
+    BCK(b, cudaMemcpyAsync(b->host_steps + (size_t)t * n, b->ctrl_all, sizeof(Ctrl) * n,
+                           cudaMemcpyDeviceToHost, st));
+  }
+  BCK(b, cudaStreamSynchronize(st));
+  const jko_status sv = check_inputs(b, b->host_steps);
+  if (sv != JKO_OK) return sv;
+  int worst = JKO_OK;
+  for (int t = 0; t < n_steps; ++t) {
+    for (int f = 0; f < n; ++f)
+      if (b->host_steps[(size_t)t * n + f].nonfinite & 2)
+        return batch_err(b, JKO_ERR_TIMEOUT, "a bounded device-side wait gave up");
+    worst = worse(worst, batch_report(b, b->host_steps + (size_t)t * n, t, infos));
+  }
+  int m = 0;
+  for (int f = 0; p_final_dev && f < n; ++f)
+    if (p_final_dev[f])
+      b->copy_host[n + m++] = {b->h[f]->q, p_final_dev[f], (long long)(b->h[f]->es * b->h[f]->ns)};
+  BCK(b, batch_copy(b, n, m, st));
+  BCK(b, cudaStreamSynchronize(st));
+  return (jko_status)worst;
 }
 
 }  // namespace
@@ -2282,6 +2409,23 @@ jko_status jko_batch_create(int n_flows, const jko_grid* grids, const jko_params
   for (auto* h : b->h) all_loop = all_loop && h->use_loop;
   if (all_loop) b->C = b->max_iter + 1;
   b->all_loop = all_loop;
+  bool all_strips = all_loop;
+  for (auto* h : b->h) all_strips = all_strips && on_strips(h);
+  if (all_strips) {
+    // every step one graph of one launch per flow: no host decision between the steps
+    auto tail = [&](cudaStream_t root) {
+      return jko::launch_gather_ctrl(b->ctrl_ptrs, b->ctrl_all, b->n, root);
+    };
+    s = capture_batch(b, no_op, [](jko_handle* h, cudaStream_t st) { return flow_strip(h, 1, 1, st); },
+                      tail, &b->g_first);
+    if (s == JKO_OK)
+      s = capture_batch(b, no_op, [](jko_handle* h, cudaStream_t st) { return flow_strip(h, 0, 1, st); },
+                        tail, &b->g_step);
+    if (s != JKO_OK) return fail(s);
+    if (cudaMallocHost((void**)&b->copy_host, sizeof(jko::CopyItem) * 2 * n_flows) != cudaSuccess ||
+        cudaMalloc((void**)&b->copy_dev, sizeof(jko::CopyItem) * 2 * n_flows) != cudaSuccess)
+      return fail(batch_err(b, JKO_ERR_OOM, "batch allocation"));
+  }
   s = capture_batch(
       b, no_op, [](jko_handle* h, cudaStream_t st) { return flow_finalize(h, st); },
       [b](cudaStream_t root) { return jko::launch_gather_ctrl(b->ctrl_ptrs, b->ctrl_all, b->n, root); },
@@ -2317,10 +2461,18 @@ jko_status jko_batch_flow(jko_batch* b, const void* const* p0_dev, int n_steps,
     jko_handle* h = b->h[f];
     h->stream = st;
     if (!p0_dev[f]) return batch_err(b, JKO_ERR_INVALID_ARG, "NULL p0 entry");
-    jko_status s = h->fp64 ? check_input<double>(h, (const double*)p0_dev[f], f, b)
-                           : check_input<float>(h, (const float*)p0_dev[f], f, b);
-    if (s != JKO_OK) return s;
   }
+  if (b->g_step && n_steps > 0) return batch_flow_strips(b, p0_dev, n_steps, p_final_dev, infos);
+  for (int f = 0; f < b->n; ++f) {
+    jko_handle* h = b->h[f];
+    BCK(b, h->fp64 ? launch_input_check<double>(h, (const double*)p0_dev[f], st)
+                   : launch_input_check<float>(h, (const float*)p0_dev[f], st));
+  }
+  BCK(b, jko::launch_gather_ctrl(b->ctrl_ptrs, b->ctrl_all, b->n, st));
+  BCK(b, cudaMemcpyAsync(b->host_all, b->ctrl_all, sizeof(Ctrl) * b->n, cudaMemcpyDeviceToHost, st));
+  BCK(b, cudaStreamSynchronize(st));
+  const jko_status sv = check_inputs(b, b->host_all);
+  if (sv != JKO_OK) return sv;
   for (int f = 0; f < b->n; ++f)
     BCK(b, cudaMemcpyAsync(b->h[f]->q, p0_dev[f], b->h[f]->es * (size_t)b->h[f]->ns,
                            cudaMemcpyDeviceToDevice, st));
@@ -2358,29 +2510,7 @@ jko_status jko_batch_flow(jko_batch* b, const void* const* p0_dev, int n_steps,
     BCK(b, cudaGraphLaunch(b->g_fin, st));
     BCK(b, cudaMemcpyAsync(b->host_all, b->ctrl_all, sizeof(Ctrl) * n, cudaMemcpyDeviceToHost, st));
     BCK(b, cudaStreamSynchronize(st));
-    int max_it = 0;
-    for (int f = 0; f < n; ++f) {
-      const Ctrl& c = b->host_all[f];
-      jko_status sf = JKO_OK;
-      if (c.nonfinite & 2) sf = JKO_ERR_TIMEOUT;
-      else if (c.done == jko::NONFINITE || c.nonfinite) sf = JKO_ERR_NUMERIC;
-      else if (c.done == jko::MAX_ITER || c.done == jko::STALLED) sf = JKO_NOT_CONVERGED;
-      worst = worse(worst, sf);
-      max_it = std::max(max_it, c.it);
-      if (infos) {
-        jko_step_info& in = infos[(size_t)t * n + f];
-        in.iters = c.it;
-        in.status = sf;
-        in.residual_l1 = c.res_last;
-        in.mass = c.mass;
-        double mx;
-        std::memcpy(&mx, &c.maxpk_bits, sizeof mx);
-        in.max_p_over_kappa = b->h[f]->has_kappa ? mx : 0.0;
-        in.ms = 0.f;
-        in.kernels = 0;
-      }
-    }
-    b->last_iters = max_it;
+    worst = worse(worst, batch_report(b, b->host_all, t, infos));
   }
   if (p_final_dev)
     for (int f = 0; f < n; ++f)

@@ -92,7 +92,14 @@ struct StripStep {
   double t;            // attraction: tau; pairwise: tau alpha
   T* a;                // final scalings (a2: two couplings; pairwise: none written)
   T* a2;
-  T* p;
+  // the launch is the whole step: the control block set to *init first (NULL: as it is; a
+  // step that has stopped returns at once), the input's checks (check), mass and max p /
+  // kappa, p written to out (may be q; renormalised; untouched where a check failed), the
+  // control block copied to record
+  T* out;
+  const Ctrl* init;
+  Ctrl* record;
+  int check, renorm;
 };
 template <typename T>
 StripPlan strip_plan(int nx, int ny, int rx, int ry, int op, int ek, const ProxArgs<T>& P,
@@ -262,6 +269,13 @@ cudaError_t heat_tile_launch(const HeatTilePlan& tp, const HeatPlan& hp, const H
 // pair counter, the budget and the smallest residual carry over).
 cudaError_t launch_resume(Ctrl* ctrl, cudaStream_t st);
 cudaError_t launch_gather_done(Ctrl* const* ctrls, int* done, int n, cudaStream_t st);
+// n device-to-device copies in one launch (4-byte elements).
+struct CopyItem {
+  const void* src;
+  void* dst;
+  long long bytes;
+};
+cudaError_t launch_copies(const CopyItem* items, int n, cudaStream_t st);
 cudaError_t launch_gather_ctrl(Ctrl* const* ctrls, Ctrl* out, int n, cudaStream_t st);
 
 }  // namespace jko

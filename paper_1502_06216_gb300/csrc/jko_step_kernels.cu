@@ -232,6 +232,26 @@ cudaError_t launch_resume(Ctrl* ctrl, cudaStream_t st) {
   return cudaGetLastError();
 }
 
+namespace {
+__global__ void copies_kernel(const CopyItem* items) {
+  const CopyItem it = items[blockIdx.y];
+  const long long i0 = blockIdx.x * (long long)blockDim.x + threadIdx.x;
+  const long long step = (long long)gridDim.x * blockDim.x;
+  if ((((uintptr_t)it.src | (uintptr_t)it.dst | (uintptr_t)it.bytes) & 15) == 0) {
+    for (long long i = i0; i < it.bytes / 16; i += step) ((uint4*)it.dst)[i] = ((const uint4*)it.src)[i];
+  } else {
+    for (long long i = i0; i < it.bytes / 4; i += step)
+      ((uint32_t*)it.dst)[i] = ((const uint32_t*)it.src)[i];
+  }
+}
+}  // namespace
+
+cudaError_t launch_copies(const CopyItem* items, int n, cudaStream_t st) {
+  for (int i = 0; i < n; i += 65535)
+    copies_kernel<<<dim3(32, (unsigned)std::min(n - i, 65535)), NT, 0, st>>>(items + i);
+  return cudaGetLastError();
+}
+
 cudaError_t launch_gather_done(Ctrl* const* ctrls, int* done, int n, cudaStream_t st) {
   gather_done_kernel<<<(n + 127) / 128, 128, 0, st>>>(ctrls, done, n);
   return cudaGetLastError();

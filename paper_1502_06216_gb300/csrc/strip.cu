@@ -52,9 +52,16 @@ struct StripArgs {
   T t, kappa;                    // attraction: tau; pairwise: tau alpha; scalar bound (coupled)
   int has_kappa;
   T* a[2];
-  T* p;
   Ctrl* ctrl;
   int pairs;
+  // the control block starts as `init` (fresh), the input is checked (check), p goes to out,
+  // renormalised on request, the control block to record
+  T* out;
+  Ctrl* record;
+  int fresh, check, renorm;
+  unsigned long long* xfin;      // at the end: the blocks' max p / kappa and checks, 6 words each
+  unsigned long long* xsum;      // and the lines' masses, 2 words each
+  Ctrl init;
 };
 
 // The plain images of a block: by rows (q and the second marginal; pairwise: q_2,
@@ -94,13 +101,21 @@ strip_kernel(const __grid_constant__ StripArgs<T> A, const __grid_constant__ Pro
   auto col = [&](int k) { return (T*)(smem + S.col + k * S.col_b); };
   Ctrl* ctrl = A.ctrl;
   const int ncg = X.ncg, nrg = X.nrg;
-  const int done0 = *(volatile int*)&ctrl->done, bad0 = *(volatile int*)&ctrl->nonfinite;
-  if (done0 != RUNNING || bad0) {   // the same state for every block: none waits for this one
-    if (done0 == RUNNING && tid == 0 && blockIdx.x == 0) ctrl->done = NONFINITE;
-    return;
+  if (A.fresh) {
+    if (tid == 0 && blockIdx.x == 0) {
+      *ctrl = A.init;
+      __threadfence();   // before this block's words, so before any block's counts below
+    }
+  } else {
+    const int done0 = *(volatile int*)&ctrl->done, bad0 = *(volatile int*)&ctrl->nonfinite;
+    if (done0 != RUNNING || bad0) {   // the same state for every block: none waits for this one
+      if (done0 == RUNNING && tid == 0 && blockIdx.x == 0) ctrl->done = NONFINITE;
+      return;
+    }
   }
-  const int maxit = ctrl->max_iter, stall = ctrl->stall;
-  const double tol = ctrl->tol;
+  const int maxit = A.fresh ? A.init.max_iter : ctrl->max_iter;
+  const int stall = A.fresh ? A.init.stall : ctrl->stall;
+  const double tol = A.fresh ? A.init.tol : ctrl->tol;
   const unsigned ep0 = *(volatile unsigned*)A.g.epoch;
   if (tid == 0) {
     s_bad = 0;
@@ -336,26 +351,148 @@ strip_kernel(const __grid_constant__ StripArgs<T> A, const __grid_constant__ Pro
     if (OP == OP_PAIR) put_residual(ep);
   }
 
-  // the final a and p (p of the pair the last residual belongs to)
+  // the final a, and p of the pair the last residual belongs to: its mass and max p / kappa
+  // first (as finalize_reduce_kernel) and the input's checks (as validate_kernel),
+  // exchanged like the residuals, then p times 1 / mass (as finalize_write_kernel)
+  const size_t N = (size_t)nx * ny;
+  double inv = 1.0;
+  bool scale = false, keep = true;
+  {
+    __shared__ double s_fin[3][NT / 32], s_mass;
+    const unsigned epf = ep0 + 2u + (unsigned)pair;
+    // p line by line in one order (lanes, then their tree), so that the mass has the same
+    // bits however the lines are split over blocks
+    T mx = T(0);
+    auto line_sum = [&](const T* p, int n, const T* kap, int at) {
+      double sum = 0.0;
+      for (int i = lane; i < n; i += 32) {
+        sum += (double)p[i];
+        if (P.has_kappa) {
+          const T r = p[i] / (kap != nullptr ? kap[i] : P.kappa_s);
+          mx = r > mx ? r : mx;
+        }
+      }
+      sum = warp_sum(sum);
+      if (lane == 0) put_elem(A.xsum + 2 * (size_t)at, sum, epf);
+    };
+    for (int l = wid; l < ncg; l += nwarps) {
+      const T* kap = FIELDS && P.kappa != nullptr ? L.kappa + l * ny : nullptr;
+      line_sum(col(OP == OP_PAIR ? 2 : 0) + l * ny, ny, kap, X.x0 + l);
+      if (OP == OP_SPECIES) line_sum(col(1) + l * ny, ny, kap, nx + X.x0 + l);
+    }
+    if (OP == OP_PAIR)
+      for (int l = wid; l < nrg; l += nwarps) line_sum(row(2) + l * nx, nx, nullptr, nx + X.y0 + l);
+    double qsum = 0.0;
+    unsigned n_neg = 0, n_bad = 0, n_over = 0, n_msk = 0;
+    auto check_q = [&](T v, size_t at) {
+      if (!isfinite(v)) {
+        ++n_bad;
+        return;
+      }
+      qsum += (double)v;
+      if (v < T(0)) ++n_neg;
+      if (P.has_kappa && (double)v > (double)(P.kappa ? P.kappa[at] : P.kappa_s) * (1.0 + 1e-2))
+        ++n_over;
+      if (P.mask != nullptr && P.mask[at] && v != T(0)) ++n_msk;
+    };
+    if (A.check) {
+      for (int e = tid; e < nx * nrg; e += nthreads) {
+        check_q(row(0)[e], (size_t)X.y0 * nx + e);
+        if (OP == OP_SPECIES) check_q(row(1)[e], (size_t)X.y0 * nx + e);
+      }
+      if (OP == OP_PAIR)   // the first density by columns
+        for (int e = tid; e < ny * ncg; e += nthreads)
+          check_q(col(0)[e], (size_t)(e % ny) * nx + X.x0 + e / ny);
+      if (n_bad) atomicAdd(&ctrl->q_bad, (unsigned long long)n_bad);
+      if (n_neg) atomicAdd(&ctrl->q_neg, (unsigned long long)n_neg);
+      if (n_over) atomicAdd(&ctrl->q_over, (unsigned long long)n_over);
+      if (n_msk) atomicAdd(&ctrl->q_masked, (unsigned long long)n_msk);
+      qsum = warp_sum(qsum);
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) mx = fmax(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+    const bool viol = __any_sync(0xffffffffu, (n_neg | n_bad | n_over | n_msk) != 0);
+    if (lane == 0) {
+      s_fin[0][wid] = (double)mx;
+      s_fin[1][wid] = qsum;
+      s_fin[2][wid] = viol ? 1.0 : 0.0;
+    }
+    __syncthreads();
+    if (wid == 1) {
+      const int n = OP == OP_SPECIES ? 2 * nx : OP == OP_PAIR ? nx + ny : nx;
+      const double mass = gather_sum(A.xsum, n, epf, &s_fault);
+      if (lane == 0) s_mass = mass;
+    }
+    if (wid == 0) {
+      double v[3];
+#pragma unroll
+      for (int k = 0; k < 3; ++k) v[k] = lane < nwarps ? s_fin[k][lane] : 0.0;
+      auto all = [&]() {
+        v[1] = warp_sum(v[1]);
+        v[2] = warp_sum(v[2]);
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) v[0] = fmax(v[0], __shfl_xor_sync(0xffffffffu, v[0], o));
+      };
+      all();
+      // a block that gave up a wait says so by a negative count
+      if (s_fault) v[2] = -1e9;
+      if (lane < 3)
+        put_elem(A.xfin + 6 * (size_t)blockIdx.x + 2 * lane, lane == 0 ? v[0] : lane == 1 ? v[1] : v[2],
+                 epf);
+      v[0] = v[1] = v[2] = 0.0;
+      for (int g = lane; g < (int)gridDim.x; g += 32) {
+        const unsigned long long* w = A.xfin + 6 * (size_t)g;
+        unsigned long long lo[3], hi[3];
+#pragma unroll
+        for (int k = 0; k < 3; ++k) get_words(w + 2 * k, lo[k], hi[k]);
+#pragma unroll
+        for (int k = 0; k < 3; ++k) {
+          if (!wait_pair(w + 2 * k, epf, lo[k], hi[k], &s_fault)) s_fault = 1;
+          const double d = words_double(lo[k], hi[k]);
+          v[k] = k == 0 ? fmax(v[k], d) : v[k] + d;
+        }
+      }
+      all();
+      if (lane < 3) s_fin[lane][0] = lane == 0 ? v[0] : lane == 1 ? v[1] : v[2];
+    }
+    __syncthreads();
+    const double mass = s_mass;
+    if (s_fin[2][0] < 0.0 && tid == 0) s_fault = 1;
+    scale = A.renorm && mass > 0.0 && isfinite(mass);
+    inv = scale ? 1.0 / mass : 1.0;
+    // a step whose input failed its checks leaves the output untouched
+    keep = !A.check || (s_fin[2][0] == 0.0 && fabs(s_fin[1][0] - 1.0) <= 1e-3);
+    if (tid == 0 && blockIdx.x == 0) {
+      ctrl->mass = mass;
+      if (s_fin[0][0] > 0.0) ctrl->maxpk_bits = (unsigned long long)__double_as_longlong(s_fin[0][0]);
+      ctrl->q_sum = s_fin[1][0];
+      if (!isfinite(mass)) atomicOr(&ctrl->nonfinite, 1);
+      ++pair;   // the epoch of this exchange
+    }
+  }
+  auto put_p = [&](size_t at, T v) {
+    if (keep) A.out[at] = scale ? (T)((double)v * inv) : v;
+  };
   for (int e = tid; e < ny * ncg; e += nthreads) {
     const int y = e / ncg, xl = e - y * ncg;
     const size_t at = (size_t)y * nx + X.x0 + xl;
     if (OP == OP_PAIR) {
-      A.p[(size_t)nx * ny + at] = col(2)[xl * ny + y];
+      put_p(N + at, col(2)[xl * ny + y]);
     } else {
 #pragma unroll
       for (int m = 0; m < (NI < 2 ? NI : 2); ++m) A.a[m][at] = X.a[X.at_c(m, xl, y)];
-      A.p[at] = col(0)[xl * ny + y];
-      if (OP == OP_SPECIES) A.p[(size_t)nx * ny + at] = col(1)[xl * ny + y];
+      put_p(at, col(0)[xl * ny + y]);
+      if (OP == OP_SPECIES) put_p(N + at, col(1)[xl * ny + y]);
     }
   }
   if (OP == OP_PAIR)
-    for (int e = tid; e < nx * nrg; e += nthreads) A.p[(size_t)X.y0 * nx + e] = row(2)[e];
+    for (int e = tid; e < nx * nrg; e += nthreads) put_p((size_t)X.y0 * nx + e, row(2)[e]);
   if (tid == 0) {
     if (s_fault) atomicOr(&ctrl->nonfinite, 2);
     if (blockIdx.x == 0) {
       ctrl->it = it;
       *A.g.epoch = ep0 + 1u + (unsigned)pair;
+      if (A.record != nullptr) *A.record = *ctrl;
     }
   }
 }
@@ -446,7 +583,7 @@ StripPlan strip_plan(int nx, int ny, int rx, int ry, int op, int ek, const ProxA
   const size_t r2 = ((size_t)ni * ny * sp.nc * kw + 1) & ~(size_t)1;
   sp.x1_words = r1 * ceil_div(ny, sp.nr);
   sp.x2_words = r2 * ceil_div(nx, sp.nc);
-  sp.words = sp.x1_words + sp.x2_words + 4 * (size_t)sp.G + 2;
+  sp.words = sp.x1_words + sp.x2_words + 10 * (size_t)sp.G + 4 * (size_t)std::max(nx, ny) + 2;
   return sp;
 }
 
@@ -480,7 +617,11 @@ cudaError_t strip_launch(const StripPlan& sp, int nx, int ny, int rx, int ry, co
                          const T* taps_y, const StripStep<T>& s, const ProxArgs<T>& P, Ctrl* ctrl,
                          unsigned long long* words, int pairs, cudaStream_t st) {
   StripArgs<T> A{strip_geo(sp, nx, ny, rx, ry, taps_x, taps_y, words), s.q, s.q2, s.E1, s.E2,
-                 (T)s.t, P.kappa_s, P.has_kappa, {s.a, s.a2}, s.p, ctrl, pairs};
+                 (T)s.t, P.kappa_s, P.has_kappa, {s.a, s.a2}, ctrl, pairs, s.out, s.record,
+                 s.init != nullptr, s.check, s.renorm,
+                 words + sp.x1_words + sp.x2_words + 4 * (size_t)sp.G,
+                 words + sp.x1_words + sp.x2_words + 10 * (size_t)sp.G,
+                 s.init ? *s.init : Ctrl{}};
   ProxArgs<T> Pc = P;
   void* args[] = {&A, &Pc};
   return strip_coop(strip_fn<T>(sp.rb, s.op, s.ek), sp, sp.smem, sp.threads, args, st);
