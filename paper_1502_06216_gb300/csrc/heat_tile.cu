@@ -54,9 +54,6 @@ __host__ __device__ inline size_t heat_tile_bytes(int tw, int th, size_t es) {
   return box * 25 + (size_t)tw * th * es * 4;
 }
 
-// quotient of small non-negative integers (exact below 2^20)
-__device__ __forceinline__ int quot(int i, float inv) { return (int)(((float)i + 0.5f) * inv); }
-
 template <typename T, int EK>
 __global__ void __launch_bounds__(HTT)
 heat_tile_kernel(const __grid_constant__ HeatTileArgs<T> A, const __grid_constant__ ProxArgs<T> P) {

@@ -78,6 +78,7 @@ struct StripPlan {
   int G = 0;           // blocks (0: not available)
   int nc = 0, nr = 0;  // columns and rows per block
   int rb = 0;          // outputs per work item
+  int parts = 1;       // parts of an output's taps (FP64)
   int threads = 0;
   size_t smem = 0;
   size_t x1_words = 0, x2_words = 0, words = 0;   // exchange buffers, 8 bytes a word

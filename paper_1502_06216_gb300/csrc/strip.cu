@@ -95,7 +95,8 @@ strip_kernel(const __grid_constant__ StripArgs<T> A, const __grid_constant__ Pro
   int n_row, n_col;
   strip_images<T>(OP, EK, P, &n_row, &n_col);
   const bool has_mask = FIELDS && P.mask != nullptr;
-  const Smem S = smem_of<T>(nx, ny, A.g.rx, A.g.ry, A.g.nc, A.g.nr, NI, n_row, n_col, has_mask);
+  const Smem S = smem_of<T>(nx, ny, A.g.rx, A.g.ry, A.g.nc, A.g.nr, NI, A.g.parts, n_row, n_col,
+                            has_mask);
   Strips<T, NI, RB> X(A.g, S, smem, &s_fault);
   auto row = [&](int k) { return (T*)(smem + S.row + k * S.row_b); };
   auto col = [&](int k) { return (T*)(smem + S.col + k * S.col_b); };
@@ -183,8 +184,10 @@ strip_kernel(const __grid_constant__ StripArgs<T> A, const __grid_constant__ Pro
   const int n_res = OP == OP_PAIR ? A.g.gc : A.g.gr;
   auto put_residual = [&](unsigned ep) {
     unsigned long long* xr = A.g.xres + (size_t)(pair & 1) * n_res * 2;
-    if (wid == 0 && (int)blockIdx.x < n_res) {
-      const double v = warp_sum(lane < nwarps ? s_wres[lane] : 0.0);
+    if (wid == nwarps - 1 && (int)blockIdx.x < n_res) {   // the warp with the fewest items
+      double v = lane < nwarps ? s_wres[lane] : 0.0;   // at most 16 warps
+#pragma unroll
+      for (int o = 8; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
       if (lane == 0) put_elem(xr + 2 * blockIdx.x, s_bad ? (double)NAN : v, ep);
     }
   };
@@ -213,9 +216,7 @@ strip_kernel(const __grid_constant__ StripArgs<T> A, const __grid_constant__ Pro
     int bad = 0;
     if (!FROM_B || pair > 0) {
       // columns: T = K_y a
-      X.filter_cols_to(X.a, X.c2);
-      __syncthreads();
-      X.send_cols(ep);
+      X.filter_send_cols(ep);
       if (OP == OP_PAIR && pair > 0 && wid == nwarps - 1) decide(pair - 1, ep - 1u);
       X.receive_rows(ep);
       __syncthreads();
@@ -247,17 +248,14 @@ strip_kernel(const __grid_constant__ StripArgs<T> A, const __grid_constant__ Pro
         const bool have_prev = it > 0;
         T res = T(0);
         X.filter_rows(X.r2, [&](int m, int l, int i0, T (&acc)[RB]) {
-          const T* qm = row(m);
-#pragma unroll
-          for (int o = 0; o < RB; ++o) {
-            if (i0 + o >= nx) continue;
-            const T qv = qm[l * nx + i0 + o];
-            T* bp = X.b + X.at_r(m, l, i0 + o);
-            if (have_prev) res += abs_residual<T>(*bp, acc[o], qv);
-            const T bn = b_update<T>(qv, acc[o]);
+          X.each(acc, i0, nx, [&](int i, T v) {
+            const T qv = row(m)[l * nx + i];
+            T* bp = X.b + X.at_r(m, l, i);
+            if (have_prev) res += abs_residual<T>(*bp, v, qv);
+            const T bn = b_update<T>(qv, v);
             bad |= !dev_finite(bn);
             *bp = bn;
-          }
+          });
         });
         // the warps' residuals in the working precision, the block's and the grid's in FP64
         const double wres = warp_res(res);
@@ -268,9 +266,7 @@ strip_kernel(const __grid_constant__ StripArgs<T> A, const __grid_constant__ Pro
       if (OP != OP_PAIR) put_residual(ep);
     }
     // U = b K_x, rows -> columns
-    X.filter_rows_to(X.b, X.r2);
-    __syncthreads();
-    X.send_rows(ep);
+    X.filter_send_rows(ep);
     if (OP != OP_PAIR && (!FROM_B || pair > 0) && wid == nwarps - 1) decide(pair, ep);
     X.receive_cols(ep);
     __syncthreads();
@@ -280,15 +276,13 @@ strip_kernel(const __grid_constant__ StripArgs<T> A, const __grid_constant__ Pro
       // columns: s = K_y U, a = Prox(s) / s, p = a s
       T* s_p = col(0);
       X.filter_cols(X.c2, [&](int, int l, int i0, T (&acc)[RB]) {
-#pragma unroll
-        for (int o = 0; o < RB; ++o) {
-          if (i0 + o >= ny) continue;
-          const int idx = l * ny + i0 + o;
-          const T a = prox_ratio<T, EK>(L, idx, acc[o]);
+        X.each(acc, i0, ny, [&](int i, T v) {
+          const int idx = l * ny + i;
+          const T a = prox_ratio<T, EK>(L, idx, v);
           bad |= !dev_finite(a);
-          X.a[X.at_c(0, l, i0 + o)] = a;
-          s_p[idx] = a * acc[o];
-        }
+          X.a[X.at_c(0, l, i)] = a;
+          s_p[idx] = a * v;
+        });
       });
     } else if (OP == OP_PAIR) {
       // columns: y_m = xi a_m; the residual against the column constraints, p_2 = b_2 y_2,
@@ -562,10 +556,13 @@ StripPlan strip_plan(int nx, int ny, int rx, int ry, int op, int ek, const ProxA
     return ni * std::max(sp.nc * ceil_div(ny, rb), sp.nr * ceil_div(nx, rb));
   };
   sp.rb = sizeof(T) == 8 ? 1 : items(8) >= 256 ? 8 : 4;
-  sp.threads = std::min(512, std::max(256, ceil_div(items(sp.rb), 32) * 32));
+  // FP64: parts of an output's taps that give every scheduler two warps where the outputs
+  // do not (us a pair, one part / now: 64^2 19 / 13.3, 128^2 30 / 26)
+  while (sizeof(T) == 8 && sp.parts < 8 && items(1) * sp.parts < 256) sp.parts *= 2;
+  sp.threads = std::min(512, std::max(256, ceil_div(items(sp.rb) * sp.parts, 32) * 32));
   int rows = 0, cols = 0;
   strip_images<T>(op, ek, P, &rows, &cols);
-  const Smem S = smem_of<T>(nx, ny, rx, ry, sp.nc, sp.nr, ni, rows, cols, P.mask != nullptr);
+  const Smem S = smem_of<T>(nx, ny, rx, ry, sp.nc, sp.nr, ni, sp.parts, rows, cols, P.mask != nullptr);
   sp.smem = S.total;
   if (S.total + 1024 > (size_t)smem_max) return StripPlan{};
   void* fn = strip_fn<T>(sp.rb, op, ek);
@@ -587,10 +584,14 @@ StripPlan strip_plan(int nx, int ny, int rx, int ry, int op, int ek, const ProxA
   return sp;
 }
 
+// Taps of each of an output's parts, which cover the longest range of a line.
+static int part_len(int n, int r, int parts) { return ceil_div(std::min(2 * r + 1, n), parts); }
+
 strip::Geo strip_geo(const StripPlan& sp, int nx, int ny, int rx, int ry, const void* taps_x,
                      const void* taps_y, unsigned long long* words) {
   return Geo{nx, ny, rx, ry, sp.nc, sp.nr, ceil_div(ny, sp.nr), ceil_div(nx, sp.nc),
-             magic(sp.nc), magic(sp.nr), taps_x, taps_y, words, words + sp.x1_words,
+             magic(sp.nc), magic(sp.nr), sp.parts, part_len(ny, ry, sp.parts),
+             part_len(nx, rx, sp.parts), taps_x, taps_y, words, words + sp.x1_words,
              words + sp.x1_words + sp.x2_words, (unsigned*)(words + sp.words - 2)};
 }
 

@@ -126,28 +126,29 @@ __device__ __forceinline__ void line_taps(float (&acc)[RB], const float* line, i
     kb += 4 * 24;
   }
 }
-// FP64 (RB = 1): bound by the FP64 pipe (64 cycles a warp instruction and
-// scheduler); each lane runs its own taps inside the line, four per test.
-template <int RB>
-__device__ __forceinline__ void line_taps(double (&acc)[RB], const double* line, int pad,
-                                          const double* s_k, int n, int r, int i0) {
-  int t_lo = r - i0 - (RB - 1);
-  if (t_lo < 0) t_lo = 0;
+// FP64 (one output): bound by the FP64 pipe (64 cycles a warp instruction and
+// scheduler); each lane runs its own taps inside the line, four per test, those of part
+// `part` of its range (parts of len taps each).
+__device__ __forceinline__ void line_taps_part(double (&acc)[1], const double* line, int pad,
+                                               const double* s_k, int n, int r, int i0, int part,
+                                               int len) {
+  int t = r - i0;
+  if (t < 0) t = 0;
+  t += part * len;
   int t_hi = n - 1 - i0 + r;
   if (t_hi > 2 * r) t_hi = 2 * r;
+  if (t_hi > t + len - 1) t_hi = t + len - 1;
   const double* x = line + pad + i0 - r;
-  for (int t = t_lo; t <= t_hi; t += 4) {
-    double xx[4 + RB - 1], kk[4];
+  for (; t + 3 <= t_hi; t += 4) {
+    double xx[4], kk[4];
 #pragma unroll
-    for (int u = 0; u < 4 + RB - 1; ++u) xx[u] = x[t + u];
+    for (int u = 0; u < 4; ++u) xx[u] = x[t + u];
 #pragma unroll
     for (int u = 0; u < 4; ++u) kk[u] = s_k[t + u];
 #pragma unroll
-    for (int u = 0; u < 4; ++u) {
-#pragma unroll
-      for (int o = 0; o < RB; ++o) acc[o] = fma(kk[u], xx[u + o], acc[o]);
-    }
+    for (int u = 0; u < 4; ++u) acc[0] = fma(kk[u], xx[u], acc[0]);
   }
+  for (; t <= t_hi; ++t) acc[0] = fma(s_k[t], x[t], acc[0]);
 }
 
 // The warp's sum of the residual terms: a tree in the working precision (FP32
@@ -159,6 +160,8 @@ __device__ __forceinline__ double warp_res(double v) { return warp_sum(v); }
 __device__ __forceinline__ int div_by(int w, int d, unsigned m) {
   return d == 1 ? w : (int)__umulhi((unsigned)w, m);
 }
+// quotient of small non-negative integers (exact below 2^20)
+__device__ __forceinline__ int quot(int i, float inv) { return (int)(((float)i + 0.5f) * inv); }
 inline unsigned magic(int d) {
   return (unsigned)((0x100000000ull + (unsigned)d - 1) / (unsigned)d);
 }
@@ -168,6 +171,7 @@ inline int ceil_div(int a, int b) { return (a + b - 1) / b; }
 struct Geo {
   int nx, ny, rx, ry, nc, nr, gr, gc;   // gr, gc: blocks that own rows, columns
   unsigned mc, mr;                      // magic of nc, nr
+  int parts, len_c, len_r;              // FP64: parts of an output's taps, taps of each by axis
   const void* taps_x;
   const void* taps_y;
   unsigned long long* x1;        // columns -> rows
@@ -181,11 +185,11 @@ struct Geo {
 // and `cols` plain images of nr nx and nc ny elements, and the mask.
 struct Smem {
   int sc, sr;          // line strides of columns and rows
-  size_t kx, ky, a, c2, b, r2, row, col, row_b, col_b, mask, total;
+  size_t kx, ky, a, c2, b, r2, part, row, col, row_b, col_b, mask, total;
 };
 template <typename T>
 __host__ __device__ inline Smem smem_of(int nx, int ny, int rx, int ry, int nc, int nr, int ni,
-                                        int rows, int cols, bool mask) {
+                                        int parts, int rows, int cols, bool mask) {
   Smem S;
   S.sc = line_stride(ny, ry);
   S.sr = line_stride(nx, rx);
@@ -197,6 +201,7 @@ __host__ __device__ inline Smem smem_of(int nx, int ny, int rx, int ry, int nc, 
   S.c2 = take((size_t)ni * nc * S.sc);
   S.b = take((size_t)ni * nr * S.sr);
   S.r2 = take((size_t)ni * nr * S.sr);
+  S.part = take(parts > 1 ? (size_t)parts * ni * (nc * ny > nr * nx ? nc * ny : nr * nx) : 0);
   S.row_b = ((size_t)nr * nx * sizeof(T) + 255) / 256 * 256;
   S.col_b = ((size_t)nc * ny * sizeof(T) + 255) / 256 * 256;
   S.row = o;
@@ -213,7 +218,7 @@ struct Strips {
   const Geo& G;
   int x0, y0, ncg, nrg;          // columns [x0, x0 + ncg), rows [y0, y0 + nrg)
   int sc, sr, padc, padr;
-  T *kx, *ky, *a, *c2, *b, *r2;
+  T *kx, *ky, *a, *c2, *b, *r2, *part;
   int* fault;
 
   __device__ __forceinline__ Strips(const Geo& g, const Smem& S, unsigned char* smem, int* s_fault)
@@ -224,6 +229,7 @@ struct Strips {
     c2 = (T*)(smem + S.c2);
     b = (T*)(smem + S.b);
     r2 = (T*)(smem + S.r2);
+    part = (T*)(smem + S.part);
     x0 = blockIdx.x * g.nc;
     y0 = blockIdx.x * g.nr;
     ncg = max(0, min(g.nc, g.nx - x0));
@@ -250,28 +256,72 @@ struct Strips {
   }
 
   // The filter along the owned axis: RB outputs per work item,
-  // op(image, line, first output, outputs).
+  // op(image, line, first output, outputs).  FP64 where the outputs of a block are few
+  // warps: each output's taps in parts on different warps, added in order by a thread per
+  // output (the FP64 units of all four schedulers work).
   template <class F>
   __device__ __forceinline__ void filter(const T* src, int stride, int pad, int per, int lines,
-                                         int n, int r, const T* s_k, F&& op) {
-    const int nseg = (n + RB - 1) / RB;
-    for (int item = threadIdx.x; item < NI * lines * nseg; item += blockDim.x) {
-      const int ml = item / nseg, i0 = (item - ml * nseg) * RB;
-      const int m = NI == 1 ? 0 : ml / lines, l = NI == 1 ? ml : ml - m * lines;
-      T acc[RB];
+                                         int n, int r, int len, const T* s_k, F&& op) {
+    const int nseg = (n + RB - 1) / RB, items = NI * lines * nseg;
+    const float inv = 1.0f / (float)nseg;
+    auto line_of = [&](int ml, int& m, int& l) {
+      m = NI == 1 ? 0 : (ml >= lines) + (NI > 2 && ml >= 2 * lines);
+      l = NI == 1 ? ml : ml - m * lines;
+    };
+    if constexpr (RB == 1) {
+      const int parts = G.parts;
+      for (int f = threadIdx.x; f < parts * items; f += blockDim.x) {
+        const int q = parts == 1 ? 0 : f / items, item = f - q * items;
+        const int ml = quot(item, inv), i0 = item - ml * nseg;
+        int m, l;
+        line_of(ml, m, l);
+        T acc[1] = {T(0)};
+        line_taps_part(acc, src + (m * per + l) * stride, pad, s_k, n, r, i0, q, len);
+        if (parts == 1) op(m, l, i0, acc);
+        else part[f] = acc[0];
+      }
+      if (parts == 1) return;
+      __syncthreads();
+      for (int item = threadIdx.x; item < items; item += blockDim.x) {
+        const int ml = quot(item, inv), i0 = item - ml * nseg;
+        int m, l;
+        line_of(ml, m, l);
+        T acc[1] = {part[item]};
+        for (int q = 1; q < parts; ++q) acc[0] += part[q * items + item];
+        op(m, l, i0, acc);
+      }
+    } else {
+      for (int item = threadIdx.x; item < items; item += blockDim.x) {
+        const int ml = quot(item, inv), i0 = (item - ml * nseg) * RB;
+        int m, l;
+        line_of(ml, m, l);
+        T acc[RB];
 #pragma unroll
-      for (int o = 0; o < RB; ++o) acc[o] = T(0);
-      line_taps<RB>(acc, src + (m * per + l) * stride, pad, s_k, n, r, i0);
-      op(m, l, i0, acc);
+        for (int o = 0; o < RB; ++o) acc[o] = T(0);
+        line_taps<RB>(acc, src + (m * per + l) * stride, pad, s_k, n, r, i0);
+        op(m, l, i0, acc);
+      }
+    }
+  }
+  // f(i, value) for the outputs i0 .. of an item inside the line, one copy of f's code for
+  // all of them (the outputs shift through acc[0]): an epilogue runs once a pair, and
+  // unrolled it was bound by the instruction fetch.
+  template <class F>
+  static __device__ __forceinline__ void each(T (&acc)[RB], int i0, int n, F&& f) {
+#pragma unroll 1
+    for (int i = i0; i < min(i0 + RB, n); ++i) {
+      f(i, acc[0]);
+#pragma unroll
+      for (int o = 0; o + 1 < RB; ++o) acc[o] = acc[o + 1];
     }
   }
   template <class F>
   __device__ __forceinline__ void filter_cols(const T* src, F&& op) {
-    filter(src, sc, padc, G.nc, ncg, G.ny, G.ry, ky, op);
+    filter(src, sc, padc, G.nc, ncg, G.ny, G.ry, G.len_c, ky, op);
   }
   template <class F>
   __device__ __forceinline__ void filter_rows(const T* src, F&& op) {
-    filter(src, sr, padr, G.nr, nrg, G.nx, G.rx, kx, op);
+    filter(src, sr, padr, G.nr, nrg, G.nx, G.rx, G.len_r, kx, op);
   }
   // ... with the outputs into the lines of dst (what lies there has been sent or read)
   __device__ __forceinline__ void filter_cols_to(const T* src, T* dst) {
@@ -355,15 +405,42 @@ struct Strips {
       }
     }
   }
-  // c2 (columns) -> r2 (rows) and back
-  __device__ __forceinline__ void send_cols(unsigned ep) {
+  // K_y a on its way to the rows, b K_x on its way to the columns, through the lines of c2
+  // and r2 (whole segments per store); FP64's parts leave an output per thread, neighbours in
+  // order, which go straight out.
+  __device__ __forceinline__ void filter_send_cols(unsigned ep) {
+    if constexpr (RB == 1) {
+      if (G.parts > 1) {
+        const size_t region = ((size_t)NI * G.nx * G.nr * KW + 1) & ~(size_t)1;
+        filter_cols(a, [&](int m, int l, int i, T (&v)[RB]) {
+          const int g = div_by(i, G.nr, G.mr), il = i - g * G.nr;
+          put_elem(G.x1 + g * region + ((size_t)(m * G.nx + x0 + l) * G.nr + il) * KW, v[0], ep);
+        });
+        return;
+      }
+    }
+    filter_cols_to(a, c2);
+    __syncthreads();
     send(G.x1, c2, sc, padc, G.nc, x0, ncg, G.nx, G.ny, G.nr, G.mr, ep);
   }
+  __device__ __forceinline__ void filter_send_rows(unsigned ep) {
+    if constexpr (RB == 1) {
+      if (G.parts > 1) {
+        const size_t region = ((size_t)NI * G.ny * G.nc * KW + 1) & ~(size_t)1;
+        filter_rows(b, [&](int m, int l, int i, T (&v)[RB]) {
+          const int g = div_by(i, G.nc, G.mc), il = i - g * G.nc;
+          put_elem(G.x2 + g * region + ((size_t)(m * G.ny + y0 + l) * G.nc + il) * KW, v[0], ep);
+        });
+        return;
+      }
+    }
+    filter_rows_to(b, r2);
+    __syncthreads();
+    send(G.x2, r2, sr, padr, G.nr, y0, nrg, G.ny, G.nx, G.nc, G.mc, ep);
+  }
+  // ... into r2 (rows), into c2 (columns)
   __device__ __forceinline__ void receive_rows(unsigned ep) {
     receive(G.x1, r2, sr, padr, nrg, G.nx, G.nr, G.mr, ep);
-  }
-  __device__ __forceinline__ void send_rows(unsigned ep) {
-    send(G.x2, r2, sr, padr, G.nr, y0, nrg, G.ny, G.nx, G.nc, G.mc, ep);
   }
   __device__ __forceinline__ void receive_cols(unsigned ep) {
     receive(G.x2, c2, sc, padc, ncg, G.ny, G.nc, G.mc, ep);

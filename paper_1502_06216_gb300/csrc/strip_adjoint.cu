@@ -55,7 +55,7 @@ strip_adjoint_kernel(const __grid_constant__ AdjArgs<T> A, const __grid_constant
     if (tid == 0 && blockIdx.x == 0) A.out->bad = A.after->bad;
     return;
   }
-  const Smem S = smem_of<T>(nx, ny, A.g.rx, A.g.ry, A.g.nc, A.g.nr, 1, kAdjRows, kAdjCols, false);
+  const Smem S = smem_of<T>(nx, ny, A.g.rx, A.g.ry, A.g.nc, A.g.nr, 1, A.g.parts, kAdjRows, kAdjCols, false);
   Strips<T, 1, RB> X(A.g, S, smem, &s_fault);
   auto row = [&](int k) { return (T*)(smem + S.row + k * S.row_b); };
   auto col = [&](int k) { return (T*)(smem + S.col + k * S.col_b); };
@@ -77,26 +77,20 @@ strip_adjoint_kernel(const __grid_constant__ AdjArgs<T> A, const __grid_constant
   // the two halves of a round: a (columns) -> r2 (rows), b (rows) -> c2 (columns)
   auto to_rows = [&]() {
     ++ep;
-    X.filter_cols_to(X.a, X.c2);
-    __syncthreads();
-    X.send_cols(ep);
+    X.filter_send_cols(ep);
     X.receive_rows(ep);
     __syncthreads();
   };
   auto to_cols = [&]() {
     __syncthreads();
-    X.filter_rows_to(X.b, X.r2);
-    __syncthreads();
-    X.send_rows(ep);
+    X.filter_send_rows(ep);
     X.receive_cols(ep);
     __syncthreads();
   };
   // op(element of the plain images, element of the lines, value) over a filter's outputs
   auto rows_out = [&](auto&& op) {
     X.filter_rows(X.r2, [&](int, int l, int i0, T (&acc)[RB]) {
-#pragma unroll
-      for (int o = 0; o < RB; ++o)
-        if (i0 + o < nx) op(l * nx + i0 + o, X.at_r(0, l, i0 + o), acc[o]);
+      X.each(acc, i0, nx, [&](int i, T v) { op(l * nx + i, X.at_r(0, l, i), v); });
     });
   };
   // the sum of every block's v, the same everywhere; twice buffered as the residuals
@@ -131,13 +125,11 @@ strip_adjoint_kernel(const __grid_constant__ AdjArgs<T> A, const __grid_constant
   // the adjoint of the renormalisation p / sum p: <g, a s>
   double acc_d = 0.0;
   X.filter_cols(X.c2, [&](int, int l, int i0, T (&acc)[RB]) {
-#pragma unroll
-    for (int o = 0; o < RB; ++o) {
-      if (i0 + o >= ny) continue;
-      const int e = l * ny + i0 + o;
-      s_s[e] = acc[o];
-      acc_d += (double)s_ab[e] * (double)X.a[X.at_c(0, l, i0 + o)] * (double)acc[o];
-    }
+    X.each(acc, i0, ny, [&](int i, T s) {
+      const int e = l * ny + i;
+      s_s[e] = s;
+      acc_d += (double)s_ab[e] * (double)X.a[X.at_c(0, l, i)] * (double)s;
+    });
   });
   {
     const double dot = grid_sum(acc_d);
@@ -159,19 +151,17 @@ strip_adjoint_kernel(const __grid_constant__ AdjArgs<T> A, const __grid_constant
   to_cols();
   acc_d = 0.0;
   X.filter_cols(X.c2, [&](int, int l, int i0, T (&acc)[RB]) {
-#pragma unroll
-    for (int o = 0; o < RB; ++o) {
-      if (i0 + o >= ny) continue;
-      const int e = l * ny + i0 + o;
-      const T ab = s_s[e] * s_ab[e] - acc[o];
+    X.each(acc, i0, ny, [&](int i, T xv) {
+      const int e = l * ny + i;
+      const T ab = s_s[e] * s_ab[e] - xv;
       T rs, rw;
-      ratio_grad<T, EK>(P, (i0 + o) * nx + X.x0 + l, s_s[e], rs, rw);
+      ratio_grad<T, EK>(P, i * nx + X.x0 + l, s_s[e], rs, rw);
       s_ab[e] = ab;
       s_lam[e] = ab;
       s_rs[e] = rs;
-      X.a[X.at_c(0, l, i0 + o)] = rs * ab;
+      X.a[X.at_c(0, l, i)] = rs * ab;
       acc_d += fabs((double)ab);
-    }
+    });
   });
   const double norm = grid_sum(acc_d);
 
@@ -184,15 +174,21 @@ strip_adjoint_kernel(const __grid_constant__ AdjArgs<T> A, const __grid_constant
     rows_out([&](int e, int i, T z) { X.b[i] = s_D[e] * z; });
     to_cols();
     X.filter_cols(X.c2, [&](int, int l, int i0, T (&acc)[RB]) {
-      T diff = T(0);
+      T diff = T(0), u[RB];
+#pragma unroll
+      for (int o = 0; o < RB; ++o) {   // (all loads before the first store)
+        const int e = l * ny + i0 + o;
+        u[o] = T(0);
+        if (i0 + o >= ny) continue;
+        acc[o] = s_ab[e] - acc[o];
+        diff += fabs(acc[o] - s_lam[e]);
+        u[o] = s_rs[e] * acc[o];
+      }
 #pragma unroll
       for (int o = 0; o < RB; ++o) {
         if (i0 + o >= ny) continue;
-        const int e = l * ny + i0 + o;
-        const T ln = s_ab[e] - acc[o];
-        diff += fabs(ln - s_lam[e]);
-        s_lam[e] = ln;
-        X.a[X.at_c(0, l, i0 + o)] = s_rs[e] * ln;
+        s_lam[l * ny + i0 + o] = acc[o];
+        X.a[X.at_c(0, l, i0 + o)] = u[o];
       }
       acc_d += (double)diff;
     });
@@ -257,7 +253,7 @@ size_t strip_adjoint_smem(const StripPlan& sp, int nx, int ny, int rx, int ry) {
   int dev = 0, smem_max = 0;
   if (sp.G == 0 || cudaGetDevice(&dev) != cudaSuccess) return 0;
   cudaDeviceGetAttribute(&smem_max, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
-  const Smem S = smem_of<T>(nx, ny, rx, ry, sp.nc, sp.nr, 1, kAdjRows, kAdjCols, false);
+  const Smem S = smem_of<T>(nx, ny, rx, ry, sp.nc, sp.nr, 1, sp.parts, kAdjRows, kAdjCols, false);
   return S.total + 1024 <= (size_t)smem_max ? S.total : 0;
 }
 
