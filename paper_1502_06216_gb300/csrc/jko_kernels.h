@@ -72,7 +72,8 @@ cudaError_t simt_pass(int epi, int ek, const PassArgs<T>& A, const ProxArgs<T>& 
 // Persistent CUDA-core form of a step (strip.cu): one cooperative launch of G
 // blocks, each owning nc columns and nr rows of the images in shared memory.
 // strip_plan: G = 0 where the kernels per pass are the faster form or the strips do
-// not fit; max_blocks > 0: at most that many blocks.
+// not fit; max_blocks > 0: at most that many blocks, an output's taps in `parts` parts (those
+// of the plan without a limit give its bits).
 enum : int { OP_ONE = 0, OP_ATTRACT = 1, OP_SPECIES = 2, OP_PAIR = 3 };   // couplings of a step
 struct StripPlan {
   int G = 0;           // blocks (0: not available)
@@ -104,7 +105,7 @@ struct StripStep {
 };
 template <typename T>
 StripPlan strip_plan(int nx, int ny, int rx, int ry, int op, int ek, const ProxArgs<T>& P,
-                     int max_blocks);
+                     int max_blocks, int parts);
 // words: sp.words 8-byte words, zeroed once before the first launch (the epochs
 // of the exchanges go on from launch to launch).
 template <typename T>

@@ -533,7 +533,7 @@ void* strip_fn<double>(int, int op, int ek) { return strip_fn_op<double, 1, 512>
 // short work anyway.
 template <typename T>
 StripPlan strip_plan(int nx, int ny, int rx, int ry, int op, int ek, const ProxArgs<T>& P,
-                     int max_blocks) {
+                     int max_blocks, int parts) {
   StripPlan sp;
   const int ni = op_images(op);
   int dev = 0, coop = 0, sms = 0, smem_max = 0;
@@ -558,7 +558,8 @@ StripPlan strip_plan(int nx, int ny, int rx, int ry, int op, int ek, const ProxA
   sp.rb = sizeof(T) == 8 ? 1 : items(8) >= 256 ? 8 : 4;
   // FP64: parts of an output's taps that give every scheduler two warps where the outputs
   // do not (us a pair, one part / now: 64^2 19 / 13.3, 128^2 30 / 26)
-  while (sizeof(T) == 8 && sp.parts < 8 && items(1) * sp.parts < 256) sp.parts *= 2;
+  if (max_blocks > 0) sp.parts = parts;
+  else while (sizeof(T) == 8 && sp.parts < 8 && items(1) * sp.parts < 256) sp.parts *= 2;
   sp.threads = std::min(512, std::max(256, ceil_div(items(sp.rb) * sp.parts, 32) * 32));
   int rows = 0, cols = 0;
   strip_images<T>(op, ek, P, &rows, &cols);
@@ -629,7 +630,7 @@ cudaError_t strip_launch(const StripPlan& sp, int nx, int ny, int rx, int ry, co
 }
 
 #define JKO_STRIP_INST(T)                                                                        \
-  template StripPlan strip_plan<T>(int, int, int, int, int, int, const ProxArgs<T>&, int);      \
+  template StripPlan strip_plan<T>(int, int, int, int, int, int, const ProxArgs<T>&, int, int); \
   template cudaError_t strip_launch<T>(const StripPlan&, int, int, int, int, const T*, const T*, \
                                        const StripStep<T>&, const ProxArgs<T>&, Ctrl*,           \
                                        unsigned long long*, int, cudaStream_t);
