@@ -722,6 +722,7 @@ struct TcPlan {
   int loop_ok = 0;
   int loop_grid = 0;
   int loop_res = 0;            // the loop kernel keeps each CTA's factor band resident
+  int loop_wide = 0;         // loop kernel: units of two tiles (TF32)
   double loop_flops_pair = 0.0;
   // log-domain form (tc_log.cu, TF32): exponent per row and 32-cell group of
   // the images a, b ([ny][gx]) and T ([nx][gy]); -sigma w log2(e) as a

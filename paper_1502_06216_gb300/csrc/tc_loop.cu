@@ -67,28 +67,30 @@ __host__ __device__ constexpr uint32_t loop_epi_bytes(bool res) {
 __host__ __device__ constexpr uint32_t loop_res_bytes(bool res) {
   return res ? (uint32_t)RES_KB * BM * KB_BYTES : 0u;
 }
-__host__ __device__ constexpr uint32_t loop_stage_bytes(int mode, bool res) {
-  return res ? (img_split(mode) ? 2u : 1u) * (uint32_t)LBN * KB_BYTES : stage_bytes(mode, LBN);
+// w: 64-column tiles per unit (see the kernel)
+__host__ __device__ constexpr uint32_t loop_stage_bytes(int mode, bool res, int w = 1) {
+  return res ? (img_split(mode) ? 2u : 1u) * (uint32_t)LBN * KB_BYTES : stage_bytes(mode, LBN * w);
 }
-__host__ __device__ constexpr int loop_stages(int mode, bool res) {
+__host__ __device__ constexpr int loop_stages(int mode, bool res, int w = 1) {
   return res ? RES_STAGES
          : (LOOP_SMEM_BUDGET - loop_epi_bytes(false) - loop_staging_bytes(mode)) /
-                       stage_bytes(mode, LBN) <
+                       stage_bytes(mode, LBN * w) <
                    (uint32_t)MAX_STAGES
              ? (int)((LOOP_SMEM_BUDGET - loop_epi_bytes(false) - loop_staging_bytes(mode)) /
-                     stage_bytes(mode, LBN))
+                     stage_bytes(mode, LBN * w))
              : MAX_STAGES;
 }
-__host__ __device__ constexpr size_t loop_smem_bytes(int mode, bool res) {
-  return (size_t)loop_res_bytes(res) + (size_t)loop_stages(mode, res) * loop_stage_bytes(mode, res) +
+__host__ __device__ constexpr size_t loop_smem_bytes(int mode, bool res, int w = 1) {
+  return (size_t)loop_res_bytes(res) +
+         (size_t)loop_stages(mode, res, w) * loop_stage_bytes(mode, res, w) +
          loop_staging_bytes(mode) + loop_epi_bytes(res) + 1024 +
-         (size_t)(2 * loop_stages(mode, res) + 8) * 8 + 16;
+         (size_t)(2 * loop_stages(mode, res, w) + 8) * 8 + 16;
 }
 
 struct LoopPass {
   int M, N;          // output D is M x N (M along the contracted axis)
-  int tiles_n;       // tiles along N
-  int ntiles;        // tiles of the pass
+  int tiles_n;       // tiles (units of W tiles) along N
+  int ntiles;        // tiles (units) of the pass
   const int4* kbt;   // per 128-row tile: band of the factor (band_tile)
 };
 
@@ -127,7 +129,14 @@ __device__ __forceinline__ bool wait_go(const int* s_go, int q) {
   return false;
 }
 
-template <int MODE, int EK, bool RES>
+// W = 2 (TF32): a unit of two neighbouring 64-column tiles.  Its K-blocks are the
+// factor's block once and the images' 128 rows, one MMA of N = 128; the epilogue
+// takes the two halves one after the other through the same staging tiles.  A pass
+// over a large grid is bound by the bytes an SM receives from L2 (~60 GB/s): at
+// 2048^2 (band 271) a 64-wide tile streams 342 KB of factor and 171 KB of image, a
+// unit 342 + 342 KB for two.  Sums per output are unchanged, and so are the bits.
+// 2048^2 TF32: 29.4 us a pass with tiles, 22.2 with units.
+template <int MODE, int EK, bool RES, int W>
 __global__ void __launch_bounds__(NTL, 1)
 tc_loop_kernel(const __grid_constant__ LoopMaps maps, const __grid_constant__ LoopArgs args) {
   // EK_CROWD_PLAIN: the congestion/potential kind with a scalar bound and no
@@ -139,8 +148,10 @@ tc_loop_kernel(const __grid_constant__ LoopMaps maps, const __grid_constant__ Lo
   constexpr int NSPLIT = img_split(MODE) ? 2 : 1;         // image hi (+ lo) blocks
   constexpr uint32_t A_BYTES = BM * KB_BYTES;
   constexpr uint32_t B_BYTES = LBN * KB_BYTES;
-  constexpr uint32_t STAGE_BYTES = loop_stage_bytes(MODE, RES);
-  constexpr int STAGES = loop_stages(MODE, RES);
+  static_assert(W == 1 || (MODE == MODE_TF32 && !RES), "wide units: TF32");
+  constexpr int TBN = W * LBN;                            // columns of a unit
+  constexpr uint32_t STAGE_BYTES = loop_stage_bytes(MODE, RES, W);
+  constexpr int STAGES = loop_stages(MODE, RES, W);
   constexpr uint32_t B_OFF = RES ? 0u : A_BYTES;          // image blocks within a stage
   constexpr uint32_t ALO_OFF = A_BYTES + NSPLIT * B_BYTES; // factor lo (BF16X3)
   static_assert(STAGES >= 2, "at least two stages");
@@ -151,7 +162,7 @@ tc_loop_kernel(const __grid_constant__ LoopMaps maps, const __grid_constant__ Lo
   // TMEM columns BPREV_COL .. +63 beside the accumulator, for the next residual
   constexpr uint32_t BPREV_COL = 128;
   static_assert(!RES || acc_cols(MODE, LBN) <= BPREV_COL, "accumulator below the old b");
-  constexpr uint32_t TMEM_COLS = RES ? 256u : acc_cols(MODE, LBN);
+  constexpr uint32_t TMEM_COLS = RES ? 256u : acc_cols(MODE, TBN);
   constexpr int CB = LBN * (int)sizeof(T) / 128;   // 128-byte column blocks of an operand tile
   constexpr uint32_t OUT_BLOCK = BM * 128;
   static_assert((uint32_t)NSPLIT * CB * OUT_BLOCK <= STG_BYTES, "staging tile");
@@ -265,35 +276,46 @@ tc_loop_kernel(const __grid_constant__ LoopMaps maps, const __grid_constant__ Lo
         for (int t = blockIdx.x; t < PS.ntiles && ok; t += G) {
           const bool first = t == (int)blockIdx.x;
           const int mt = t / PS.tiles_n;
-          const int m0 = mt * BM, n0 = (t - mt * PS.tiles_n) * LBN;
+          const int m0 = mt * BM, n0 = (t - mt * PS.tiles_n) * TBN;
           const int4 kb = PS.kbt[mt];
-          if (epi_pass) {
+          // the epilogue tiles of the 64 columns from nn
+          auto epi_load = [&](int nn) -> bool {
             // resident mode: the staging region is free once the stores of
             // the previous pass have read it (one arrival before every grid
             // barrier, the q-th before barrier q)
-            if (RES) ok = mbar_wait(epi_free_bar, (uint32_t)(q - 1) & 1);
-            else if (ec > 0) ok = mbar_wait(epi_free_bar, (ec - 1) & 1);
-            if (!ok) break;
+            if (RES) {
+              if (!mbar_wait(epi_free_bar, (uint32_t)(q - 1) & 1)) return false;
+            } else if (ec > 0) {
+              if (!mbar_wait(epi_free_bar, (ec - 1) & 1)) return false;
+            }
             if (p == 1) {
               mbar_arrive_expect_tx(epi_full_bar, RES ? F32_TILE : EPI_B_LOAD);
 #pragma unroll
               for (int cb = 0; cb < LBN / 32; ++cb)
-                tma_load_2d(epi_f + cb * (BM * 128), &maps.Q, epi_full_bar, n0 + cb * 32, m0);
+                tma_load_2d(epi_f + cb * (BM * 128), &maps.Q, epi_full_bar, nn + cb * 32, m0);
               constexpr int KEO = 128 / (int)sizeof(T);
 #pragma unroll
               for (int cb = 0; cb < (RES ? 0 : CB); ++cb) {
-                tma_load_2d(epi_g + cb * OUT_BLOCK, &maps.O[1][0], epi_full_bar, n0 + cb * KEO, m0);
+                tma_load_2d(epi_g + cb * OUT_BLOCK, &maps.O[1][0], epi_full_bar, nn + cb * KEO, m0);
                 if constexpr (NSPLIT == 2)
                   tma_load_2d(epi_g + (CB + cb) * OUT_BLOCK, &maps.O[1][1], epi_full_bar,
-                              n0 + cb * KEO, m0);
+                              nn + cb * KEO, m0);
               }
             } else {
               mbar_arrive_expect_tx(epi_full_bar, EPI_A_LOAD);
 #pragma unroll
               for (int cb = 0; cb < LBN / 32; ++cb)
-                tma_load_2d(epi_f + cb * (BM * 128), &maps.E, epi_full_bar, n0 + cb * 32, m0);
+                tma_load_2d(epi_f + cb * (BM * 128), &maps.E, epi_full_bar, nn + cb * 32, m0);
             }
             ++ec;
+            return true;
+          };
+          // a later wide unit loads its tiles behind its first K-blocks: their region is
+          // busy until the previous unit's second half has been stored
+          const int epi_at = W == 1 || first ? -1 : (kb.y < STAGES ? kb.y : STAGES) - 1;
+          if (epi_pass && epi_at < 0) {
+            ok = epi_load(n0);
+            if (!ok) break;
             epi_pending = first;
           }
           if (first && q > 0) {
@@ -344,11 +366,15 @@ tc_loop_kernel(const __grid_constant__ LoopMaps maps, const __grid_constant__ Lo
               if constexpr (fac_split(MODE))
                 tma_load_2d(st + ALO_OFF, &maps.K[p][1], &full_bar[s], kx, m0);
             }
-            mbar_arrive_expect_tx(&full_bar[s], NSPLIT * B_BYTES);
+            mbar_arrive_expect_tx(&full_bar[s], NSPLIT * W * B_BYTES);
             tma_load_2d(st + B_OFF, &maps.B[p][0], &full_bar[s], kx, n0);
+            if constexpr (W == 2)   // (zeros beyond the image)
+              tma_load_2d(st + B_OFF + B_BYTES, &maps.B[p][0], &full_bar[s], kx, n0 + LBN);
             if constexpr (NSPLIT == 2)
               tma_load_2d(st + B_OFF + B_BYTES, &maps.B[p][1], &full_bar[s], kx, n0);
+            if (W == 2 && epi_pass && i == epi_at) ok = epi_load(n0);
           }
+          if (W == 2 && ok && epi_pass && n0 + LBN < PS.N) ok = epi_load(n0 + LBN);
           kc += kb.y;
         }
         if (ok && q > 0 && q < nq && (int)blockIdx.x >= PS.ntiles) {
@@ -389,7 +415,7 @@ tc_loop_kernel(const __grid_constant__ LoopMaps maps, const __grid_constant__ Lo
             const uint64_t b = sdesc_sw128(sa + B_OFF);
 #pragma unroll
             for (int kk = 0; kk < KB_BYTES / 32; ++kk)
-              umma_kstep<MODE, LBN>(tmem_base, a_hi, a_lo, b, kk, (i > 0 || kk > 0) ? 1u : 0u);
+              umma_kstep<MODE, TBN>(tmem_base, a_hi, a_lo, b, kk, (i > 0 || kk > 0) ? 1u : 0u);
             umma_commit(&empty_bar[s]);
           }
           umma_commit(accum_bar);
@@ -491,7 +517,10 @@ tc_loop_kernel(const __grid_constant__ LoopMaps maps, const __grid_constant__ Lo
       bool first = true;
       for (int t = blockIdx.x; t < PS.ntiles; t += G) {
         const int mt = t / PS.tiles_n;
-        const int m0 = mt * BM, n0 = (t - mt * PS.tiles_n) * LBN;
+        const int m0 = mt * BM, nu = (t - mt * PS.tiles_n) * TBN;
+        const int halves = W == 2 && nu + LBN < PS.N ? 2 : 1;
+        for (int hf = 0; hf < halves; ++hf) {
+        const int n0 = nu + hf * LBN;
         if (!first) {
           // the previous tile's stores must have read the staging and
           // epilogue tiles; the producer waits for that before it refills them
@@ -524,7 +553,7 @@ tc_loop_kernel(const __grid_constant__ LoopMaps maps, const __grid_constant__ Lo
             bprev_ok = true;
           }
         }
-        bool have = mbar_wait(accum_bar, tc & 1);
+        bool have = hf > 0 || mbar_wait(accum_bar, tc & 1);
         if (have && epi_pass) have = mbar_wait(epi_full_bar, ec & 1);
         if (!have && lane == 0) atomicOr(&s_fault, 1);
         __syncwarp();
@@ -533,11 +562,11 @@ tc_loop_kernel(const __grid_constant__ LoopMaps maps, const __grid_constant__ Lo
         // resident mode: the old b of the residual from TMEM
         const bool ld_old = RES && p == 1 && have_prev;
         const uint32_t t_old = tmem_base + ((uint32_t)(quad * 32) << 16) + BPREV_COL + (uint32_t)(grp * 16);
-        tmem_tile16<MODE, LBN>(tmem_base + ((uint32_t)(quad * 32) << 16), grp * 16, v);
+        tmem_tile16<MODE, LBN>(tmem_base + ((uint32_t)(quad * 32) << 16), hf * LBN + grp * 16, v);
         if (ld_old) tmem_wait_st();   // this thread's store of it, one pair ago
         tc_fence_before();
         __syncwarp();
-        if (lane == 0) mbar_arrive(tmem_free_bar);
+        if (lane == 0 && hf == halves - 1) mbar_arrive(tmem_free_bar);
         float res_f = 0.0f;
         if (p == 0 || p == 2) {
 #pragma unroll
@@ -674,7 +703,7 @@ tc_loop_kernel(const __grid_constant__ LoopMaps maps, const __grid_constant__ Lo
         else
           named_bar_sync(EPI_BAR, NEPI);
         if (threadIdx.x == 0) {
-          if (p == 1) args.part[t] = res;
+          if (p == 1) args.part[W == 1 ? t : mt * ((PS.N + LBN - 1) / LBN) + n0 / LBN] = res;
           constexpr int KEo = 128 / (int)sizeof(T);
 #pragma unroll
           for (int cb = 0; cb < CB; ++cb) {
@@ -693,8 +722,9 @@ tc_loop_kernel(const __grid_constant__ LoopMaps maps, const __grid_constant__ Lo
         // the producer refills before the next barrier
         free_pending = RES ? true : epi_pass;
         first = false;
-        ++tc;
         if (epi_pass) ++ec;
+        }
+        ++tc;
       }
       if (p == 3 && q == nq - 1) pairs_done = pair + 1;
     }
@@ -1238,66 +1268,66 @@ __global__ void __launch_bounds__(NTB, 1) tc_batch_kernel(const __grid_constant_
   }
 }
 
-template <int MODE, int EK, bool RES>
+template <int MODE, int EK, bool RES, int W>
 cudaError_t set_loop_attr() {
-  return cudaFuncSetAttribute(tc_loop_kernel<MODE, EK, RES>,
+  return cudaFuncSetAttribute(tc_loop_kernel<MODE, EK, RES, W>,
                               cudaFuncAttributeMaxDynamicSharedMemorySize,
-                              (int)loop_smem_bytes(MODE, RES));
+                              (int)loop_smem_bytes(MODE, RES, W));
 }
 
-template <int MODE, int EK, bool RES>
+template <int MODE, int EK, bool RES, int W>
 cudaError_t launch_loop(const LoopMaps& maps, const LoopArgs& args, int grid, cudaStream_t st) {
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(grid);
   cfg.blockDim = dim3(NTL);
-  cfg.dynamicSmemBytes = loop_smem_bytes(MODE, RES);
+  cfg.dynamicSmemBytes = loop_smem_bytes(MODE, RES, W);
   cfg.stream = st;
   cudaLaunchAttribute attr[1];
   attr[0].id = cudaLaunchAttributeCooperative;
   attr[0].val.cooperative = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, tc_loop_kernel<MODE, EK, RES>, maps, args);
+  return cudaLaunchKernelEx(&cfg, tc_loop_kernel<MODE, EK, RES, W>, maps, args);
 }
 
-template <int MODE, bool RES>
+template <int MODE, bool RES, int W = 1>
 cudaError_t dispatch_loop(int ek, const LoopMaps& maps, const LoopArgs& args, int grid,
                           cudaStream_t st) {
   const ProxArgs<float>& P = args.P;
   if (ek == EK_CROWD && P.mask == nullptr && P.kappa == nullptr && P.binary == 0)
-    return launch_loop<MODE, EK_CROWD_PLAIN, RES>(maps, args, grid, st);
-  if (ek == EK_CROWD) return launch_loop<MODE, EK_CROWD, RES>(maps, args, grid, st);
-  if (ek == EK_ENTROPY) return launch_loop<MODE, EK_ENTROPY, RES>(maps, args, grid, st);
-  return launch_loop<MODE, EK_POWER, RES>(maps, args, grid, st);
+    return launch_loop<MODE, EK_CROWD_PLAIN, RES, W>(maps, args, grid, st);
+  if (ek == EK_CROWD) return launch_loop<MODE, EK_CROWD, RES, W>(maps, args, grid, st);
+  if (ek == EK_ENTROPY) return launch_loop<MODE, EK_ENTROPY, RES, W>(maps, args, grid, st);
+  return launch_loop<MODE, EK_POWER, RES, W>(maps, args, grid, st);
 }
 
-template <int MODE, int EK, bool RES>
+template <int MODE, int EK, bool RES, int W>
 int blocks_per_sm() {
   int nb = 0;
-  if (set_loop_attr<MODE, EK, RES>() != cudaSuccess) return 0;
-  if (EK == EK_CROWD && set_loop_attr<MODE, EK_CROWD_PLAIN, RES>() != cudaSuccess) return 0;
-  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, tc_loop_kernel<MODE, EK, RES>, NTL,
-                                                    loop_smem_bytes(MODE, RES)) != cudaSuccess)
+  if (set_loop_attr<MODE, EK, RES, W>() != cudaSuccess) return 0;
+  if (EK == EK_CROWD && set_loop_attr<MODE, EK_CROWD_PLAIN, RES, W>() != cudaSuccess) return 0;
+  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, tc_loop_kernel<MODE, EK, RES, W>, NTL,
+                                                    loop_smem_bytes(MODE, RES, W)) != cudaSuccess)
     return 0;
   return nb;
 }
 
-template <int MODE, bool RES>
+template <int MODE, bool RES, int W = 1>
 int loop_blocks_per_sm(int ek) {
-  if (ek == EK_CROWD) return blocks_per_sm<MODE, EK_CROWD, RES>();
-  if (ek == EK_ENTROPY) return blocks_per_sm<MODE, EK_ENTROPY, RES>();
-  return blocks_per_sm<MODE, EK_POWER, RES>();
+  if (ek == EK_CROWD) return blocks_per_sm<MODE, EK_CROWD, RES, W>();
+  if (ek == EK_ENTROPY) return blocks_per_sm<MODE, EK_ENTROPY, RES, W>();
+  return blocks_per_sm<MODE, EK_POWER, RES, W>();
 }
 
-// Geometry of pass `which` (0..3) with 64-wide tiles.
-LoopPass loop_pass(const TcPlan* P, int which) {
+// Geometry of pass `which` (0..3) with 64-wide tiles, w of them per unit.
+LoopPass loop_pass(const TcPlan* P, int which, int w = 1) {
   const TcConfig& c = P->cfg;
   const bool over_x = (which & 1) == 0;
   const int side = P->absorbed ? (which >> 1) : 0;
   LoopPass L;
   L.M = over_x ? c.nx : c.ny;
   L.N = over_x ? c.ny : c.nx;
-  L.tiles_n = (L.N + LBN - 1) / LBN;
+  L.tiles_n = (L.N + w * LBN - 1) / (w * LBN);
   L.ntiles = L.tiles_n * ((L.M + BM - 1) / BM);
   L.kbt = P->kbt[over_x ? 0 : 1][side];
   return L;
@@ -1322,6 +1352,15 @@ int tc_loop_setup(TcPlan* P, std::string* msg) {
   int maxt = 0;
   for (int w = 0; w < 4; ++w) maxt = std::max(maxt, loop_pass(P, w).ntiles);
   P->loop_grid = std::min(maxt, sms * nb);
+  // units of two tiles (TF32) where they need fewer bytes of the CTA with the most: rounds
+  // of units at A + 2 B against rounds of tiles at A + B, A = 2 B
+  P->loop_wide = 0;
+  if (P->mode == MODE_TF32 && loop_blocks_per_sm<MODE_TF32, false, 2>(ek) >= 1) {
+    int maxu = 0;
+    for (int w = 0; w < 4; ++w) maxu = std::max(maxu, loop_pass(P, w, 2).ntiles);
+    auto rounds = [&](int n) { return (n + P->loop_grid - 1) / P->loop_grid; };
+    P->loop_wide = 4 * rounds(maxu) < 3 * rounds(maxt) ? 1 : 0;
+  }
   // resident factors: BF16, the same factor and band table in every pass
   // (square grid, equal lengths, no absorption), one tile per CTA and a band
   // of at most RES_KB K-blocks per 128-row tile
@@ -1394,18 +1433,20 @@ cudaError_t tc_enqueue_loop(TcPlan* P, int pairs, cudaStream_t st) {
   LoopMaps maps;
   loop_maps_of(P, &maps);
   LoopArgs args{};
-  for (int w = 0; w < 4; ++w) args.pass[w] = loop_pass(P, w);
+  for (int w = 0; w < 4; ++w) args.pass[w] = loop_pass(P, w, P->loop_wide ? 2 : 1);
   args.ctrl = c.ctrl;
   args.P = c.prox;
   args.part = c.part;
-  args.nparts = args.pass[1].ntiles;
+  args.nparts = loop_pass(P, 1).ntiles;   // one per 64-wide tile
   args.pairs = pairs;
   args.q = c.q;
   args.b_hi = P->img_b[0];
   args.b_lo = P->img_b[1];
   args.pitch_b = P->px;
   switch (P->mode) {
-    case MODE_TF32: return dispatch_loop<MODE_TF32, false>(c.ek, maps, args, P->loop_grid, st);
+    case MODE_TF32:
+      return P->loop_wide ? dispatch_loop<MODE_TF32, false, 2>(c.ek, maps, args, P->loop_grid, st)
+                          : dispatch_loop<MODE_TF32, false>(c.ek, maps, args, P->loop_grid, st);
     case MODE_BF16X3: return dispatch_loop<MODE_BF16X3, false>(c.ek, maps, args, P->loop_grid, st);
     default:
       return P->loop_res ? dispatch_loop<MODE_BF16, true>(c.ek, maps, args, P->loop_grid, st)
