@@ -753,7 +753,9 @@ jko_status jko_flow_record(jko_handle* h, const void* p0_dev, int n_steps, void*
   cudaStream_t st = h->stream;
   int worst = JKO_OK;
   const void* q = p0_dev;
-  for (int t = 0; t < n_steps; ++t) {
+  // on strips the first step alone waits (its input is checked), the others follow it
+  const int waits = h->strip.G > 0 ? 1 : n_steps;
+  for (int t = 0; t < waits; ++t) {
     char* slot = (char*)h->tape + es * N * per * t;
     if (q != (const void*)slot)  // from step 1 on the previous step wrote its output here
       ACK(cudaMemcpyAsync(slot, q, es * ns, cudaMemcpyDeviceToDevice, st));
@@ -775,6 +777,19 @@ jko_status jko_flow_record(jko_handle* h, const void* p0_dev, int n_steps, void*
     h->tape_mass[t] = info.mass;
     h->tape_steps = t + 1;
     q = dst;
+  }
+  if (waits < n_steps) {
+    void* last = p_final_dev;
+    if (!last) {
+      if (!h->stage_out) ACK(cudaMalloc(&h->stage_out, es * ns));
+      last = h->stage_out;
+    }
+    const jko_status s = jko::record_strip(h, h->tape, per, n_steps, last, infos,
+                                           h->tape_mass.data());
+    if (s == JKO_ERR_CUDA || s == JKO_ERR_OOM || s == JKO_ERR_TIMEOUT) return s;
+    h->tape_steps = n_steps;
+    if (s == JKO_ERR_NUMERIC) worst = JKO_ERR_NUMERIC;
+    else if (s == JKO_NOT_CONVERGED && worst == JKO_OK) worst = JKO_NOT_CONVERGED;
   }
   ACK(cudaStreamSynchronize(st));
   return (jko_status)worst;

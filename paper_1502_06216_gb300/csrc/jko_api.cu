@@ -519,7 +519,7 @@ int strip_op(const jko_handle* h) {
 // block itself.
 template <typename T>
 cudaError_t enqueue_strip(jko_handle* h, const T* q_in, T* out, int check, int fresh, Ctrl* record,
-                          cudaStream_t st) {
+                          cudaStream_t st, T* a = nullptr, T* a2 = nullptr) {
   jko::StripStep<T> s{};
   s.out = out;
   s.init = fresh ? h->ctrl_init : nullptr;
@@ -533,8 +533,8 @@ cudaError_t enqueue_strip(jko_handle* h, const T* q_in, T* out, int check, int f
   s.E1 = (const T*)h->E;
   s.E2 = (const T*)h->E2;
   s.t = h->pair_alpha > 0 ? h->prm.tau * h->pair_alpha : h->prm.tau;
-  s.a = (T*)h->a;
-  s.a2 = (T*)h->a2;
+  s.a = a ? a : (T*)h->a;
+  s.a2 = a2 ? a2 : (T*)h->a2;
   return jko::strip_launch<T>(h->strip, h->grid.nx, h->grid.ny, h->rx, h->ry, (const T*)h->taps_x,
                               (const T*)h->taps_y, s, jko::prox_args<T>(h), h->ctrl,
                               h->strip_words, h->prm.max_iter + 1, st);
@@ -1306,6 +1306,43 @@ jko_status jko::step_internal(jko_handle* h, const void* q_in, void* p_out, jko_
                  : step_impl<float>(h, (const float*)q_in, (float*)p_out, info, validate);
 }
 
+namespace {
+jko_status prepare_reports(jko_handle* h, int n_steps);
+jko_status report_steps(jko_handle* h, int t0, int n_steps, jko_step_info* infos, int* worst);
+
+// The steps 1 .. n_steps - 1 of a recorded flow on strips, enqueued before one wait: each
+// reads its slot of the tape and writes its scalings behind it.
+template <typename T>
+jko_status record_rest(jko_handle* h, T* tape, size_t per, int n_steps, T* last, jko_step_info* infos,
+                       double* mass) {
+  cudaStream_t st = h->stream;
+  const size_t N = (size_t)h->N, ns = (size_t)h->ns;
+  jko_status s = prepare_reports(h, n_steps);
+  if (s != JKO_OK) return s;
+  for (int t = 1; t < n_steps; ++t) {
+    T* slot = tape + per * N * t;
+    T* out = t + 1 < n_steps ? slot + per * N : last;
+    CK(h, cudaEventRecord(h->flow_ev[2 * t], st));
+    CK(h, enqueue_strip<T>(h, slot, out, 0, 1, h->flow_ctrl_dev + t, st, slot + ns, slot + ns + N));
+    CK(h, cudaEventRecord(h->flow_ev[2 * t + 1], st));
+  }
+  CK(h, cudaMemcpyAsync(h->flow_ctrl + 1, h->flow_ctrl_dev + 1, sizeof(Ctrl) * (size_t)(n_steps - 1),
+                        cudaMemcpyDeviceToHost, st));
+  CK(h, cudaStreamSynchronize(st));
+  int worst = JKO_OK;
+  s = report_steps(h, 1, n_steps, infos, &worst);
+  if (s != JKO_OK) return s;
+  for (int t = 1; t < n_steps; ++t) mass[t] = h->flow_ctrl[t].mass;
+  return (jko_status)worst;
+}
+}  // namespace
+
+jko_status jko::record_strip(jko_handle* h, void* tape, size_t per, int n_steps, void* last,
+                             jko_step_info* infos, double* mass) {
+  return h->fp64 ? record_rest<double>(h, (double*)tape, per, n_steps, (double*)last, infos, mass)
+                 : record_rest<float>(h, (float*)tape, per, n_steps, (float*)last, infos, mass);
+}
+
 jko_status jko::handle_error(jko_handle* h, jko_status st, const std::string& msg) {
   return set_err(h, st, msg);
 }
@@ -1315,6 +1352,69 @@ namespace {
 int worse(int a, int b) {
   auto rank = [](int s) { return s == JKO_OK ? 0 : (s == JKO_NOT_CONVERGED ? 1 : 2); };
   return rank(b) > rank(a) ? b : a;
+}
+
+// The control blocks and events of a flow whose steps are all enqueued before one wait.
+jko_status prepare_reports(jko_handle* h, int n_steps) {
+  if (h->flow_cap < n_steps) {
+    const int cap = std::max(n_steps, 64);
+    if (h->flow_ctrl) cudaFreeHost(h->flow_ctrl);
+    if (h->flow_ctrl_dev) cudaFree(h->flow_ctrl_dev);
+    h->flow_ctrl = nullptr;
+    h->flow_ctrl_dev = nullptr;
+    h->flow_cap = 0;
+    CK(h, cudaMallocHost((void**)&h->flow_ctrl, sizeof(Ctrl) * (size_t)cap));
+    CK(h, cudaMalloc((void**)&h->flow_ctrl_dev, sizeof(Ctrl) * (size_t)cap));
+    h->flow_cap = cap;
+  }
+  while ((int)h->flow_ev.size() < 2 * h->flow_cap) {
+    cudaEvent_t ev = nullptr;
+    CK(h, cudaEventCreate(&ev));
+    h->flow_ev.push_back(ev);
+  }
+  return JKO_OK;
+}
+
+// The reports of steps t0 .. n_steps - 1 from their control blocks (read back); an error
+// only for a wait that gave up.
+jko_status report_steps(jko_handle* h, int t0, int n_steps, jko_step_info* infos, int* worst_) {
+  int worst = *worst_;
+  const long long per_chunk = h->use_loop ? 1 : pair_kernels(h) * h->chunk_iters;
+  for (int k = t0; k < n_steps; ++k) {
+    const Ctrl& c = h->flow_ctrl[k];
+    const jko_status sk = step_status(c);
+    if (sk == JKO_ERR_TIMEOUT) return set_err(h, sk, "a bounded device-side wait gave up");
+    h->last_iters = c.it;
+    if (infos) {
+      jko_step_info& info = infos[k];
+      info = jko_step_info{};
+      info.iters = c.it;
+      info.status = sk;
+      info.residual_l1 = c.res_last;
+      info.mass = c.mass;
+      unsigned long long bits = c.maxpk_bits;
+      double mx;
+      std::memcpy(&mx, &bits, sizeof mx);
+      info.max_p_over_kappa = h->has_kappa ? mx : 0.0;
+      float ms = 0.f;
+      cudaEventElapsedTime(&ms, h->flow_ev[2 * k], h->flow_ev[2 * k + 1]);
+      info.ms = ms;
+      // the step's start, the chunks (the stop is decided in the pair after
+      // the last one completed) and their loop conditions, the finalisation
+      const long long chunks =
+          h->use_loop ? 1 : (c.it + 1 + h->chunk_iters - 1) / h->chunk_iters;
+      info.kernels = h->strip.G > 0
+                         ? 1 : (int)(1 + chunks * (per_chunk + (h->use_loop ? 0 : 1)) + 2);
+      info.iters_finish = 0;
+    }
+    if (sk == JKO_ERR_NUMERIC) set_err(h, sk, "NaN or Inf in the scaling iterates");
+    else if (sk == JKO_NOT_CONVERGED)
+      set_err(h, sk, c.done == jko::STALLED ? "the residual stalled above tol (stall rule)"
+                                            : "max_iter reached before tol");
+    worst = worse(worst, sk);
+  }
+  *worst_ = worst;
+  return JKO_OK;
 }
 
 template <typename T>
@@ -1347,21 +1447,9 @@ jko_status flow_impl(jko_handle* h, const T* p0, int n_steps, T* traj, T* p_fina
   if (!(h->prm.finish && h->tc)) {
     if (h->use_loop) h->step_loop_state = 1;
     else build_step_loop(h);
-    if (h->step_loop_state == 1 && h->flow_cap < n_steps) {
-      const int cap = std::max(n_steps, 64);
-      if (h->flow_ctrl) cudaFreeHost(h->flow_ctrl);
-      if (h->flow_ctrl_dev) cudaFree(h->flow_ctrl_dev);
-      h->flow_ctrl = nullptr;
-      h->flow_ctrl_dev = nullptr;
-      h->flow_cap = 0;
-      CK(h, cudaMallocHost((void**)&h->flow_ctrl, sizeof(Ctrl) * (size_t)cap));
-      CK(h, cudaMalloc((void**)&h->flow_ctrl_dev, sizeof(Ctrl) * (size_t)cap));
-      h->flow_cap = cap;
-    }
-    while (h->step_loop_state == 1 && (int)h->flow_ev.size() < 2 * h->flow_cap) {
-      cudaEvent_t ev = nullptr;
-      CK(h, cudaEventCreate(&ev));
-      h->flow_ev.push_back(ev);
+    if (h->step_loop_state == 1) {
+      const jko_status sp = prepare_reports(h, n_steps);
+      if (sp != JKO_OK) return sp;
     }
   }
   const bool device_loop = n_steps > 1 && h->step_loop_state == 1 && !(h->prm.finish && h->tc);
@@ -1408,40 +1496,8 @@ jko_status flow_impl(jko_handle* h, const T* p0, int n_steps, T* traj, T* p_fina
     CK(h, cudaMemcpyAsync(h->flow_ctrl + t0, h->flow_ctrl_dev + t0,
                           sizeof(Ctrl) * (size_t)(n_steps - t0), cudaMemcpyDeviceToHost, st));
     CK(h, cudaStreamSynchronize(st));
-    const long long per_chunk = h->use_loop ? 1 : pair_kernels(h) * h->chunk_iters;
-    for (int k = t0; k < n_steps; ++k) {
-      const Ctrl& c = h->flow_ctrl[k];
-      const jko_status sk = step_status(c);
-      if (sk == JKO_ERR_TIMEOUT) return set_err(h, sk, "a bounded device-side wait gave up");
-      h->last_iters = c.it;
-      if (infos) {
-        jko_step_info& info = infos[k];
-        info = jko_step_info{};
-        info.iters = c.it;
-        info.status = sk;
-        info.residual_l1 = c.res_last;
-        info.mass = c.mass;
-        unsigned long long bits = c.maxpk_bits;
-        double mx;
-        std::memcpy(&mx, &bits, sizeof mx);
-        info.max_p_over_kappa = h->has_kappa ? mx : 0.0;
-        float ms = 0.f;
-        cudaEventElapsedTime(&ms, h->flow_ev[2 * k], h->flow_ev[2 * k + 1]);
-        info.ms = ms;
-        // the step's start, the chunks (the stop is decided in the pair after
-        // the last one completed) and their loop conditions, the finalisation
-        const long long chunks =
-            h->use_loop ? 1 : (c.it + 1 + h->chunk_iters - 1) / h->chunk_iters;
-        info.kernels = h->strip.G > 0
-                           ? 1 : (int)(1 + chunks * (per_chunk + (h->use_loop ? 0 : 1)) + 2);
-        info.iters_finish = 0;
-      }
-      if (sk == JKO_ERR_NUMERIC) set_err(h, sk, "NaN or Inf in the scaling iterates");
-      else if (sk == JKO_NOT_CONVERGED)
-        set_err(h, sk, c.done == jko::STALLED ? "the residual stalled above tol (stall rule)"
-                                              : "max_iter reached before tol");
-      worst = worse(worst, sk);
-    }
+    const jko_status sr = report_steps(h, t0, n_steps, infos, &worst);
+    if (sr != JKO_OK) return sr;
   }
   if (p_final && n_steps > 0)
     CK(h, cudaMemcpyAsync(p_final, q, N * sizeof(T), cudaMemcpyDeviceToDevice, st));

@@ -139,6 +139,9 @@ inline ProxArgs<T> prox_args(const jko_handle* h) {
 jko_status step_internal(jko_handle* h, const void* q_in, void* p_out, jko_step_info* info,
                          bool validate);
 // Records an error message on the handle and returns the status.
+// Steps 1 .. n_steps - 1 of a recorded flow on strips (tape: per images a step).
+jko_status record_strip(jko_handle* h, void* tape, size_t per, int n_steps, void* last,
+                        jko_step_info* infos, double* mass);
 jko_status handle_error(jko_handle* h, jko_status st, const std::string& msg);
 // Argument checks of jko_create (sizes, parameters, energy fields): JKO_OK, or
 // the error status with *msg set to a static description.  Allocates nothing
