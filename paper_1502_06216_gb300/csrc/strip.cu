@@ -520,13 +520,25 @@ void* strip_fn<double>(int, int op, int ek) { return strip_fn_op<double, 1, 512>
 
 }  // namespace
 
+// The kernel's limit of dynamic shared memory: the same for every handle, so that none lowers
+// it under another's (or under a captured graph).  The plans leave 1 KB for static arrays.
+cudaError_t strip_cap(void* fn) {
+  int dev = 0, most = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e == cudaSuccess)
+    e = cudaDeviceGetAttribute(&most, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+  return e != cudaSuccess
+             ? e : cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, most - 1024);
+}
+
 // The rule for the persistent form, on the grid, the band and the precision.
-// Both sides measured on a GB300 (us a pair, this form / a kernel per pass, flows
-// to tol with their launches and finalisations): FP32 128^2 8.4 / 21.4, 201 x 149
-// 9.8 / 26, 256^2 10.8 / 26, 512^2 porous 42 / 56 (three pairs a step), 700^2
-// 31 / 52, 1024^2 64 / 81; FP64 128^2 36 / 111, 201 x 149 57 / 132, 256^2 162 /
-// 197, 512^2 1253 / 1124.  FP64 is bound by its pipe, so whole lines per block
-// (4 against 3.4 on average at 512^2) cost what the launches save: up to two
+// Both sides measured on a GB300 (us a pair, this form / a kernel per pass, 30 pairs a
+// step): crowd FP32 128^2 9.1 / 21.2, 256^2 10.5 / 25.2, 512^2 25 / 43, 600 x 200
+// 18 / 32, 800 x 64 15 / 31, 1024^2 62 / 81; FP64 128^2 27 / 102, 256^2 145 / 176,
+// 300^2 221 / 385.  Attraction FP32 256^2 17.9 / 35.8, 512^2 67 / 111, FP64 256^2
+// 292 / 350; two species and pairwise alike.  FP64 512^2 (four lines a block) was
+// 1253 / 1124: bound by its pipe, whole lines per block (4 against 3.4 on average)
+// cost what the launches save, so FP64 takes up to two
 // lines a block.  FP32: wherever the strips fit the shared memory of one block
 // per SM (about 1060 cells a side).  Long thin grids, whose short side has too
 // few lines for the blocks, keep the per-pass form unless a block's line is
@@ -568,8 +580,7 @@ StripPlan strip_plan(int nx, int ny, int rx, int ry, int op, int ek, const ProxA
   if (S.total + 1024 > (size_t)smem_max) return StripPlan{};
   void* fn = strip_fn<T>(sp.rb, op, ek);
   int per_sm = 0;
-  if (cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)S.total) !=
-          cudaSuccess ||
+  if (strip_cap(fn) != cudaSuccess ||
       cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, sp.threads, S.total) !=
           cudaSuccess ||
       per_sm * sms < sp.G) {
@@ -608,8 +619,7 @@ cudaError_t strip_coop(void* fn, const StripPlan& sp, size_t smem, int threads, 
   at[0].val.cooperative = 1;
   cfg.attrs = at;
   cfg.numAttrs = 1;
-  // another handle of the same kernel may have set a smaller limit
-  cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  const cudaError_t e = strip_cap(fn);
   if (e != cudaSuccess) return e;
   return cudaLaunchKernelExC(&cfg, fn, args);
 }
