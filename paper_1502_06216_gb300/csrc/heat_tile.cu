@@ -7,8 +7,9 @@
 // words {32 bits, epoch} (strip.cuh), polled by their readers, so there is no grid
 // barrier, and the interior never leaves the SM.  The words are twice buffered by
 // epoch parity: a block writes exchange e + 2 only after it has every
-// neighbour's e + 1, which they wrote after reading e ("neighbour" is symmetric:
-// within H cells).  The arithmetic of a cell and the stop rule are those of heat.cu's
+// neighbour's e + 1, which they wrote after reading e.  So every block that reads a block's
+// words has to be one it waits for: the blocks with a cell within H cells of its tile,
+// whatever the obstacles are (heat_geom.h).  The arithmetic of a cell and the stop rule are those of heat.cu's
 // kernels, so the iterates have the same bits; the residual is added by tiles.
 //
 // Bound by the exchange and by the FP64 latency of its steps (five operations a cell, four
@@ -20,6 +21,7 @@
 #include <algorithm>
 
 #include "heat_cell.cuh"
+#include "heat_geom.h"
 #include "jko_kernels.h"
 #include "strip.cuh"
 
@@ -30,7 +32,8 @@ namespace {
 using namespace strip;
 
 constexpr int HTT = 512;   // threads at most: work warps and one that takes the decision
-constexpr int H = 4;       // Clenshaw steps per exchange at most, and cells of the halo
+using heat_geom::FREE;
+using heat_geom::H;
 
 template <typename T>
 struct HeatTileArgs {
@@ -74,9 +77,8 @@ heat_tile_kernel(const __grid_constant__ HeatTileArgs<T> A, const __grid_constan
   unsigned ep = *(volatile unsigned*)A.epoch;
   const int nx = A.nx, ny = A.ny;
   const size_t N = (size_t)nx * ny;
-  const int by = blockIdx.x / A.ntx, bx = blockIdx.x - by * A.ntx;
-  const int x0 = bx * A.tw, y0 = by * A.th;
-  const int w = min(A.tw, nx - x0), h = min(A.th, ny - y0);
+  const heat_geom::Tile tile = heat_geom::tile_of(blockIdx.x, A.tw, A.th, A.ntx, nx, ny);
+  const int x0 = tile.x0, y0 = tile.y0, w = tile.w, h = tile.h;
   const int SX = A.tw + 2 * H, box = SX * (A.th + 2 * H);
   double* sv = (double*)smem;
   double* cur1 = sv + box;
@@ -91,17 +93,12 @@ heat_tile_kernel(const __grid_constant__ HeatTileArgs<T> A, const __grid_constan
     s_fault = 0;
     s_dec = 0;
   }
-  // free flags of a cell and its four neighbours; v = a = 1 (Sec. 3.4)
-  auto is_free = [&](int x, int y) {
-    return x >= 0 && x < nx && y >= 0 && y < ny &&
-           (A.mask == nullptr || A.mask[(size_t)y * nx + x] == 0);
-  };
+  // the cells' flags; v = a = 1 (Sec. 3.4)
   for (int c = tid; c < box; c += blockDim.x) {
     const int ey = c / SX, ex = c - ey * SX, x = x0 + ex - H, y = y0 + ey - H;
-    const bool f = is_free(x, y);
-    s_nb[c] = !f ? 0 : 1 | is_free(x - 1, y) << 1 | is_free(x + 1, y) << 2 | is_free(x, y - 1) << 3 |
-                           is_free(x, y + 1) << 4;
-    sv[c] = f ? 1.0 : 0.0;
+    const int f = heat_geom::cell_flags(x, y, nx, ny, A.mask);
+    s_nb[c] = (uint8_t)f;
+    sv[c] = f & FREE ? 1.0 : 0.0;
     cur1[c] = cur2[c] = 0.0;
   }
   for (int c = tid; c < w * h; c += blockDim.x) {
@@ -111,25 +108,15 @@ heat_tile_kernel(const __grid_constant__ HeatTileArgs<T> A, const __grid_constan
     s_b[c] = s_p[c] = T(0);
   }
   __syncthreads();
-  const int BX = w + 2 * H, ring_tb = 2 * H * BX, ring = ring_tb + 2 * H * h;
-  const float inv_bx = 1.0f / (float)BX, inv_2h = 1.0f / (float)(2 * H);
-  // cell i of the halo ring: its place in the box and in the grid, -1 where nothing is free
+  const int ring = heat_geom::ring_cells(tile);
+  const float inv_bx = 1.0f / (float)(w + 2 * H);
+  // cell i of the halo ring: its place in the box and in the grid, -1 outside the grid
   auto ring_cell = [&](int i, int& c) -> int {
     int ex, ey;
-    if (i < ring_tb) {
-      const int r = quot(i, inv_bx);
-      ex = i - r * BX;
-      ey = r < H ? r : h + r;
-    } else {
-      i -= ring_tb;
-      const int r = quot(i, inv_2h), col = i - r * 2 * H;
-      ex = col < H ? col : w + col;
-      ey = H + r;
-    }
+    heat_geom::ring_place(i, tile, inv_bx, ex, ey);
     c = ey * SX + ex;
-    return (s_nb[c] & 1) ? (y0 + ey - H) * nx + x0 + ex - H : -1;
+    return heat_geom::awaited(s_nb[c]) ? (y0 + ey - H) * nx + x0 + ex - H : -1;
   };
-  auto edge = [&](int x, int y) { return x < H || x >= w - H || y < H || y >= h - H; };
 
   // the cell a work thread takes in a step on the tile and an e-cell halo, where every
   // step has a thread per cell (else the steps loop over cells)
@@ -154,7 +141,7 @@ heat_tile_kernel(const __grid_constant__ HeatTileArgs<T> A, const __grid_constan
         const float inv_w = 1.0f / (float)w;
         for (int i = tid; i < w * h; i += nwork) {
           const int y = quot(i, inv_w), x = i - y * w, c = (y + H) * SX + x + H;
-          if (edge(x, y) && (s_nb[c] & 1))
+          if (heat_geom::sent(x, y, tile))
             put_elem(xv + 2 * ((size_t)(y0 + y) * nx + x0 + x), sv[c], ep);
         }
         for (int i = tid; i < ring; i += nwork) {
@@ -213,18 +200,19 @@ heat_tile_kernel(const __grid_constant__ HeatTileArgs<T> A, const __grid_constan
         const int f = s_nb[c];
         const double bc = cur1[c], b2 = cur2[c];
         const double bl = cur1[c - 1], br = cur1[c + 1], bu = cur1[c - SX], bd = cur1[c + SX];
-        const double r = cl_value(ck, v, b2, s * A.ax, s * A.ay, f & 2 ? bl : bc, f & 4 ? br : bc,
-                                  f & 8 ? bu : bc, f & 16 ? bd : bc);
-        return f ? r : 0.0;
+        const double r = cl_value(ck, v, b2, s * A.ax, s * A.ay, f & heat_geom::LEFT ? bl : bc,
+                                  f & heat_geom::RIGHT ? br : bc, f & heat_geom::UP ? bu : bc,
+                                  f & heat_geom::DOWN ? bd : bc);
+        return f & FREE ? r : 0.0;
       };
       // the last step of a phase at cell i = (x, y) of the tile: to the neighbours, or closed
       // into the b-update or the prox
       auto finish = [&](int i, int x, int y, int c, int kk, double r) {
-        const bool f = s_nb[c] & 1;
+        const bool f = s_nb[c] & FREE;
         if (kk > 0) {
           const double bc = cur1[c];
           cur2[c] = r;
-          if (f && edge(x, y)) {
+          if (heat_geom::sent(x, y, tile)) {
             unsigned long long* x4 = A.xb + (size_t)((ep + 1) & 1) * N * 4 +
                                      4 * ((size_t)(y0 + y) * nx + x0 + x);
             put_elem(x4, r, ep + 1);
@@ -369,13 +357,6 @@ void* heat_tile_fn(int ek) {
   return (void*)heat_tile_kernel<T, EK_POWER>;
 }
 
-// Work of a phase of H steps on a w x h tile, in warps.
-long long phase_warps(int w, int h) {
-  long long s = 0;
-  for (int e = 0; e < H; ++e) s += ((long long)(w + 2 * e) * (h + 2 * e) + 31) / 32;
-  return s;
-}
-
 }  // namespace
 
 // One tile per block and at most one block per SM: the tile shape with the least work per
@@ -390,17 +371,7 @@ HeatTilePlan heat_tile_plan(int nx, int ny, int ek) {
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   cudaDeviceGetAttribute(&smem_max, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
   if (!coop || sms < 1) return tp;
-  long long best = -1;
-  for (int gx = 1; gx <= std::min(nx, sms); ++gx) {
-    const int gy = std::min(ny, sms / gx);
-    const int w = ceil_div(nx, gx), h = ceil_div(ny, gy);
-    const long long c = phase_warps(w, h);
-    if (best < 0 || c < best) {
-      best = c;
-      tp.tw = w;
-      tp.th = h;
-    }
-  }
+  heat_geom::tile_shape(nx, ny, sms, &tp.tw, &tp.th);
   tp.ntx = ceil_div(nx, tp.tw);
   const int nb = tp.ntx * ceil_div(ny, tp.th);
   tp.smem = heat_tile_bytes(tp.tw, tp.th, sizeof(T));
