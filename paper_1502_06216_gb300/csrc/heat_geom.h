@@ -6,10 +6,12 @@
 #include <algorithm>
 #include <cstdint>
 
+#ifndef JKO_HD
 #ifdef __CUDACC__
 #define JKO_HD __host__ __device__ __forceinline__
 #else
 #define JKO_HD inline
+#endif
 #endif
 
 namespace jko {

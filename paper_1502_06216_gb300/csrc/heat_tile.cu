@@ -20,6 +20,7 @@
 // halo work).
 #include <algorithm>
 
+#include "epoch.h"
 #include "heat_cell.cuh"
 #include "heat_geom.h"
 #include "jko_kernels.h"
@@ -74,7 +75,8 @@ heat_tile_kernel(const __grid_constant__ HeatTileArgs<T> A, const __grid_constan
   }
   const int maxit = ctrl->max_iter, stall = ctrl->stall;
   const double tol = ctrl->tol;
-  unsigned ep = *(volatile unsigned*)A.epoch;
+  const unsigned ep0 = *(volatile unsigned*)A.epoch;
+  unsigned ep = ep0;
   const int nx = A.nx, ny = A.ny;
   const size_t N = (size_t)nx * ny;
   const heat_geom::Tile tile = heat_geom::tile_of(blockIdx.x, A.tw, A.th, A.ntx, nx, ny);
@@ -345,7 +347,7 @@ heat_tile_kernel(const __grid_constant__ HeatTileArgs<T> A, const __grid_constan
     if (s_fault) atomicOr(&ctrl->nonfinite, 2);
     if (blockIdx.x == 0) {
       ctrl->it = it;
-      *A.epoch = ep;
+      *A.epoch = epoch::after(ep0, ep, epoch::of_heat(A.pairs, A.D, H), s_fault);
     }
   }
 }

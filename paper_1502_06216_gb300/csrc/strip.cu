@@ -26,6 +26,7 @@
 #include <algorithm>
 
 #include "coupled_prox.cuh"
+#include "epoch.h"
 #include "jko_kernels.h"
 #include "strip.cuh"
 
@@ -485,7 +486,7 @@ strip_kernel(const __grid_constant__ StripArgs<T> A, const __grid_constant__ Pro
     if (s_fault) atomicOr(&ctrl->nonfinite, 2);
     if (blockIdx.x == 0) {
       ctrl->it = it;
-      *A.g.epoch = ep0 + 1u + (unsigned)pair;
+      *A.g.epoch = epoch::after(ep0, ep0 + 1u + (unsigned)pair, epoch::of_strip(A.pairs), s_fault);
       if (A.record != nullptr) *A.record = *ctrl;
     }
   }

@@ -14,6 +14,7 @@
 // every eight: the ten-step gradient at 256^2 FP32 took 14.4 ms (11.9 of them here), now 5.3.
 // Four steps of the reverse pass alone, a kernel per pass / here: 512^2 FP32 3.2 / 1.5 ms,
 // 700^2 4.8 / 2.6, 256^2 FP64 8.5 / 6.2.
+#include "epoch.h"
 #include "jko_kernels.h"
 #include "strip.cuh"
 
@@ -64,7 +65,8 @@ strip_adjoint_kernel(const __grid_constant__ AdjArgs<T> A, const __grid_constant
   T *s_D = row(0), *s_iY = row(1), *s_qb = row(2);
   T *s_ab = col(0), *s_s = col(1), *s_lam = col(2), *s_rs = col(3);
   const int ncg = X.ncg, nrg = X.nrg;
-  unsigned ep = *(volatile unsigned*)A.g.epoch;
+  const unsigned ep0 = *(volatile unsigned*)A.g.epoch;
+  unsigned ep = ep0;
   if (tid == 0) s_fault = 0;
   X.load_taps();
   X.load_rows(A.q, s_D);
@@ -228,7 +230,7 @@ strip_adjoint_kernel(const __grid_constant__ AdjArgs<T> A, const __grid_constant
     if (blockIdx.x == 0) {
       if (bad) atomicOr(&A.out->bad, 1);
       A.out->iters = k;
-      *A.g.epoch = ep;
+      *A.g.epoch = epoch::after(ep0, ep, epoch::of_adjoint(A.budget), s_fault);
     }
   }
 }
