@@ -27,7 +27,6 @@ namespace jko {
 
 namespace {
 
-constexpr int HBX = 16, HBY = 8;   // small tiles: the work is FP64-bound per SM, so more blocks spread it
 
 struct HeatGeom {
   int nx, ny;

@@ -6,6 +6,10 @@
 
 namespace jko {
 
+// Block of the kernels per phase (small tiles: the work is FP64-bound per SM, so more blocks
+// spread it), and the cells whose terms of the residual are added together first.
+constexpr int HBX = 16, HBY = 8;
+
 // ---- the per-cell arithmetic of the recurrence ----
 // Written with explicit roundings, so that every kernel below (per phase or
 // persistent) performs the same operations whatever the compiler contracts.

@@ -9,8 +9,10 @@
 // epoch parity: a block writes exchange e + 2 only after it has every
 // neighbour's e + 1, which they wrote after reading e.  So every block that reads a block's
 // words has to be one it waits for: the blocks with a cell within H cells of its tile,
-// whatever the obstacles are (heat_geom.h).  The arithmetic of a cell and the stop rule are those of heat.cu's
-// kernels, so the iterates have the same bits; the residual is added by tiles.
+// whatever the obstacles are (heat_geom.h).  The arithmetic of a cell and the stop rule are
+// those of heat.cu's kernels, and the residual is added in their order (in FP64, by groups of
+// 16 x 8 cells: the cells' terms travel to the block of their group, its sums to every block),
+// so the iterates, the pair counts and the residuals have the same bits.
 //
 // Bound by the exchange and by the FP64 latency of its steps (five operations a cell, four
 // deep, on a pipe of half a lane a cycle and scheduler): 100^2, 150 tiles, degree 54, a
@@ -38,7 +40,8 @@ using heat_geom::H;
 
 template <typename T>
 struct HeatTileArgs {
-  int nx, ny, tw, th, ntx, nb, D;
+  int nx, ny, tw, th, ntx, D;
+  int gx, ng;                // groups along x, and all of them
   double ax, ay;
   const double* coef;
   const uint8_t* mask;
@@ -48,7 +51,8 @@ struct HeatTileArgs {
   Ctrl* ctrl;
   unsigned long long* xb;    // iterates: [2][cells][4]
   unsigned long long* xv;    // v: [2][cells][2]
-  unsigned long long* xres;  // residuals: [2][nb][2]
+  unsigned long long* xt;    // terms of the residual, an element a cell
+  unsigned long long* xres;  // its sums over groups of HBX x HBY cells: [2][ng][2]
   unsigned* epoch;
   int pairs;
 };
@@ -58,14 +62,65 @@ __host__ __device__ inline size_t heat_tile_bytes(int tw, int th, size_t es) {
   return box * 25 + (size_t)tw * th * es * 4;
 }
 
+// A cell's term of the residual (its word or words), polled until it carries epoch ep.
+__device__ __forceinline__ void load_term(const unsigned long long* w, unsigned long long& x,
+                                          unsigned long long&, float) {
+  x = get_word(w);
+}
+__device__ __forceinline__ void load_term(const unsigned long long* w, unsigned long long& x,
+                                          unsigned long long& y, double) {
+  get_words(w, x, y);
+}
+__device__ __forceinline__ double wait_term(const unsigned long long* w, unsigned ep,
+                                            unsigned long long x, unsigned long long, float,
+                                            int* fault) {
+  for (unsigned i = 0; (unsigned)(x >> 32) != ep; ++i) {
+    if (i >= kSpin || *(volatile int*)fault) {
+      *fault = 1;
+      break;
+    }
+    x = get_word(w);
+  }
+  return (double)__uint_as_float((unsigned)x);
+}
+__device__ __forceinline__ double wait_term(const unsigned long long* w, unsigned ep,
+                                            unsigned long long x, unsigned long long y, double,
+                                            int* fault) {
+  if (!wait_pair(w, ep, x, y, fault)) *fault = 1;
+  return words_double(x, y);
+}
+
+// The residual's terms over group g of HBX x HBY cells, in FP64 and in the order in which
+// heat_bupdate's block of these cells adds them (block_sum: 32 cells a warp, then the warps).
+// One warp; every lane gets it.
+template <typename T>
+__device__ __forceinline__ double group_sum(const HeatTileArgs<T>& A, int g, int lane, unsigned ep,
+                                            int* fault) {
+  constexpr int W = HBX * HBY / 32;   // warps of that block
+  static_assert(W == 4 && 32 % HBX == 0, "the order below");
+  const int gy = g / A.gx, xx = (g - gy * A.gx) * HBX + (lane & (HBX - 1));
+  unsigned long long x[W], y[W];
+  double t[W];
+  auto at = [&](int k) -> const unsigned long long* {
+    const int yy = gy * HBY + k * (32 / HBX) + lane / HBX;
+    return xx < A.nx && yy < A.ny ? A.xt + kWords<T> * ((size_t)yy * A.nx + xx) : nullptr;
+  };
+#pragma unroll
+  for (int k = 0; k < W; ++k)
+    if (at(k) != nullptr) load_term(at(k), x[k], y[k], T(0));
+#pragma unroll
+  for (int k = 0; k < W; ++k)
+    t[k] = warp_sum(at(k) != nullptr ? wait_term(at(k), ep, x[k], y[k], T(0), fault) : 0.0);
+  return (t[0] + t[2]) + (t[1] + t[3]);
+}
+
 template <typename T, int EK>
 __global__ void __launch_bounds__(HTT)
 heat_tile_kernel(const __grid_constant__ HeatTileArgs<T> A, const __grid_constant__ ProxArgs<T> P) {
   extern __shared__ __align__(16) unsigned char smem[];
   __shared__ int s_bad, s_fault, s_dec;
-  __shared__ double s_wres[HTT / 32];
-  const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
-  const int nwork = blockDim.x - 32, nww = nwork >> 5;   // the last warp decides
+  const int tid = threadIdx.x, lane = tid & 31;
+  const int nwork = blockDim.x - 32;   // the last warp decides
   const bool work = tid < nwork;
   Ctrl* ctrl = A.ctrl;
   const int done0 = *(volatile int*)&ctrl->done, bad0 = *(volatile int*)&ctrl->nonfinite;
@@ -156,10 +211,12 @@ heat_tile_kernel(const __grid_constant__ HeatTileArgs<T> A, const __grid_constan
           sv[c] = words_double(lo, hi);
         }
       } else if (app == 1) {
-        unsigned long long* xr = A.xres + (size_t)(pair & 1) * A.nb * 2;
-        const double mine = warp_sum(lane < nww ? s_wres[lane] : 0.0);
-        if (lane == 0) put_elem(xr + 2 * blockIdx.x, s_bad ? (double)NAN : mine, ep);
-        const double v = gather_sum(xr, A.nb, ep, &s_fault);
+        unsigned long long* xr = A.xres + (size_t)(pair & 1) * A.ng * 2;
+        for (int g = blockIdx.x; g < A.ng; g += gridDim.x) {
+          const double mine = group_sum<T>(A, g, lane, ep, &s_fault);
+          if (lane == 0) put_elem(xr + 2 * g, mine, ep);
+        }
+        const double v = gather_sum(xr, A.ng, ep, &s_fault);
         const bool first = lane == 0 && blockIdx.x == 0;
         int d = RUNNING;
         if (!isfinite(v)) d = NONFINITE;
@@ -189,7 +246,6 @@ heat_tile_kernel(const __grid_constant__ HeatTileArgs<T> A, const __grid_constan
         cur2[c] = 0.0;
       }
       __syncthreads();
-      T res = T(0);
       int bad = 0;
       const bool have_prev = app == 0 && it > 0;
       int ns = A.D % H == 0 ? H : A.D % H;
@@ -225,10 +281,14 @@ heat_tile_kernel(const __grid_constant__ HeatTileArgs<T> A, const __grid_constan
         const T yv = close_out<T>(r);
         if (app == 0) {
           const T qi = s_q[i];
-          if (have_prev) res += abs_residual<T>(s_b[i], yv, qi);
+          const T res = have_prev ? abs_residual<T>(s_b[i], yv, qi) : T(0);
           const T bn = b_update<T>(qi, yv);
-          bad |= !dev_finite(bn);
+          const bool inf = !dev_finite(bn);
+          bad |= inf;
           s_b[i] = bn;
+          // (NaN where the block has met a non-finite scaling)
+          put_elem(A.xt + kWords<T> * ((size_t)(y0 + y) * nx + x0 + x), inf || s_bad ? (T)NAN : res,
+                   ep + 1);
           sv[c] = f ? (double)bn : 0.0;
         } else {
           const T ai = prox_ratio<T, EK>(P, (y0 + y) * nx + x0 + x, yv);
@@ -325,12 +385,7 @@ heat_tile_kernel(const __grid_constant__ HeatTileArgs<T> A, const __grid_constan
         __syncthreads();
         if (s_fault) break;
       }
-      if (app == 0) {
-        const double wres = warp_res(res);
-        if (lane == 0) s_wres[wid] = wres;
-      } else {
-        ++it;
-      }
+      if (app == 1) ++it;
       if (bad) s_bad = 1;
       __syncthreads();
     }
@@ -390,7 +445,9 @@ HeatTilePlan heat_tile_plan(int nx, int ny, int ek) {
     return tp;
   }
   tp.G = nb;
-  tp.words = (size_t)nx * ny * 12 + 4 * (size_t)nb + 2;
+  const size_t N = (size_t)nx * ny;
+  tp.words = N * 12 + ((N * kWords<T> + 1) & ~(size_t)1) +
+             4 * (size_t)(ceil_div(nx, HBX) * ceil_div(ny, HBY)) + 2;
   return tp;
 }
 
@@ -401,9 +458,11 @@ cudaError_t heat_tile_launch(const HeatTilePlan& tp, const HeatPlan& hp, const H
                              int pairs, cudaStream_t st) {
   const size_t N = (size_t)nx * ny;
   const double inv_delta = hp.delta > 0 ? 1.0 / hp.delta : 0.0;
-  HeatTileArgs<T> A{nx, ny, tp.tw, tp.th, tp.ntx, tp.G, hp.D, 2.0 * inv_delta * hp.cx,
+  const int gx = ceil_div(nx, HBX), ng = gx * ceil_div(ny, HBY);
+  HeatTileArgs<T> A{nx, ny, tp.tw, tp.th, tp.ntx, hp.D, gx, ng, 2.0 * inv_delta * hp.cx,
                     2.0 * inv_delta * hp.cy, (const double*)B.coef, mask, q, a, p, ctrl, words,
-                    words + 8 * N, words + 12 * N, (unsigned*)(words + tp.words - 2), pairs};
+                    words + 8 * N, words + 12 * N, words + tp.words - 2 - 4 * (size_t)ng,
+                    (unsigned*)(words + tp.words - 2), pairs};
   ProxArgs<T> Pc = P;
   void* args[] = {&A, &Pc};
   StripPlan sp;

@@ -25,6 +25,11 @@ __device__ __forceinline__ void put_word(unsigned long long* w, unsigned v, unsi
   const unsigned long long x = (unsigned long long)ep << 32 | v;
   asm volatile("st.relaxed.gpu.global.u64 [%0], %1;" ::"l"(w), "l"(x) : "memory");
 }
+__device__ __forceinline__ unsigned long long get_word(const unsigned long long* w) {
+  unsigned long long x;
+  asm volatile("ld.relaxed.gpu.global.u64 %0, [%1];" : "=l"(x) : "l"(w) : "memory");
+  return x;
+}
 __device__ __forceinline__ void get_words(const unsigned long long* w, unsigned long long& x,
                                           unsigned long long& y) {
   asm volatile("ld.relaxed.gpu.global.v2.u64 {%0, %1}, [%2];"

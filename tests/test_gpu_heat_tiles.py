@@ -42,3 +42,32 @@ def test_tiles_equal_the_kernels_per_phase_beside_obstacles(prec, nx, ny, kind):
         out.append(traj)
         jko.jko_destroy(h)
     assert torch.equal(out[0], out[1])
+
+
+@pytest.mark.parametrize("prec,nx,ny,steps", [
+    ("FP32", 64, 64, 2), ("FP64", 40, 56, 2), ("FP32", 100, 100, 2), ("FP64", 50, 50, 2),
+    ("FP32", 37, 61, 1), ("FP32", 1, 64, 1), ("FP64", 5, 4, 1)])
+def test_residuals_have_the_bits_of_the_kernels_per_phase(prec, nx, ny, steps):
+    """The residual decides the stop, so it is added in FP64 and in one order in every
+    form: the reports are equal, not only the images."""
+    torch = need_gpu()
+    from paper_1502_06216_gb300 import jko
+    pb = inputs.heat_crowd_problem(nx, ny=ny, n_steps=steps, tol=1e-6, max_iter=60) \
+        if min(nx, ny) > 5 else problem_1d(nx, ny)
+    out = []
+    for loop in (2, 1):
+        h = jko.create_from_problem(pb, precision=jko.Precision[prec], loop=loop)
+        p0 = torch.tensor(pb.q0, dtype=h.dtype, device="cuda")
+        _, traj, infos = jko.jko_flow(h, p0, steps)
+        out.append([(i["iters"], int(i["status"]), i["residual_l1"], i["mass"]) for i in infos])
+        jko.jko_destroy(h)
+    print(prec, nx, ny, out)
+    assert out[0] == out[1]
+
+
+def problem_1d(nx, ny):
+    n = nx * ny
+    t = (np.arange(n) + 0.5) / n
+    q0 = (t < 0.3).astype(np.float64)
+    return inputs.Problem(nx=nx, ny=ny, gamma=1e-3, tau=0.01, q0=q0 / q0.sum(), w=3.0 * t,
+                          kappa=float((q0 / q0.sum()).max()), heat_L=10, n_steps=1, tol=1e-6, max_iter=40)
