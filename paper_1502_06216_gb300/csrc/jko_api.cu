@@ -1002,13 +1002,16 @@ jko_status setup_simt(jko_handle* h) {
   return JKO_OK;
 }
 
-// The persistent CUDA-core form, where its rule takes this grid; max_blocks > 0: the same
-// form on fewer blocks where its strips fit them (else it stays as it is).
+// The persistent CUDA-core form, where its rule takes this grid; max_blocks > 0: the form of a
+// flow in a batch, on at most so many blocks where its strips fit them (else on as many as alone).
 template <typename T>
 jko_status setup_strip(jko_handle* h, int max_blocks) {
-  const jko::StripPlan sp =
-      jko::strip_plan<T>(h->grid.nx, h->grid.ny, h->rx, h->ry, strip_op(h), h->ek,
-                         jko::prox_args<T>(h), max_blocks, h->strip.parts);
+  auto plan = [&](int blocks) {
+    return jko::strip_plan<T>(h->grid.nx, h->grid.ny, h->rx, h->ry, strip_op(h), h->ek,
+                              jko::prox_args<T>(h), blocks, h->strip.parts);
+  };
+  jko::StripPlan sp = plan(max_blocks);
+  if (sp.G == 0 && max_blocks > 0) sp = plan(1 << 30);
   if (sp.G == 0) return JKO_OK;
   if (h->strip_words) cudaFree(h->strip_words);
   h->strip_words = nullptr;
@@ -2402,7 +2405,6 @@ jko_status jko_batch_create(int n_flows, const jko_grid* grids, const jko_params
     for (auto* h : b->h) {
       if (h->strip.G == 0) continue;
       const int most = std::max(19, (int)(2.0 * sms * work(h) / all));
-      if (most >= h->strip.G) continue;
       const jko_status s = h->fp64 ? setup_strip<double>(h, most) : setup_strip<float>(h, most);
       if (s != JKO_OK) return fail(batch_err(b, s, h->err));
     }

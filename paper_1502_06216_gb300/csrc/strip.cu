@@ -181,14 +181,18 @@ strip_kernel(const __grid_constant__ StripArgs<T> A, const __grid_constant__ Pro
 
   int it = 0, pair = 0, since = 0;
   double best = INFINITY;
+  // warps whose threads have terms of the residual
+  const int active =
+      OP == OP_PAIR ? nwarps : min(nwarps, (NI * A.g.nr * ((nx + RB - 1) / RB) + 31) >> 5);
   // the block's residual (NaN where it met a non-finite scaling) to every block
   const int n_res = OP == OP_PAIR ? A.g.gc : A.g.gr;
   auto put_residual = [&](unsigned ep) {
     unsigned long long* xr = A.g.xres + (size_t)(pair & 1) * n_res * 2;
     if (wid == nwarps - 1 && (int)blockIdx.x < n_res) {   // the warp with the fewest items
-      double v = lane < nwarps ? s_wres[lane] : 0.0;   // at most 16 warps
+      double v = lane < active ? s_wres[lane] : 0.0;   // at most 16 warps
 #pragma unroll
-      for (int o = 8; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+      for (int o = 8; o > 0; o >>= 1)
+        if (o < active) v += __shfl_xor_sync(0xffffffffu, v, o);
       if (lane == 0) put_elem(xr + 2 * blockIdx.x, s_bad ? (double)NAN : v, ep);
     }
   };
@@ -247,8 +251,11 @@ strip_kernel(const __grid_constant__ StripArgs<T> A, const __grid_constant__ Pro
       } else {
         // rows: Y = T K_x, the residual |b_old Y - q| and b = q / Y
         const bool have_prev = it > 0;
-        T res = T(0);
+        // an item's terms in the working precision, as a thread of filter_pass adds its own, and
+        // in FP64 from there on
+        double sum = 0.0;
         X.filter_rows(X.r2, [&](int m, int l, int i0, T (&acc)[RB]) {
+          T res = T(0);
           X.each(acc, i0, nx, [&](int i, T v) {
             const T qv = row(m)[l * nx + i];
             T* bp = X.b + X.at_r(m, l, i);
@@ -257,10 +264,13 @@ strip_kernel(const __grid_constant__ StripArgs<T> A, const __grid_constant__ Pro
             bad |= !dev_finite(bn);
             *bp = bn;
           });
+          sum += (double)res;
         });
-        // the warps' residuals in the working precision, the block's and the grid's in FP64
-        const double wres = warp_res(res);
-        if (lane == 0) s_wres[wid] = wres;
+        // warps without items have nothing to add (an FP64 tree takes ~450 cycles)
+        if (wid < active) {
+          const double wres = warp_sum(sum);
+          if (lane == 0) s_wres[wid] = wres;
+        }
         if (bad) s_bad = 1;
       }
       __syncthreads();
@@ -573,7 +583,10 @@ StripPlan strip_plan(int nx, int ny, int rx, int ry, int op, int ek, const ProxA
   // do not (us a pair, one part / now: 64^2 19 / 13.3, 128^2 30 / 26)
   if (max_blocks > 0) sp.parts = parts;
   else while (sizeof(T) == 8 && sp.parts < 8 && items(1) * sp.parts < 256) sp.parts *= 2;
-  sp.threads = std::min(512, std::max(256, ceil_div(items(sp.rb) * sp.parts, 32) * 32));
+  // a warp more than the items fill: it adds and sends the residual while the others filter
+  // (not in a batch, whose flows' blocks share the SMs' registers)
+  sp.threads = std::min(512, std::max(256, ceil_div(items(sp.rb) * sp.parts, 32) * 32 +
+                                               (max_blocks > 0 ? 0 : 32)));
   int rows = 0, cols = 0;
   strip_images<T>(op, ek, P, &rows, &cols);
   const Smem S = smem_of<T>(nx, ny, rx, ry, sp.nc, sp.nr, ni, sp.parts, rows, cols, P.mask != nullptr);

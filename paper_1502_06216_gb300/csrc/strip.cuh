@@ -156,11 +156,6 @@ __device__ __forceinline__ void line_taps_part(double (&acc)[1], const double* l
   for (; t <= t_hi; ++t) acc[0] = fma(s_k[t], x[t], acc[0]);
 }
 
-// The warp's sum of the residual terms: a tree in the working precision (FP32
-// terms carry ~2^-24 each; the blocks and the grid are added in FP64).
-__device__ __forceinline__ double warp_res(float v) { return (double)warp_sum_f(v); }
-__device__ __forceinline__ double warp_res(double v) { return warp_sum(v); }
-
 // w / d for w < 2^16 d with m = ceil(2^32 / d) (d = 1: m wraps to 0)
 __device__ __forceinline__ int div_by(int w, int d, unsigned m) {
   return d == 1 ? w : (int)__umulhi((unsigned)w, m);
