@@ -21,6 +21,7 @@
 #include <cstring>
 #include <vector>
 
+#include "adjoint_cell.h"
 #include "jko.h"
 #include "jko_handle.h"
 #include "jko_kernels.h"
@@ -108,7 +109,7 @@ __global__ void k_lambda(const T* abar, const T* w2, T* lam, double* diff, doubl
   double d = 0.0, a = 0.0;
   GS(i, n) {
     const T ln = abar[i] - w2[i];
-    d += fabs((double)ln - (double)lam[i]);
+    d += jko::lambda_change(ln, lam[i]);
     a += fabs((double)abar[i]);
     lam[i] = ln;
   }

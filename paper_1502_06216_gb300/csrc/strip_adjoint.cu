@@ -14,6 +14,7 @@
 // every eight: the ten-step gradient at 256^2 FP32 took 14.4 ms (11.9 of them here), now 5.3.
 // Four steps of the reverse pass alone, a kernel per pass / here: 512^2 FP32 3.2 / 1.5 ms,
 // 700^2 4.8 / 2.6, 256^2 FP64 8.5 / 6.2.
+#include "adjoint_cell.h"
 #include "epoch.h"
 #include "jko_kernels.h"
 #include "strip.cuh"
@@ -178,14 +179,14 @@ strip_adjoint_kernel(const __grid_constant__ AdjArgs<T> A, const __grid_constant
     rows_out([&](int e, int i, T z) { X.b[i] = s_D[e] * z; });
     to_cols();
     X.filter_cols(X.c2, [&](int, int l, int i0, T (&acc)[RB]) {
-      T diff = T(0), u[RB];
+      T u[RB];
 #pragma unroll
       for (int o = 0; o < RB; ++o) {   // (all loads before the first store)
         const int e = l * ny + i0 + o;
         u[o] = T(0);
         if (i0 + o >= ny) continue;
         acc[o] = s_ab[e] - acc[o];
-        diff += fabs(acc[o] - s_lam[e]);
+        acc_d += lambda_change(acc[o], s_lam[e]);
         u[o] = s_rs[e] * acc[o];
       }
 #pragma unroll
@@ -194,7 +195,6 @@ strip_adjoint_kernel(const __grid_constant__ AdjArgs<T> A, const __grid_constant
         s_lam[l * ny + i0 + o] = acc[o];
         X.a[X.at_c(0, l, i0 + o)] = u[o];
       }
-      acc_d += (double)diff;
     });
     ++k;
     if ((k & 7) == 0) {
