@@ -2305,7 +2305,9 @@ cudaError_t batch_copy(jko_batch* b, int first, int n, cudaStream_t st) {
 }
 
 // A flow of a batch whose every step is one launch per flow (g_first, g_step): the steps
-// follow each other on the device, the host reads all control blocks once.
+// follow each other on the device, the host reads their control blocks at the end.  It waits
+// for the first step's alone, with the second one enqueued behind it, so that an invalid
+// input costs two steps and not all of them.
 jko_status batch_flow_strips(jko_batch* b, const void* const* p0_dev, int n_steps,
                              void* const* p_final_dev, jko_step_info* infos) {
   cudaStream_t st = b->stream;
@@ -2325,10 +2327,17 @@ jko_status batch_flow_strips(jko_batch* b, const void* const* p0_dev, int n_step
     BCK(b, cudaGraphLaunch(t == 0 ? b->g_first : b->g_step, st));
     BCK(b, cudaMemcpyAsync(b->host_steps + (size_t)t * n, b->ctrl_all, sizeof(Ctrl) * n,
                            cudaMemcpyDeviceToHost, st));
+    if (t == 0) BCK(b, cudaEventRecord(b->ev_poll[0], st));
+    if (t == std::min(1, n_steps - 1)) {
+      BCK(b, cudaEventSynchronize(b->ev_poll[0]));
+      const jko_status sv = check_inputs(b, b->host_steps);
+      if (sv != JKO_OK) {
+        BCK(b, cudaStreamSynchronize(st));
+        return sv;
+      }
+    }
   }
   BCK(b, cudaStreamSynchronize(st));
-  const jko_status sv = check_inputs(b, b->host_steps);
-  if (sv != JKO_OK) return sv;
   int worst = JKO_OK;
   for (int t = 0; t < n_steps; ++t) {
     for (int f = 0; f < n; ++f)
