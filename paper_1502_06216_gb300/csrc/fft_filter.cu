@@ -273,7 +273,7 @@ cudaError_t launch_fft_fj(const PassArgs<T>& A, const ProxArgs<T>& P, const FftA
                           cudaStream_t st) {
   const size_t smem = fft_smem<T>(F.L, FJ);
   auto kern = fft_pass_kernel<T, EPI, EK, FJ>;
-  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  cudaError_t e = max_dynamic_smem((const void*)kern);
   if (e != cudaSuccess) return e;
   // one thread per four points and line, 64 to 512
   int threads = FJ / 2 * F.L / 4;

@@ -437,7 +437,7 @@ HeatTilePlan heat_tile_plan(int nx, int ny, int ek) {
   if (tp.smem + 1024 > (size_t)smem_max) return tp;
   void* fn = heat_tile_fn<T>(ek);
   int per_sm = 0;
-  if (strip_cap(fn) != cudaSuccess ||
+  if (max_dynamic_smem(fn) != cudaSuccess ||
       cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, tp.threads, tp.smem) !=
           cudaSuccess ||
       per_sm * sms < nb) {

@@ -140,6 +140,11 @@ cudaError_t strip_adjoint_launch(const StripPlan& sp, size_t smem, int ek, int n
                                  int ry, const T* taps_x, const T* taps_y, const StripAdjoint<T>& s,
                                  const ProxArgs<T>& P, unsigned long long* words, cudaStream_t st);
 
+// Sets a kernel's limit of dynamic shared memory: the device's, less 1 KB for its static
+// arrays.  The same whatever the launch needs: a limit of a launch's own size, set by a small
+// grid, would stand under a larger one's launch from another thread, or a captured graph's.
+cudaError_t max_dynamic_smem(const void* fn);
+
 // Step prologue / epilogue kernels (jko_step_kernels.cu).
 template <typename T>
 cudaError_t launch_fill(T* x, T v, long long n, cudaStream_t st);

@@ -252,6 +252,15 @@ cudaError_t launch_copies(const CopyItem* items, int n, cudaStream_t st) {
   return cudaGetLastError();
 }
 
+cudaError_t max_dynamic_smem(const void* fn) {
+  int dev = 0, most = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e == cudaSuccess)
+    e = cudaDeviceGetAttribute(&most, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+  return e != cudaSuccess
+             ? e : cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, most - 1024);
+}
+
 cudaError_t launch_gather_done(Ctrl* const* ctrls, int* done, int n, cudaStream_t st) {
   gather_done_kernel<<<(n + 127) / 128, 128, 0, st>>>(ctrls, done, n);
   return cudaGetLastError();

@@ -345,8 +345,7 @@ cudaError_t launch_rb(const PassArgs<T>& A, const ProxArgs<T>& P, cudaStream_t s
   // opt in well below 48 KB: the kernel's static shared memory (stop gate,
   // reductions) counts against the same default limit
   if (smem > 32 * 1024) {
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)smem);
+    cudaError_t e = max_dynamic_smem((const void*)kern);
     if (e != cudaSuccess) return e;
   }
   dim3 block(BJ, BI);

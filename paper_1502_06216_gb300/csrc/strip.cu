@@ -531,17 +531,6 @@ void* strip_fn<double>(int, int op, int ek) { return strip_fn_op<double, 1, 512>
 
 }  // namespace
 
-// The kernel's limit of dynamic shared memory: the same for every handle, so that none lowers
-// it under another's (or under a captured graph).  The plans leave 1 KB for static arrays.
-cudaError_t strip_cap(void* fn) {
-  int dev = 0, most = 0;
-  cudaError_t e = cudaGetDevice(&dev);
-  if (e == cudaSuccess)
-    e = cudaDeviceGetAttribute(&most, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
-  return e != cudaSuccess
-             ? e : cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, most - 1024);
-}
-
 // The rule for the persistent form, on the grid, the band and the precision.
 // Both sides measured on a GB300 (us a pair, this form / a kernel per pass, 30 pairs a
 // step): crowd FP32 128^2 9.1 / 21.2, 256^2 10.5 / 25.2, 512^2 25 / 43, 600 x 200
@@ -594,7 +583,7 @@ StripPlan strip_plan(int nx, int ny, int rx, int ry, int op, int ek, const ProxA
   if (S.total + 1024 > (size_t)smem_max) return StripPlan{};
   void* fn = strip_fn<T>(sp.rb, op, ek);
   int per_sm = 0;
-  if (strip_cap(fn) != cudaSuccess ||
+  if (max_dynamic_smem(fn) != cudaSuccess ||
       cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, sp.threads, S.total) !=
           cudaSuccess ||
       per_sm * sms < sp.G) {
@@ -633,7 +622,7 @@ cudaError_t strip_coop(void* fn, const StripPlan& sp, size_t smem, int threads, 
   at[0].val.cooperative = 1;
   cfg.attrs = at;
   cfg.numAttrs = 1;
-  const cudaError_t e = strip_cap(fn);
+  const cudaError_t e = max_dynamic_smem(fn);
   if (e != cudaSuccess) return e;
   return cudaLaunchKernelExC(&cfg, fn, args);
 }

@@ -488,7 +488,6 @@ __device__ __forceinline__ double gather_sum(const unsigned long long* xr, int b
 struct StripPlan;
 strip::Geo strip_geo(const StripPlan& sp, int nx, int ny, int rx, int ry, const void* taps_x,
                      const void* taps_y, unsigned long long* words);
-cudaError_t strip_cap(void* fn);
 cudaError_t strip_coop(void* fn, const StripPlan& sp, size_t smem, int threads, void** args,
                        cudaStream_t st);
 
