@@ -1060,8 +1060,8 @@ jko_status step_status(const Ctrl& c) {
   return JKO_OK;
 }
 
-// The chunk loop of a step as a graph: a WHILE node whose body is one chunk
-// (the pairs of h->chunk, or one launch of the persistent loop kernel) and the
+// The chunk loop of a step as a graph (handles whose steps are not one persistent launch):
+// a WHILE node whose body is one chunk (the pairs of h->chunk) and the
 // loop condition, which ends it when the step has stopped or after the chunk
 // budget of the host-driven loop.  Built once, at the first flow of more than
 // one step; where the runtime refuses it (state -1) flows keep host-driven chunks.
@@ -1092,9 +1092,7 @@ void build_step_loop(jko_handle* h) {
                                       cudaStreamCaptureModeThreadLocal);
     if (e == cudaSuccess) {
       cudaError_t e1 = cudaSuccess;
-      if (h->use_loop) e1 = enqueue_loop(h, C, h->cap);
-      else
-        for (int i = 0; i < C && e1 == cudaSuccess; ++i) e1 = enqueue_pair(h, h->cap);
+      for (int i = 0; i < C && e1 == cudaSuccess; ++i) e1 = enqueue_pair(h, h->cap);
       if (e1 == cudaSuccess)
         e1 = jko::launch_chunk_loop_cond(h->chunk_ctr, h->ctrl, hc, max_chunks, h->cap);
       cudaGraph_t captured = nullptr;
@@ -2464,7 +2462,35 @@ jko_status jko_batch_create(int n_flows, const jko_grid* grids, const jko_params
   }
   for (auto* h : b->h)
     h->chunk_iters = h->use_loop ? h->prm.max_iter + 1 : C;
-  jko_status s = capture_batch(
+  auto gather = [b](cudaStream_t root) {
+    return jko::launch_gather_ctrl(b->ctrl_ptrs, b->ctrl_all, b->n, root);
+  };
+  jko_status s = JKO_OK;
+  bool all_strips = true;
+  for (auto* h : b->h) all_strips = all_strips && on_strips(h);
+  if (all_strips) {
+    // every step one graph of one launch per flow: no host decision between the steps
+    s = capture_batch(b, no_op, [](jko_handle* h, cudaStream_t st) { return flow_strip(h, 1, 1, st); },
+                      gather, &b->g_first);
+    if (s == JKO_OK)
+      s = capture_batch(b, no_op, [](jko_handle* h, cudaStream_t st) { return flow_strip(h, 0, 1, st); },
+                        gather, &b->g_step);
+    if (s == JKO_OK) {
+      if (cudaMallocHost((void**)&b->copy_host, sizeof(jko::CopyItem) * 2 * n_flows) != cudaSuccess ||
+          cudaMalloc((void**)&b->copy_dev, sizeof(jko::CopyItem) * 2 * n_flows) != cudaSuccess)
+        return fail(batch_err(b, JKO_ERR_OOM, "batch allocation"));
+      *out = b;
+      return JKO_OK;
+    }
+    // cooperative launches that cannot be captured: per-pass kernels instead
+    cudaGetLastError();
+    b->per_pass = true;
+  }
+  // (a flow of the kernels per pass starts its scalings by itself: not on_strips)
+  if (b->per_pass)
+    for (auto* h : b->h)
+      if (h->strip.G > 0) h->use_loop = 0;
+  s = capture_batch(
       b, no_op, [](jko_handle* h, cudaStream_t st) { return flow_prologue(h, st); },
       [b](cudaStream_t root) { return begin_groups(b, root); }, &b->g_pro);
   if (s != JKO_OK) return fail(s);
@@ -2477,8 +2503,8 @@ jko_status jko_batch_create(int n_flows, const jko_grid* grids, const jko_params
         &b->g_chunk, !pp);
   };
   s = capture_chunks();
-  if (s != JKO_OK) {
-    // cooperative launches that cannot be captured: per-pass kernels instead
+  if (s != JKO_OK && !b->per_pass) {
+    // as above, where only some flows run on strips
     cudaGetLastError();
     b->per_pass = true;
     s = capture_chunks();
@@ -2503,27 +2529,8 @@ jko_status jko_batch_create(int n_flows, const jko_grid* grids, const jko_params
   for (auto* h : b->h) all_loop = all_loop && h->use_loop;
   if (all_loop) b->C = b->max_iter + 1;
   b->all_loop = all_loop;
-  bool all_strips = all_loop;
-  for (auto* h : b->h) all_strips = all_strips && on_strips(h);
-  if (all_strips) {
-    // every step one graph of one launch per flow: no host decision between the steps
-    auto tail = [&](cudaStream_t root) {
-      return jko::launch_gather_ctrl(b->ctrl_ptrs, b->ctrl_all, b->n, root);
-    };
-    s = capture_batch(b, no_op, [](jko_handle* h, cudaStream_t st) { return flow_strip(h, 1, 1, st); },
-                      tail, &b->g_first);
-    if (s == JKO_OK)
-      s = capture_batch(b, no_op, [](jko_handle* h, cudaStream_t st) { return flow_strip(h, 0, 1, st); },
-                        tail, &b->g_step);
-    if (s != JKO_OK) return fail(s);
-    if (cudaMallocHost((void**)&b->copy_host, sizeof(jko::CopyItem) * 2 * n_flows) != cudaSuccess ||
-        cudaMalloc((void**)&b->copy_dev, sizeof(jko::CopyItem) * 2 * n_flows) != cudaSuccess)
-      return fail(batch_err(b, JKO_ERR_OOM, "batch allocation"));
-  }
   s = capture_batch(
-      b, no_op, [](jko_handle* h, cudaStream_t st) { return flow_finalize(h, st); },
-      [b](cudaStream_t root) { return jko::launch_gather_ctrl(b->ctrl_ptrs, b->ctrl_all, b->n, root); },
-      &b->g_fin);
+      b, no_op, [](jko_handle* h, cudaStream_t st) { return flow_finalize(h, st); }, gather, &b->g_fin);
   if (s != JKO_OK) return fail(s);
   *out = b;
   return JKO_OK;
