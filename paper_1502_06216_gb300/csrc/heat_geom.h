@@ -4,6 +4,7 @@
 #pragma once
 
 #include <algorithm>
+#include <cstddef>
 #include <cstdint>
 
 #ifndef JKO_HD
@@ -72,6 +73,13 @@ JKO_HD bool sent(int x, int y, const Tile& t) {
   return x < H || x >= t.w - H || y < H || y >= t.h - H;
 }
 JKO_HD bool awaited(int flags) { return flags & IN_GRID; }
+
+// Shared memory of a block: three FP64 images and the flags over the tile's box, four images of
+// `es` bytes an element over the tile.
+JKO_HD size_t tile_bytes(int tw, int th, size_t es) {
+  const size_t box = (size_t)(tw + 2 * H) * (th + 2 * H);
+  return box * 25 + (size_t)tw * th * es * 4;
+}
 
 // The tile shape for at most `blocks` blocks: the least work of a phase of H steps, in warps.
 inline void tile_shape(int nx, int ny, int blocks, int* tw, int* th) {

@@ -57,11 +57,6 @@ struct HeatTileArgs {
   int pairs;
 };
 
-__host__ __device__ inline size_t heat_tile_bytes(int tw, int th, size_t es) {
-  const size_t box = (size_t)(tw + 2 * H) * (th + 2 * H);
-  return box * 25 + (size_t)tw * th * es * 4;
-}
-
 // A cell's term of the residual (its word or words), polled until it carries epoch ep.
 __device__ __forceinline__ void load_term(const unsigned long long* w, unsigned long long& x,
                                           unsigned long long&, float) {
@@ -417,8 +412,8 @@ void* heat_tile_fn(int ek) {
 }  // namespace
 
 // One tile per block and at most one block per SM: the tile shape with the least work per
-// phase.  Where a tile with its halo does not fit the shared memory (about 900 cells a
-// side) heat.cu's form stays, whose blocks walk over several tiles.
+// phase.  Where a tile with its halo does not fit the shared memory (on 152 SMs beyond about 850
+// cells a side in FP32, 730 in FP64) heat.cu's form stays, whose blocks walk over several tiles.
 template <typename T>
 HeatTilePlan heat_tile_plan(int nx, int ny, int ek) {
   HeatTilePlan tp;
@@ -431,7 +426,7 @@ HeatTilePlan heat_tile_plan(int nx, int ny, int ek) {
   heat_geom::tile_shape(nx, ny, sms, &tp.tw, &tp.th);
   tp.ntx = ceil_div(nx, tp.tw);
   const int nb = tp.ntx * ceil_div(ny, tp.th);
-  tp.smem = heat_tile_bytes(tp.tw, tp.th, sizeof(T));
+  tp.smem = heat_geom::tile_bytes(tp.tw, tp.th, sizeof(T));
   const int area = (tp.tw + 2 * H - 2) * (tp.th + 2 * H - 2);
   tp.threads = 32 + std::min(HTT - 32, (area + 31) / 32 * 32);
   if (tp.smem + 1024 > (size_t)smem_max) return tp;

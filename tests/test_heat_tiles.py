@@ -47,7 +47,8 @@ int main(int, char** a) {
   }
   int one_way = 0;
   for (auto& p : waits) one_way += !waits.count({p.second, p.first});
-  std::printf("%d %d %d %d %d\n", nb, (int)waits.size(), one_way, unsent, outside);
+  std::printf("%d %d %d %d %d %d %d\n", nb, (int)waits.size(), one_way, unsent, outside,
+              (int)tile_bytes(tw, th, 4), (int)tile_bytes(tw, th, 8));
 }
 """
 
@@ -86,9 +87,19 @@ def obstacles(nx, ny):
 def test_waiting_is_symmetric_and_awaited_cells_are_sent(relation, nx, ny):
     for sms in (148, 152):
         for name, mask in obstacles(nx, ny):
-            blocks, waits, one_way, unsent, outside = relation(nx, ny, sms, mask)
+            blocks, waits, one_way, unsent, outside, _, _ = relation(nx, ny, sms, mask)
             print(nx, ny, sms, name, blocks, waits, one_way, unsent, outside)
             assert blocks <= sms
             assert one_way == 0, name
             assert unsent == 0, name
             assert outside == 0, name
+
+
+def test_grids_beyond_the_tiles(relation):
+    """The sizes at which heat.cu's persistent kernel (several tiles a block) still runs, as
+    the GPU test of that kernel takes them: the tile does not fit the 227 KB of a block."""
+    smem = 227 * 1024
+    for sms in (148, 152):
+        fits = lambda n, m: relation(n, m, sms, np.zeros((m, n), bool))[5:]
+        assert fits(900, 880)[0] > smem and fits(760, 800)[1] > smem
+        assert fits(840, 840)[0] <= smem and fits(700, 700)[1] <= smem
