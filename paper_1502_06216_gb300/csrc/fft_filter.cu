@@ -45,9 +45,17 @@ namespace {
 
 constexpr int FNT = 512;   // threads per block at most
 
-// Input columns per block: four (a 32-byte sector of FP64 per row), or two where four
-// would leave SMs without a block.
-__host__ __device__ constexpr int fft_cols(int n_j) { return n_j > 4 * 100 ? 4 : 2; }
+// Input columns per block: four (a 32-byte sector of FP64 per row), or two where blocks of
+// four would leave more than a third of the SMs without one.  Us a pair with two / four (porous,
+// 152 SMs: the line lies at 404): FP64 200^2 96 / 139, 300^2 134 / 234, 400^2 244 / 254, 512^2
+// 260 / 270, 600^2 479 / 487, 800^2 755 / 981, 1000^2 1035 / 1043; FP32 300^2 37.6 / 40.5, 400^2
+// 51.3 / 53.4, 512^2 52.5 / 53.8, 800^2 123 / 145, 1000^2 162 / 148, 1200^2 170 / 153, 2000^2 557 / 614.
+int fft_cols(int n_j) {
+  int dev = 0, sms = 0;
+  cudaGetDevice(&dev);
+  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  return n_j > 4 * (2 * sms / 3) ? 4 : 2;
+}
 
 template <typename T> struct C2;
 template <> struct C2<float> { using t = float2; };

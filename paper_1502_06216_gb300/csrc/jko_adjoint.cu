@@ -625,7 +625,7 @@ template <typename T>
 jko_status backward_dispatch(jko_handle* h, const void* gf, void* gp, void* gw, int* it) {
   if (h->attract) return backward_attraction<T>(h, (const T*)gf, (T*)gp, (T*)gw, it);
   if (h->species == 2) return backward_species<T>(h, (const T*)gf, (T*)gp, (T*)gw, it);
-  if (const size_t smem = jko::strip_adjoint_smem<T>(h->strip, h->grid.nx, h->grid.ny, h->rx, h->ry))
+  if (const size_t smem = jko::strip_adjoint_smem<T>(h->strip, h->ek, h->grid.nx, h->grid.ny, h->rx, h->ry))
     return backward_strip<T>(h, smem, (const T*)gf, (T*)gp, (T*)gw, it);
   switch (h->ek) {
     case jko::EK_CROWD:

@@ -547,8 +547,8 @@ cudaError_t enqueue_heat_tiles(jko_handle* h, int pairs, cudaStream_t st) {
                                   jko::prox_args<T>(h), h->ctrl, h->htile_words, pairs, st);
 }
 
-// `pairs` pairs as one persistent launch: the tensor-core loop kernel, the
-// heat kernel's persistent form.
+// `pairs` pairs as one persistent launch: the tensor-core loop kernel or one of the heat
+// kernel's persistent forms.
 cudaError_t enqueue_loop(jko_handle* h, int pairs, cudaStream_t st) {
   if (h->tc) return jko::tc_enqueue_loop(h->tc, pairs, st);
   if (h->htile.G > 0)
@@ -2395,10 +2395,11 @@ jko_status jko_batch_create(int n_flows, const jko_grid* grids, const jko_params
     b->h.push_back(h);
     b->max_iter = std::max(b->max_iter, params[f].max_iter);
   }
-  // Flows on strips share the SMs: each gets blocks for twice its share of the work, 19 at
-  // least, so that the exchanges of one flow run beside the filters of others.  32 flows of
-  // 64^2 to 512^2 (us a four-step flow): 5850 with every flow on all
-  // SMs, 4440 so; 256 of them, five steps, 57.8 and 41.3 ms.
+  // Flows on strips share the SMs: each gets blocks for twice its share of the work, an eighth
+  // of the SMs at least, so that the exchanges of one flow run beside the filters of others.
+  // 32 flows of 64^2 to 512^2 (us a four-step flow): 5850 with every flow on all SMs, 4440
+  // so; 256 of them, five steps, 57.8 and 41.3 ms.  At least 8, 13, 19, 26, 38 blocks of 152: the
+  // bench's first 32 flows, four steps, 5.34 5.23 5.11 5.48 5.48 ms, all 256 36.6 34.4 34.0 36.7 36.9.
   {
     double all = 0.0;
     auto work = [](const jko_handle* h) {
@@ -2411,7 +2412,7 @@ jko_status jko_batch_create(int n_flows, const jko_grid* grids, const jko_params
     for (auto* h : b->h) all += h->strip.G > 0 ? work(h) : 0.0;
     for (auto* h : b->h) {
       if (h->strip.G == 0) continue;
-      const int most = std::max(19, (int)(2.0 * sms * work(h) / all));
+      const int most = std::max(sms / 8, (int)(2.0 * sms * work(h) / all));
       const jko_status s = h->fp64 ? setup_strip<double>(h, most) : setup_strip<float>(h, most);
       if (s != JKO_OK) return fail(batch_err(b, s, h->err));
     }

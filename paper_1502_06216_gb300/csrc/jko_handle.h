@@ -68,7 +68,7 @@ struct jko_handle {
   double* part = nullptr;      // residual partials of the b-update pass (one per block)
   int nparts_simt = 0;
   int part_cap = 0;       // entries of part (residual and mass partials)
-  int use_loop = 0;       // chunks run as one persistent kernel (tensor cores or heat kernel)
+  int use_loop = 0;       // steps run as one persistent kernel (tensor cores, heat kernel, strips)
   int heat_G = 0;         // blocks of the heat kernel's persistent form
   jko::StripPlan strip;   // the CUDA-core form's persistent kernel (G = 0: per-pass kernels)
   unsigned long long* strip_words = nullptr;   // its exchange buffers
@@ -138,10 +138,10 @@ inline ProxArgs<T> prox_args(const jko_handle* h) {
 // One JKO step on device buffers (jko_api.cu); validate = check q first.
 jko_status step_internal(jko_handle* h, const void* q_in, void* p_out, jko_step_info* info,
                          bool validate);
-// Records an error message on the handle and returns the status.
 // Steps 1 .. n_steps - 1 of a recorded flow on strips (tape: per images a step).
 jko_status record_strip(jko_handle* h, void* tape, size_t per, int n_steps, void* last,
                         jko_step_info* infos, double* mass);
+// Records an error message on the handle and returns the status.
 jko_status handle_error(jko_handle* h, jko_status st, const std::string& msg);
 // Argument checks of jko_create (sizes, parameters, energy fields): JKO_OK, or
 // the error status with *msg set to a static description.  Allocates nothing

@@ -73,7 +73,9 @@ cudaError_t simt_pass(int epi, int ek, const PassArgs<T>& A, const ProxArgs<T>& 
 // blocks, each owning nc columns and nr rows of the images in shared memory.
 // strip_plan: G = 0 where the kernels per pass are the faster form or the strips do
 // not fit; max_blocks > 0: at most that many blocks, an output's taps in `parts` parts (those
-// of the plan without a limit give its bits).
+// of the plan without a limit give its images' bits at equal pair counts; the residual is
+// added block by block, so its last bits depend on the split, and with them the pair at which
+// a residual within that rounding of tol stops the step).
 enum : int { OP_ONE = 0, OP_ATTRACT = 1, OP_SPECIES = 2, OP_PAIR = 3 };   // couplings of a step
 struct StripPlan {
   int G = 0;           // blocks (0: not available)
@@ -132,9 +134,9 @@ struct StripAdjoint {
   AdjStatus* out;          // device, zeroed
   const AdjStatus* after;  // status of the step walked before this one, or NULL
 };
-// shared memory of its launch; 0: the kernels per pass
+// shared memory of its launch (and its limit set); 0: the kernels per pass
 template <typename T>
-size_t strip_adjoint_smem(const StripPlan& sp, int nx, int ny, int rx, int ry);
+size_t strip_adjoint_smem(const StripPlan& sp, int ek, int nx, int ny, int rx, int ry);
 template <typename T>
 cudaError_t strip_adjoint_launch(const StripPlan& sp, size_t smem, int ek, int nx, int ny, int rx,
                                  int ry, const T* taps_x, const T* taps_y, const StripAdjoint<T>& s,

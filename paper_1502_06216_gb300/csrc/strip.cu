@@ -540,9 +540,15 @@ void* strip_fn<double>(int, int op, int ek) { return strip_fn_op<double, 1, 512>
 // 1253 / 1124: bound by its pipe, whole lines per block (4 against 3.4 on average)
 // cost what the launches save, so FP64 takes up to two
 // lines a block.  FP32: wherever the strips fit the shared memory of one block
-// per SM (about 1060 cells a side).  Long thin grids, whose short side has too
-// few lines for the blocks, keep the per-pass form unless a block's line is
-// short work anyway.
+// per SM (about 1060 cells a side).
+// Long thin grids, whose short side has too few lines for the blocks (the busiest block has
+// more than four times its share of the cells), keep the kernels per pass unless a block's
+// lines are little work (in multiply-adds: 5e5, FP64 4e4).  Up to there this form won
+// everywhere it was timed (FP32 600 x 8 9.5 / 23.9, 2048 x 32 with a narrow kernel 2.2 / 3.3; FP64
+// 152 x 4 19.7 / 62.8).  The line is a cautious one: beyond it the kernels per pass won only where
+// lines of 3500 cells and more meet a narrow kernel (FP32 4096 x 16, gamma 1e-4: 47.6 / 38.9;
+// 3500 x 24, 5e-5: 33.7 / 31.4) and lost elsewhere (FP32 1000 x 16 14.7 / 29.2, 2000 x 16 36.5 / 178,
+// gamma 1e-3; FP64 300 x 8 33.8 / 65.7).
 template <typename T>
 StripPlan strip_plan(int nx, int ny, int rx, int ry, int op, int ek, const ProxArgs<T>& P,
                      int max_blocks, int parts) {
@@ -622,8 +628,6 @@ cudaError_t strip_coop(void* fn, const StripPlan& sp, size_t smem, int threads, 
   at[0].val.cooperative = 1;
   cfg.attrs = at;
   cfg.numAttrs = 1;
-  const cudaError_t e = max_dynamic_smem(fn);
-  if (e != cudaSuccess) return e;
   return cudaLaunchKernelExC(&cfg, fn, args);
 }
 

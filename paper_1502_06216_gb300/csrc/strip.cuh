@@ -484,7 +484,8 @@ __device__ __forceinline__ double gather_sum(const unsigned long long* xr, int b
 
 }  // namespace strip
 
-// Geometry of a plan's launch, and the cooperative launch of one of these kernels.
+// Geometry of a plan's launch, and the cooperative launch of one of these kernels (whose
+// max_dynamic_smem the plan has set).
 struct StripPlan;
 strip::Geo strip_geo(const StripPlan& sp, int nx, int ny, int rx, int ry, const void* taps_x,
                      const void* taps_y, unsigned long long* words);

@@ -253,12 +253,17 @@ void* adj_fn<double>(int, int ek) { return adj_fn_ek<double, 1>(ek); }
 // Wherever the step itself runs on strips and the larger set of images still
 // fits one block per SM (FP32 up to ~760 cells a side).
 template <typename T>
-size_t strip_adjoint_smem(const StripPlan& sp, int nx, int ny, int rx, int ry) {
+size_t strip_adjoint_smem(const StripPlan& sp, int ek, int nx, int ny, int rx, int ry) {
   int dev = 0, smem_max = 0;
   if (sp.G == 0 || cudaGetDevice(&dev) != cudaSuccess) return 0;
   cudaDeviceGetAttribute(&smem_max, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
   const Smem S = smem_of<T>(nx, ny, rx, ry, sp.nc, sp.nr, 1, sp.parts, kAdjRows, kAdjCols, false);
-  return S.total + 1024 <= (size_t)smem_max ? S.total : 0;
+  if (S.total + 1024 > (size_t)smem_max) return 0;
+  if (max_dynamic_smem(adj_fn<T>(sp.rb, ek)) != cudaSuccess) {
+    cudaGetLastError();
+    return 0;
+  }
+  return S.total;
 }
 
 template <typename T>
@@ -274,7 +279,7 @@ cudaError_t strip_adjoint_launch(const StripPlan& sp, size_t smem, int ek, int n
 }
 
 #define JKO_STRIP_ADJ_INST(T)                                                                     \
-  template size_t strip_adjoint_smem<T>(const StripPlan&, int, int, int, int);                   \
+  template size_t strip_adjoint_smem<T>(const StripPlan&, int, int, int, int, int);              \
   template cudaError_t strip_adjoint_launch<T>(const StripPlan&, size_t, int, int, int, int, int, \
                                                const T*, const T*, const StripAdjoint<T>&,        \
                                                const ProxArgs<T>&, unsigned long long*,           \
