@@ -379,7 +379,11 @@ typedef struct jko_batch jko_batch;
  * branches are the flows, so small and large flows share the GPU; a flow that
  * has met its stopping rule (Sec. 3.4) turns its remaining kernels into
  * no-ops, and a flow on the persistent loop kernel is one launch per step in
- * its branch.  Grouped launch: the flows with loop = 3 (or all loop-capable
+ * its branch.  A batch whose flows all run their steps as one persistent CUDA-core launch
+ * (jko_params.loop) is one graph a step, enqueued without host decisions between the
+ * steps; such a flow's images are those of the flow alone at equal pair counts, but the
+ * residual is added by the blocks that the batch gives the flow, so a residual within
+ * FP64 rounding of tol may stop it a pair earlier or later.  Grouped launch: the flows with loop = 3 (or all loop-capable
  * flows, when the autotuner picks it) that share a tensor-core precision run
  * their steps in ONE cooperative launch of a persistent kernel that walks
  * the tiles of all of them between grid barriers, each flow with its own
@@ -403,7 +407,8 @@ jko_status jko_batch_info(const jko_batch* b, int* out);
 
 /* n_steps steps of every flow (Eq. smooth-jko) from p0_dev[f] (device image of
  * flow f, double for JKO_FP64 flows, float otherwise; validated as in
- * jko_step).  p_final_dev[f] (array and entries may be NULL) receives the last
+ * jko_step; an invalid entry is reported before any output is written, after at most two
+ * steps have run).  p_final_dev[f] (array and entries may be NULL) receives the last
  * iterate; infos (may be NULL) receives n_steps * n_flows reports, step-major
  * (infos[t * n_flows + f]).  Returns the worst status over flows and steps. */
 jko_status jko_batch_flow(jko_batch* b, const void* const* p0_dev, int n_steps,

@@ -277,7 +277,7 @@ jko_status backward_strip(jko_handle* h, size_t smem, const T* grad_final, T* gr
   cudaStream_t st = h->stream;
   const size_t N = (size_t)h->N;
   const int n = h->tape_steps;
-  if (!h->adj) ACK(cudaMalloc(&h->adj, sizeof(T) * N));
+  if (!h->adj_strip) ACK(cudaMalloc(&h->adj_strip, sizeof(T) * N));
   if (h->adj_status_cap < n) {
     if (h->adj_status) cudaFree(h->adj_status);
     h->adj_status = nullptr;
@@ -296,7 +296,7 @@ jko_status backward_strip(jko_handle* h, size_t smem, const T* grad_final, T* gr
   for (int t = n - 1; t >= 0; --t) {
     s.q = (const T*)h->tape + 2 * (size_t)t * N;
     s.a = s.q + N;
-    s.gout = t == 0 && grad_p0 ? grad_p0 : (T*)h->adj;
+    s.gout = t == 0 && grad_p0 ? grad_p0 : (T*)h->adj_strip;
     s.mass = h->tape_mass[t];
     s.out = h->adj_status + t;
     ACK(jko::strip_adjoint_launch<T>(h->strip, smem, h->ek, h->grid.nx, h->grid.ny, h->rx, h->ry,

@@ -109,6 +109,7 @@ struct jko_handle {
   void* tape = nullptr;         // per step: q_t and the final a_t (2 N elements)
   std::vector<double> tape_mass;  // sum of the unnormalised output per step
   void* adj = nullptr;          // adjoint work images (10 N elements)
+  void* adj_strip = nullptr;    // the strips' adjoint: the gradient between two steps (N elements)
   void* adj2 = nullptr;         // the attraction's adjoint work images (18 N elements)
   double* adj_red = nullptr;    // device reduction slots
 

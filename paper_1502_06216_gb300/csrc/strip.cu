@@ -16,8 +16,8 @@
 // or three images together: the same two exchanges a pair, the joint proxes cell
 // by cell on the owned strip (attraction and two species: on the columns;
 // pairwise attraction: p_1 on the rows, p_2 on the columns).  A
-// five-step attraction flow at 256^2 FP32 (band 168): 6596 us a kernel per pass
-// (five launches a pair), 3324 us here.
+// five-step attraction flow at 256^2 FP32 (band 168, 195 pairs): 6774 us a kernel per pass
+// (five launches a pair), 3163 us here.
 //
 // The exchange is strip.cuh's.  The residual of each block's rows (pairwise:
 // columns) travels the same way, twice buffered by pair parity (a block may still
@@ -532,11 +532,11 @@ void* strip_fn<double>(int, int op, int ek) { return strip_fn_op<double, 1, 512>
 }  // namespace
 
 // The rule for the persistent form, on the grid, the band and the precision.
-// Both sides measured on a GB300 (us a pair, this form / a kernel per pass, 30 pairs a
-// step): crowd FP32 128^2 9.1 / 21.2, 256^2 10.5 / 25.2, 512^2 25 / 43, 600 x 200
-// 18 / 32, 800 x 64 15 / 31, 1024^2 62 / 81; FP64 128^2 27 / 102, 256^2 145 / 176,
-// 300^2 221 / 385.  Attraction FP32 256^2 17.9 / 35.8, 512^2 67 / 111, FP64 256^2
-// 292 / 350; two species and pairwise alike.  FP64 512^2 (four lines a block) was
+// Both sides measured on a GB300 (us a pair, this form / a kernel per pass, 40 pairs a
+// step): crowd FP32 64^2 5.8 / 16.5, 128^2 6.4 / 17.9, 256^2 8.5 / 22.3, 512^2 22.9 / 39.1, 600 x 200
+// 15.6 / 29.7, 800 x 64 12.7 / 27.4, 700^2 51 / 80, 1024^2 63 / 79; FP64 64^2 10.2 / 57.4, 128^2
+// 23.7 / 96.4, 256^2 140 / 170, 300^2 215 / 376.  Attraction 256^2 FP32 15.5 / 32.4, FP64
+// 287 / 343; two species and pairwise alike.  FP64 512^2 (four lines a block) was
 // 1253 / 1124: bound by its pipe, whole lines per block (4 against 3.4 on average)
 // cost what the launches save, so FP64 takes up to two
 // lines a block.  FP32: wherever the strips fit the shared memory of one block
@@ -569,13 +569,14 @@ StripPlan strip_plan(int nx, int ny, int rx, int ry, int op, int ek, const ProxA
   if (most * G > 4.0 * nx * ny && work > (sizeof(T) == 8 ? 4e4 : 5e5)) return StripPlan{};
   sp.G = std::max(ceil_div(nx, sp.nc), ceil_div(ny, sp.nr));
   // eight outputs per work item where that leaves every scheduler two warps, else four
-  // (256^2: 8.8 us a pair with four, 11.4 with eight; 1024^2 72 and 64); FP64: one
+  // (256^2: 8.8 us a pair with four, 11.4 with eight; 1024^2 72 and 64, both before the epilogues
+  // were rolled); FP64: one
   auto items = [&](int rb) {
     return ni * std::max(sp.nc * ceil_div(ny, rb), sp.nr * ceil_div(nx, rb));
   };
   sp.rb = sizeof(T) == 8 ? 1 : items(8) >= 256 ? 8 : 4;
   // FP64: parts of an output's taps that give every scheduler two warps where the outputs
-  // do not (us a pair, one part / now: 64^2 19 / 13.3, 128^2 30 / 26)
+  // do not (us a pair over whole flows, one part / now: 64^2 19 / 13.3, 128^2 30 / 26)
   if (max_blocks > 0) sp.parts = parts;
   else while (sizeof(T) == 8 && sp.parts < 8 && items(1) * sp.parts < 256) sp.parts *= 2;
   // a warp more than the items fill: it adds and sends the residual while the others filter

@@ -11,7 +11,8 @@
 // lambda, abar, R_s and s stay in shared memory by columns, D, 1 / Y and the
 // direct term of qbar by rows.  A kernel per filter pass and per pointwise update
 // took nine launches an iteration, each a few us of launch and L2 latency, and a host wait
-// every eight: the ten-step gradient at 256^2 FP32 took 14.4 ms (11.9 of them here), now 5.3.
+// every eight: the ten-step gradient at 256^2 FP32 took 12.1 ms (106 pairs forward; most of them
+// here), with the step and its reverse on strips 3.8.
 // Four steps of the reverse pass alone, a kernel per pass / here: 512^2 FP32 3.2 / 1.5 ms,
 // 700^2 4.8 / 2.6, 256^2 FP64 8.5 / 6.2.
 #include "adjoint_cell.h"
