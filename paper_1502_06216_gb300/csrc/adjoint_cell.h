@@ -15,7 +15,7 @@
 namespace jko {
 
 // |change of lambda| at a cell in an iteration, which the solve's stop adds: in FP64 whatever the
-// working precision (256^2 FP32, the ten-step gradient: 2 % against FP32 differences; with
+// working precision (256^2 FP32, the ten-step gradient: 2-3 % against FP32 differences; with
 // the conversions and the difference split off to other pipes the same).
 template <typename T>
 JKO_HD double lambda_change(T now, T before) {
